@@ -271,24 +271,22 @@ static jac_status batch_upload_impl(jac_batch *b, int g, const jac_fields *f, bo
         if (!f->f[q]) return bfail(b, JAC_EINVAL, "field " + std::to_string(q) + " is NULL");
     const size_t n = (size_t)b->I[g] * b->J[g] * b->K[g];
     const jac_grid &gr = b->grids[g];
-    for (int q = 0; q < JAC_NFIELDS; ++q) {
-        const double *src = f->f[q];
-        if (!on_device) {
-            cudaError_t e = cudaMemcpyAsync(b->staging, src, n * sizeof(double), cudaMemcpyHostToDevice, b->stream);
-            if (e != cudaSuccess) return bcuda(b, e, "host-to-device copy");
-            src = b->staging;
-        }
-        void *dst = (q == JAC_P) ? gr.p[0] : const_cast<void *>(gr.coef[q]);
-        jac_status s = jac::pack_dev(b->I[g], b->J[g], b->K[g], b->prec, q, src, dst, b->stream);
+    void *dst[JAC_NFIELDS];
+    for (int q = 0; q < JAC_NFIELDS; ++q) dst[q] = (q == JAC_P) ? gr.p[0] : const_cast<void *>(gr.coef[q]);
+    if (on_device) {
+        jac_status s = jac::pack_fields(b->I[g], b->J[g], b->K[g], b->prec, f->f, dst, gr.p[1], b->stream);
+        if (s != JAC_OK) return bthread(b, s);
+        return JAC_OK;
+    }
+    for (int q = 0; q < JAC_NFIELDS; ++q) {      // one staging array, reused per field
+        cudaError_t e = cudaMemcpyAsync(b->staging, f->f[q], n * sizeof(double), cudaMemcpyHostToDevice, b->stream);
+        if (e != cudaSuccess) return bcuda(b, e, "host-to-device copy");
+        jac_status s = jac::pack_dev(b->I[g], b->J[g], b->K[g], b->prec, q, b->staging, dst[q], b->stream,
+                                     q == JAC_P ? gr.p[1] : nullptr);
         if (s != JAC_OK) return bthread(b, s);
     }
-    cudaError_t e = cudaMemcpyAsync(gr.p[1], gr.p[0], arr_bytes(b, g, JAC_P), cudaMemcpyDeviceToDevice, b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "device copy of p0");
-    if (!on_device) {
-        e = cudaStreamSynchronize(b->stream);
-        if (e != cudaSuccess) return bcuda(b, e, "cudaStreamSynchronize");
-    }
-    return JAC_OK;
+    cudaError_t e = cudaStreamSynchronize(b->stream);
+    return e == cudaSuccess ? JAC_OK : bcuda(b, e, "cudaStreamSynchronize");
 }
 
 jac_status jac_batch_upload(jac_batch *b, int g, const jac_fields *host) { return batch_upload_impl(b, g, host, false); }

@@ -274,14 +274,14 @@ jac_status upload_impl(jac_ctx *c, const jac_fields *f, Src from)
                                             c->stream);
             if (e != cudaSuccess) return ctx_cuda(c, e, "host-to-device copy");
         }
+        const float *staged[JAC_NFIELDS];
+        void *dst[JAC_NFIELDS];
         for (int q = 0; q < JAC_NFIELDS; ++q) {
-            jac_status s = jac::pack_dev_f32(c->I, c->J, c->K, c->prec, q, st32 + (size_t)q * n,
-                                             q == JAC_P ? c->pbuf[0] : c->arr[q], c->stream);
-            if (s != JAC_OK) return ctx_from_thread(c, s);
+            staged[q] = st32 + (size_t)q * n;
+            dst[q] = q == JAC_P ? c->pbuf[0] : c->arr[q];
         }
-        cudaError_t e = cudaMemcpyAsync(c->pbuf[1], c->pbuf[0], data_bytes(c, JAC_P), cudaMemcpyDeviceToDevice,
-                                        c->stream);
-        if (e != cudaSuccess) return ctx_cuda(c, e, "device copy of p0");
+        jac_status s = jac::pack_fields_f32(c->I, c->J, c->K, c->prec, staged, dst, c->pbuf[1], c->stream);
+        if (s != JAC_OK) return ctx_from_thread(c, s);
         c->cur = 0;
         c->count = 0;
         c->uploaded = true;
@@ -297,8 +297,10 @@ jac_status upload_impl(jac_ctx *c, const jac_fields *f, Src from)
         }
     }
     const double *src[JAC_NFIELDS];
+    void *dst[JAC_NFIELDS];
     for (int q = 0; q < JAC_NFIELDS; ++q) {
         src[q] = f->f[q];
+        dst[q] = q == JAC_P ? c->pbuf[0] : c->arr[q];
         if (from != Src::device) {
             double *stage = (from == Src::host) ? c->staging : c->stage_all + (size_t)q * n;
             cudaError_t e = cudaMemcpyAsync(stage, src[q], n * sizeof(double), cudaMemcpyHostToDevice, c->stream);
@@ -307,20 +309,17 @@ jac_status upload_impl(jac_ctx *c, const jac_fields *f, Src from)
         }
         // one reused staging array: pack each field before the next copy
         if (from == Src::host) {
-            jac_status s = jac::pack_dev(c->I, c->J, c->K, c->prec, q, src[q],
-                                         q == JAC_P ? c->pbuf[0] : c->arr[q], c->stream);
+            jac_status s = jac::pack_dev(c->I, c->J, c->K, c->prec, q, src[q], dst[q], c->stream,
+                                         q == JAC_P ? c->pbuf[1] : nullptr);
             if (s != JAC_OK) return ctx_from_thread(c, s);
         }
     }
-    for (int q = 0; q < JAC_NFIELDS && from != Src::host; ++q) {
-        jac_status s = jac::pack_dev(c->I, c->J, c->K, c->prec, q, src[q], q == JAC_P ? c->pbuf[0] : c->arr[q],
-                                     c->stream);
+    if (from != Src::host) {
+        jac_status s = jac::pack_fields(c->I, c->J, c->K, c->prec, src, dst, c->pbuf[1], c->stream);
         if (s != JAC_OK) return ctx_from_thread(c, s);
     }
-    cudaError_t e = cudaMemcpyAsync(c->pbuf[1], c->pbuf[0], data_bytes(c, JAC_P), cudaMemcpyDeviceToDevice, c->stream);
-    if (e != cudaSuccess) return ctx_cuda(c, e, "device copy of p0");
     if (from == Src::host) {
-        e = cudaStreamSynchronize(c->stream);
+        cudaError_t e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return ctx_cuda(c, e, "cudaStreamSynchronize");
     }
     c->cur = 0;

@@ -30,10 +30,17 @@ struct LaunchOpts {
 };
 jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double *d_residual, void *workspace,
                      size_t ws_bytes, void *stream, const LaunchOpts *opts = nullptr);
-jac_status pack_dev(int I, int J, int K, jac_prec prec, int which, const double *src, void *dst, cudaStream_t st);
+// Dense FP64 (or FP32) arrays into storage layout and back (jac_pack.cu).
+// pack_fields packs all thirteen arrays of a grid in one launch, p into dst[0]
+// and p2; pack_dev packs one array, into dst and, if not NULL, dst2.
+jac_status pack_dev(int I, int J, int K, jac_prec prec, int which, const double *src, void *dst, cudaStream_t st,
+                    void *dst2 = nullptr);
+jac_status pack_fields(int I, int J, int K, jac_prec prec, const double *const *src, void *const *dst, void *p2,
+                       cudaStream_t st);
+jac_status pack_fields_f32(int I, int J, int K, jac_prec prec, const float *const *src, void *const *dst, void *p2,
+                           cudaStream_t st);
 jac_status unpack_dev(int I, int J, int K, jac_prec prec, int which, const void *src, double *dst,
                       cudaStream_t st);
-jac_status pack_dev_f32(int I, int J, int K, jac_prec prec, int which, const float *src, void *dst, cudaStream_t st);
 jac_status unpack_dev_f32(int I, int J, int K, jac_prec prec, int which, const void *src, float *dst,
                           cudaStream_t st);
 jac_status workspace_check(void *workspace, cudaStream_t st);

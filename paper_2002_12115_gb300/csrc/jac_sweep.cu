@@ -1,6 +1,5 @@
 // Single-grid host side of the forward sweep (the kernel is in
-// jac_sweep_kernel.cuh), the storage-layout conversions and the stateless
-// device entry points of libjac.
+// jac_sweep_kernel.cuh) and the stateless device entry points of libjac.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -14,80 +13,6 @@
 #include "jac_sweep_kernel.cuh"
 
 namespace jac {
-
-// ------------------------------------------------------- pack / unpack
-template <typename C>
-__device__ __forceinline__ C cvt_from_f64(double x);
-template <>
-__device__ __forceinline__ double cvt_from_f64<double>(double x) { return x; }
-template <>
-__device__ __forceinline__ float cvt_from_f64<float>(double x) { return __double2float_rn(x); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 cvt_from_f64<__nv_bfloat16>(double x)
-{
-    return __float2bfloat16_rn(__double2float_rn(x));  // FP64 -> FP32 -> BF16, each RNE
-}
-
-__device__ __forceinline__ double to_f64(double x) { return x; }
-__device__ __forceinline__ double to_f64(float x) { return (double)x; }
-__device__ __forceinline__ double to_f64(__nv_bfloat16 x) { return (double)__bfloat162float(x); }
-
-template <typename C>
-__global__ void k_pack(const double *__restrict__ src, C *__restrict__ dst, int I, int J, int K, int pitch)
-{
-    const size_t total = (size_t)pitch * J * K;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total; x += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(x % (size_t)pitch);
-        const size_t row = x / (size_t)pitch;
-        dst[x] = (i < I) ? cvt_from_f64<C>(src[row * I + i]) : cvt_from_f64<C>(0.0);
-    }
-}
-
-// The same from dense FP32 values (inputs that are FP32 numbers): FP64 and
-// FP32 storage keep the value, BF16 storage rounds it RNE -- the storage
-// values k_pack gives for the same numbers in FP64.
-template <typename C>
-__device__ __forceinline__ C cvt_from_f32(float x);
-template <>
-__device__ __forceinline__ double cvt_from_f32<double>(float x) { return (double)x; }
-template <>
-__device__ __forceinline__ float cvt_from_f32<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ __nv_bfloat16 cvt_from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
-template <typename C>
-__global__ void k_pack_f32(const float *__restrict__ src, C *__restrict__ dst, int I, int J, int K, int pitch)
-{
-    const size_t total = (size_t)pitch * J * K;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total; x += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(x % (size_t)pitch);
-        const size_t row = x / (size_t)pitch;
-        dst[x] = (i < I) ? cvt_from_f32<C>(src[row * I + i]) : cvt_from_f32<C>(0.0f);
-    }
-}
-
-// Storage layout to dense FP32 (RNE from FP64 storage; exact otherwise).
-template <typename C>
-__global__ void k_unpack_f32(const C *__restrict__ src, float *__restrict__ dst, int I, int J, int K, int pitch)
-{
-    const size_t total = (size_t)I * J * K;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total; x += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(x % (size_t)I);
-        const size_t row = x / (size_t)I;
-        dst[x] = (float)to_f64(src[row * pitch + i]);
-    }
-}
-
-template <typename C>
-__global__ void k_unpack(const C *__restrict__ src, double *__restrict__ dst, int I, int J, int K, int pitch)
-{
-    const size_t total = (size_t)I * J * K;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total; x += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(x % (size_t)I);
-        const size_t row = x / (size_t)I;
-        dst[x] = to_f64(src[row * pitch + i]);
-    }
-}
 
 // ------------------------------------------------------------ host side
 namespace {
@@ -570,80 +495,6 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     return launch_sweep<false>(g->prec, tj, d0, a, nblocks, static_cast<cudaStream_t>(stream));
 }
 
-jac_status pack_dev(int I, int J, int K, jac_prec prec, int which, const double *src, void *dst, cudaStream_t st)
-{
-    if (I < 3 || J < 3 || K < 3 || which < 0 || which >= JAC_NFIELDS || !src || !dst)
-        return fail(JAC_EINVAL, "bad pack arguments");
-    const int pitch = jac_pitch(I);
-    const size_t total = (size_t)pitch * J * K;
-    const int threads = 256;
-    const unsigned blocks = (unsigned)std::min<size_t>((total + threads - 1) / threads, (size_t)num_sms() * 32);
-    switch (elem_bytes(prec, which)) {
-    case 8: k_pack<double><<<blocks, threads, 0, st>>>(src, static_cast<double *>(dst), I, J, K, pitch); break;
-    case 4: k_pack<float><<<blocks, threads, 0, st>>>(src, static_cast<float *>(dst), I, J, K, pitch); break;
-    default:
-        k_pack<__nv_bfloat16><<<blocks, threads, 0, st>>>(src, static_cast<__nv_bfloat16 *>(dst), I, J, K, pitch);
-    }
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? JAC_OK : cuda_fail(e, "pack launch");
-}
-
-jac_status pack_dev_f32(int I, int J, int K, jac_prec prec, int which, const float *src, void *dst, cudaStream_t st)
-{
-    if (I < 3 || J < 3 || K < 3 || which < 0 || which >= JAC_NFIELDS || !src || !dst)
-        return fail(JAC_EINVAL, "bad pack arguments");
-    const int pitch = jac_pitch(I);
-    const size_t total = (size_t)pitch * J * K;
-    const int threads = 256;
-    const unsigned blocks = (unsigned)std::min<size_t>((total + threads - 1) / threads, (size_t)num_sms() * 32);
-    switch (elem_bytes(prec, which)) {
-    case 8: k_pack_f32<double><<<blocks, threads, 0, st>>>(src, static_cast<double *>(dst), I, J, K, pitch); break;
-    case 4: k_pack_f32<float><<<blocks, threads, 0, st>>>(src, static_cast<float *>(dst), I, J, K, pitch); break;
-    default:
-        k_pack_f32<__nv_bfloat16><<<blocks, threads, 0, st>>>(src, static_cast<__nv_bfloat16 *>(dst), I, J, K, pitch);
-    }
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? JAC_OK : cuda_fail(e, "pack launch");
-}
-
-jac_status unpack_dev_f32(int I, int J, int K, jac_prec prec, int which, const void *src, float *dst, cudaStream_t st)
-{
-    if (I < 3 || J < 3 || K < 3 || which < 0 || which >= JAC_NFIELDS || !src || !dst)
-        return fail(JAC_EINVAL, "bad unpack arguments");
-    const int pitch = jac_pitch(I);
-    const size_t total = (size_t)I * J * K;
-    const int threads = 256;
-    const unsigned blocks = (unsigned)std::min<size_t>((total + threads - 1) / threads, (size_t)num_sms() * 32);
-    switch (elem_bytes(prec, which)) {
-    case 8: k_unpack_f32<double><<<blocks, threads, 0, st>>>(static_cast<const double *>(src), dst, I, J, K, pitch); break;
-    case 4: k_unpack_f32<float><<<blocks, threads, 0, st>>>(static_cast<const float *>(src), dst, I, J, K, pitch); break;
-    default:
-        k_unpack_f32<__nv_bfloat16>
-            <<<blocks, threads, 0, st>>>(static_cast<const __nv_bfloat16 *>(src), dst, I, J, K, pitch);
-    }
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? JAC_OK : cuda_fail(e, "unpack launch");
-}
-
-jac_status unpack_dev(int I, int J, int K, jac_prec prec, int which, const void *src, double *dst, cudaStream_t st)
-{
-    if (I < 3 || J < 3 || K < 3 || which < 0 || which >= JAC_NFIELDS || !src || !dst)
-        return fail(JAC_EINVAL, "bad unpack arguments");
-    const int pitch = jac_pitch(I);
-    const size_t total = (size_t)I * J * K;
-    const int threads = 256;
-    const unsigned blocks = (unsigned)std::min<size_t>((total + threads - 1) / threads, (size_t)num_sms() * 32);
-    switch (elem_bytes(prec, which)) {
-    case 8: k_unpack<double><<<blocks, threads, 0, st>>>(static_cast<const double *>(src), dst, I, J, K, pitch); break;
-    case 4: k_unpack<float><<<blocks, threads, 0, st>>>(static_cast<const float *>(src), dst, I, J, K, pitch); break;
-    default:
-        k_unpack<__nv_bfloat16>
-            <<<blocks, threads, 0, st>>>(static_cast<const __nv_bfloat16 *>(src), dst, I, J, K, pitch);
-    }
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? JAC_OK : cuda_fail(e, "unpack launch");
-}
-
 jac_status workspace_check(void *workspace, cudaStream_t st)
 {
     if (!workspace) return fail(JAC_EINVAL, "workspace is NULL");
@@ -704,17 +555,6 @@ jac_status jac_resolve_plan(const jac_grid *g, const jac_plan *plan, int sm_coun
 jac_status jac_workspace_check(void *workspace, void *stream)
 {
     return jac::workspace_check(workspace, static_cast<cudaStream_t>(stream));
-}
-
-jac_status jac_pack_dev(int I, int J, int K, jac_prec prec, int which, const double *d_src, void *d_dst, void *stream)
-{
-    return jac::pack_dev(I, J, K, prec, which, d_src, d_dst, static_cast<cudaStream_t>(stream));
-}
-
-jac_status jac_unpack_dev(int I, int J, int K, jac_prec prec, int which, const void *d_src, double *d_dst,
-                          void *stream)
-{
-    return jac::unpack_dev(I, J, K, prec, which, d_src, d_dst, static_cast<cudaStream_t>(stream));
 }
 
 }  // extern "C"
