@@ -48,14 +48,13 @@ struct jac_ctx {
     // checkpoint tape of the sweeps since jac_tape_begin
     struct Tape {
         int C = 0, max_sweeps = 0, taped = 0;
-        void *mem = nullptr;      // checkpoints, segment states 1..C-1, two lambda buffers, one double
+        void *mem = nullptr;      // checkpoints, segment states 1..C-1, two lambda buffers
         size_t state_bytes = 0;
         int n_ckpt = 0;
         char *ckpt(int s) const { return static_cast<char *>(mem) + (size_t)s * state_bytes; }
         // state m (1 <= m < C) of a segment; state 0 is the segment's checkpoint
         char *seg(int m) const { return ckpt(n_ckpt) + (size_t)(m - 1) * state_bytes; }
         char *lam(int b) const { return seg(C) + (size_t)b * state_bytes; }
-        double *scratch() const { return reinterpret_cast<double *>(lam(2)); }
     } tape;
 };
 
@@ -225,6 +224,7 @@ jac_status sweep_impl(jac_ctx *c, int n_iter)
         }
         jac_grid g = make_grid(c);
         jac::LaunchOpts opts;
+        opts.no_residual = chunk < n_iter;   // only the call's last sweep's residual is kept
         if (c->stall_ns) {            // the grid barrier of this launch is never reached
             opts.wait_ns = c->stall_ns;
             opts.gbar_extra = 1;
@@ -672,6 +672,8 @@ jac_status jac_sweep_adjoint(jac_ctx *c, const double *lam_T, double *g_wrk1, do
     }
     jac_grid g = make_grid(c);
     const bool pairs = c->prec == JAC_F32 && jac::resolve_plan(&g, &c->plan).fuse == 2;
+    jac::LaunchOpts recompute;
+    recompute.no_residual = true;
     int lc = 0;
     const int nseg = (tp.taped + tp.C - 1) / tp.C;
     for (int sgi = nseg - 1; sgi >= 0; --sgi) {
@@ -690,7 +692,7 @@ jac_status jac_sweep_adjoint(jac_ctx *c, const double *lam_T, double *g_wrk1, do
                 m += 2;
             } else {
                 g.p[1] = tp.seg(m);
-                s = jac::sweep_dev(&g, &c->plan, 1, tp.scratch(), c->ws, c->ws_bytes, c->stream);
+                s = jac::sweep_dev(&g, &c->plan, 1, nullptr, c->ws, c->ws_bytes, c->stream, &recompute);
                 m += 1;
             }
             if (s != JAC_OK) return ctx_from_thread(c, s);

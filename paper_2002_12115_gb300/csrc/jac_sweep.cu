@@ -438,6 +438,7 @@ bool use_two_sweep_passes(const jac_grid *g, const jac_plan &p, int n_iter)
 jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double *d_residual, void *workspace,
                      size_t ws_bytes, void *stream, const LaunchOpts *opts)
 {
+    const bool no_res = opts && opts->no_residual;
     const bool injected = opts && (opts->wait_ns != 0 || opts->gbar_extra != 0);
     jac_status s = validate_grid(g);
     if (s != JAC_OK) return s;
@@ -456,7 +457,7 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
         const int n_pass = (n_iter / 2) & ~1;
         const int rest = n_iter - 2 * n_pass;
         double *res2 = nullptr;
-        if (rest == 0) res2 = d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual;
+        if (rest == 0 && !no_res) res2 = d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual;
         if ((s = sweep2_run(g, 0, n_pass, res2, workspace, ws_bytes, static_cast<cudaStream_t>(stream))) != JAC_OK)
             return s;
         if (rest == 0) return JAC_OK;
@@ -473,7 +474,7 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     a.par = 0;
     a.omega = g->omega;
     a.partials = reinterpret_cast<double *>(static_cast<char *>(workspace) + kWsHeaderBytes);
-    a.res = d_residual ? d_residual : &hdr->residual;
+    a.res = no_res ? nullptr : (d_residual ? d_residual : &hdr->residual);
     a.hdr = hdr;
     if (injected) {
         a.wait_ns = opts->wait_ns;

@@ -567,10 +567,9 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
                 if (lane == 0) s_part[w] = v;
                 if (!cons_sync()) { ok = false; break; }
-                if (threadIdx.x == 0) {
-                    double sum = 0.0, comp = 0.0;
-                    for (int q = 0; q < R1; ++q) neumaier_add(sum, comp, s_part[q]);
-                    a.partials[blockIdx.x] = sum + comp;
+                if (w == 0) {
+                    const double sum = warp_sum(lane < R1 ? s_part[lane] : 0.0, 0.0);
+                    if (lane == 0) a.partials[blockIdx.x] = sum;
                 }
                 acc = 0.0;
                 if (!cons_sync()) { ok = false; break; }
@@ -592,7 +591,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         cp_async_wait_all();   // no copy into this CTA's shared memory outlives it
     }
 
-    // CTA epilogue: the last CTA to finish sums the partials in CTA order
+    // CTA epilogue: the last CTA to finish sums the partials in a fixed order
     // and resets the workspace counters for the next launch.
     // If any CTA gave up a wait, the residual is written as NaN.
     __syncthreads();
@@ -605,19 +604,17 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
     __syncthreads();
     if (s_last) {
         __threadfence();
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
             if (a.res != nullptr) {
-                if (s_abort || workspace_failed(a.hdr)) {
-                    *a.res = __longlong_as_double(0x7ff8000000000000ll);
-                } else {
-                    double sum = 0.0, comp = 0.0;
-                    for (int b = 0; b < G; ++b) neumaier_add(sum, comp, __ldcg(&a.partials[b]));
-                    *a.res = sum + comp;
-                }
+                const double sum = sum_partials(a.partials, G, lane);
+                if (lane == 0)
+                    *a.res = (s_abort || workspace_failed(a.hdr)) ? __longlong_as_double(0x7ff8000000000000ll) : sum;
             }
-            a.hdr->gbar = 0u;
-            a.hdr->counter = 0u;
-            __threadfence();
+            if (lane == 0) {
+                a.hdr->gbar = 0u;
+                a.hdr->counter = 0u;
+                __threadfence();
+            }
         }
     }
 }

@@ -29,8 +29,8 @@
 //     cancelling s0*a3 against p.  FP64 uses the written form with FMAs;
 //   * the last sweep sums each lane's squares of one step in FP32 and
 //     accumulates them in FP64; at every change of grid in a CTA's item list
-//     the consumer warps reduce (shuffle, then Neumaier) into one partial per
-//     (grid, CTA); the last CTA to finish sums each grid's partials in CTA
+//     the consumer warps reduce (shuffles, compensated) into one partial per
+//     (grid, CTA); the last CTA to finish sums each grid's partials in a fixed
 //     order, so every residual is bitwise reproducible;
 //   * when both state buffers fit in half the L2 (129 MB on GB300), the state
 //     copies and stores carry an evict_last policy and the coefficient copies
@@ -153,6 +153,37 @@ __device__ __forceinline__ void neumaier_add(double &s, double &c, double x)
     if (fabs(s) >= fabs(x)) c += (s - t) + x;
     else c += (x - t) + s;
     s = t;
+}
+
+// Compensated sum over the lanes of a warp of (s, c) pairs, in a fixed order;
+// complete in lane 0.  GB300 issues a warp's FP64 instruction over 64 clocks
+// whether one lane or 32 take part, so sums run across lanes wherever they
+// can: one thread adding the 152 partials of a launch one after the other,
+// each behind its own load, took 25 us or more of every sweep call.
+__device__ __forceinline__ double warp_sum(double s, double c)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+        neumaier_add(s, c, s2);
+        c += c2;
+    }
+    return s + c;
+}
+
+// Sum of the n partials of a launch by one warp; complete in lane 0.
+__device__ __forceinline__ double sum_partials(const double *partials, int n, int lane)
+{
+    constexpr int U = 5;               // loads in flight per lane: all of a 152-CTA launch
+    double s = 0.0, c = 0.0;
+    for (int b0 = lane; b0 < n; b0 += 32 * U) {
+        double v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = b0 + 32 * u < n ? __ldcg(partials + b0 + 32 * u) : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) neumaier_add(s, c, v[u]);
+    }
+    return warp_sum(s, c);
 }
 
 // Compile-time shape of a kernel instantiation: TJ consumer warps, VI points
@@ -444,10 +475,9 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
             for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
             if (lane == 0) s_part[wy] = v;
             if (!cons_sync()) return false;
-            if (threadIdx.x == 0) {
-                double s = 0.0, c = 0.0;
-                for (int w = 0; w < TJ; ++w) neumaier_add(s, c, s_part[w]);
-                a.partials[(size_t)g * G + blockIdx.x] = s + c;
+            if (wy == 0) {
+                const double sum = warp_sum(lane < TJ ? s_part[lane] : 0.0, 0.0);
+                if (lane == 0) a.partials[(size_t)g * G + blockIdx.x] = sum;
             }
             acc = 0.0;
             return cons_sync();
@@ -606,7 +636,7 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
         }
     }
 
-    // CTA epilogue: the last CTA to finish sums each grid's partials in CTA
+    // CTA epilogue: the last CTA to finish sums each grid's partials in a fixed
     // order and resets the workspace counters for the next launch.  If any
     // CTA gave up a wait (the error word is set), the partials may be stale
     // and every residual is written as NaN instead, so that a caller who
@@ -624,11 +654,11 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
         if (threadIdx.x == 0) s_failed = s_abort || workspace_failed(a.hdr);
         __syncthreads();
         if (a.res != nullptr) {
-            for (int g = threadIdx.x; g < a.ngrids; g += blockDim.x) {
-                double s = 0.0, c = 0.0;
-                if (!s_failed)
-                    for (int b = 0; b < G; ++b) neumaier_add(s, c, __ldcg(&a.partials[(size_t)g * G + b]));
-                a.res[g] = s_failed ? __longlong_as_double(0x7ff8000000000000ll) : s + c;
+            // a warp per grid
+            for (int g = warp; g < a.ngrids; g += TJ + 2) {
+                const double sum = s_failed ? __longlong_as_double(0x7ff8000000000000ll)
+                                            : sum_partials(a.partials + (size_t)g * G, G, lane);
+                if (lane == 0) a.res[g] = sum;
             }
         }
         __syncthreads();
