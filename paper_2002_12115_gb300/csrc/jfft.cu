@@ -202,6 +202,15 @@ __device__ __forceinline__ double kbar2(int k, int n)
     return (double)s * (double)s;
 }
 
+// Programmatic dependent launch: a pass lets the next launch of the stream
+// start its prologue as soon as every CTA of this one runs, and waits for
+// everything before it in the stream ahead of its own first data access.
+// Small transforms are bound by their launches: 64x32x128 FP32 forward and
+// inverse 28.7 -> 22.4 us (with the twiddle copy and the data loads in flight
+// together); 512^3 gains 2.8% from overlapped tails.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prior_grids() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // The spectral factor along each axis, exp(c kbar^2) for every index of
 // n1, then n2, then n3 (FP64 exp, stored as T): one small launch per step,
 // so that a pass multiplies by a table entry per element and one per line.
@@ -209,15 +218,37 @@ template <typename T>
 __global__ void k_fft_factors(double c, int n1, int n2, int n3, T *f1, T *f2, T *f3)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    launch_dependents();
+    wait_prior_grids();            // an earlier step may still read the tables
     if (i < n1) f1[i] = (T)exp(c * kbar2(i, n1));
     else if (i < n1 + n2) f2[i - n1] = (T)exp(c * kbar2(i - n1, n2));
     else if (i < n1 + n2 + n3) f3[i - n1 - n2] = (T)exp(c * kbar2(i - n1 - n2, n3));
 }
 
-// One Stockham stage for the BPT = RMAX / R butterflies of this thread.
+// 8 or 16 bytes global -> shared without a register round trip.
+template <typename E>
+__device__ __forceinline__ void copy_async(E *smem_dst, const E *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(smem_dst)),
+                 "l"(src), "n"((int)sizeof(E))
+                 : "memory");
+}
+
+// The first stage's inputs: radix R butterflies at stride N / R.
+template <typename T, int N, int R, int RMAX>
+__device__ __forceinline__ void load_line(C2<T> (&v)[RMAX], const C2<T> *gin, long long lb, long long es, int t)
+{
+    constexpr int TT = N / RMAX;
+#pragma unroll
+    for (int q = 0; q < RMAX / R; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[q * R + r] = gin[lb + (long long)(t + q * TT + r * (N / R)) * es];
+}
+
+// One Stockham stage for the BPT = RMAX / R butterflies of this thread (the
+// first stage finds its inputs in v).
 template <typename T, int N, int R, int RMAX, int NS, bool INV, bool FIRST, bool LAST>
-__device__ __forceinline__ void stage(C2<T> (&v)[RMAX], C2<T> *tile, const C2<T> *tw, const C2<T> *gin, C2<T> *gout,
-                                      long long lb, long long es, int w, int t, const T *fe, T fl, T scale,
+__device__ __forceinline__ void stage(C2<T> (&v)[RMAX], C2<T> *tile, const C2<T> *tw, C2<T> *gout, long long lb, long long es, int w, int t, const T *fe, T fl, T scale,
                                       bool factor, T &esum, bool want_energy)
 {
     constexpr int TT = N / RMAX;       // threads per line
@@ -231,13 +262,11 @@ __device__ __forceinline__ void stage(C2<T> (&v)[RMAX], C2<T> *tile, const C2<T>
         for (int r = 0; r < R; ++r) {
             const int e = j + r * (N / R);
             if constexpr (FIRST) {
-                C2<T> x = gin[lb + (long long)e * es];
                 if (factor) {
                     const T f = fe[e] * fl;
-                    x.x *= f;
-                    x.y *= f;
+                    v[q * R + r].x *= f;
+                    v[q * R + r].y *= f;
                 }
-                v[q * R + r] = x;
             } else {
                 v[q * R + r] = row[pad_idx<T>(e)];
             }
@@ -298,57 +327,63 @@ __global__ void __launch_bounds__(YZ ? 512 : 256, min_ctas_per_sm<T, YZ>()) k_ff
     else { w = threadIdx.x % W; t = threadIdx.x / W; }
     const long long n1 = a.n1, n2 = a.n2;
     long long lb, es;              // first element of the line, element stride
-    int ia, ib, na, nb;            // the line's indices on the other two axes, and their extents
+    int ia, ib;                    // the line's indices on the other two axes
     if (a.axis == 0) {
         const long long row = (long long)blockIdx.x * W + w;     // row = z * n2 + y
         lb = row * n1;
         es = 1;
-        ia = (int)(row % n2); na = a.n2;
-        ib = (int)(row / n2); nb = a.n3;
+        ia = (int)(row % n2);
+        ib = (int)(row / n2);
     } else {
         const int xt = blockIdx.x % (a.n1 / W);
         const int o = blockIdx.x / (a.n1 / W);                   // z (y pass) or y (z pass)
         const int x = xt * W + w;
-        ia = x; na = a.n1;
-        ib = o; nb = a.axis == 1 ? a.n3 : a.n2;
+        ia = x;
+        ib = o;
         lb = a.axis == 1 ? (long long)o * n1 * n2 + x : (long long)o * n1 + x;
         es = a.axis == 1 ? n1 : n1 * n2;
     }
 
-    // twiddles (and the spectral factor along this axis) into shared memory
+    launch_dependents();
+    // the twiddles into shared memory (constant since the plan was made, so
+    // their copies need not wait for earlier launches) ...
     const C2<T> *gtw = static_cast<const C2<T> *>(a.tw);
-    const T *gfa = static_cast<const T *>(a.fa);
-    for (int m = threadIdx.x; m < N; m += blockDim.x) {
-        if constexpr (RX::R2 > 1) tw[m] = gtw[m];
-        if (a.factor) fe[m] = gfa[m];
-    }
-    if (a.factor && t == 0) fl[w] = static_cast<const T *>(a.fb)[ia] * static_cast<const T *>(a.fc)[ib];
-    (void)na;
-    (void)nb;
-    __syncthreads();
-
+    if constexpr (RX::R2 > 1)
+        for (int m = threadIdx.x; m < N; m += blockDim.x) copy_async(&tw[m], &gtw[m]);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    wait_prior_grids();
+    // ... and, with them in flight, this thread's part of its line
     const C2<T> *gin = static_cast<const C2<T> *>(a.in);
     C2<T> *gout = static_cast<C2<T> *>(a.out);
+    C2<T> v[RMAX];
+    load_line<T, N, RX::R1, RMAX>(v, gin, lb, es, t);
+    if (a.factor) {                // the spectral factor along this axis and of this line
+        const T *gfa = static_cast<const T *>(a.fa);
+        for (int m = threadIdx.x; m < N; m += blockDim.x) fe[m] = gfa[m];
+        if (t == 0) fl[w] = static_cast<const T *>(a.fb)[ia] * static_cast<const T *>(a.fc)[ib];
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+
     const bool want_energy = a.energy != nullptr;
     const T scale = (T)a.scale;
     const T flw = a.factor ? fl[w] : (T)1;
     T esum = (T)0;
-    C2<T> v[RMAX];
     constexpr int R1 = RX::R1, R2 = RX::R2, R3 = RX::R3;
     if constexpr (R2 == 1) {
-        stage<T, N, R1, RMAX, 1, INV, true, true>(v, tile, tw, gin, gout, lb, es, w, t, fe, flw, scale,
+        stage<T, N, R1, RMAX, 1, INV, true, true>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
                                                   a.factor, esum, want_energy);
     } else if constexpr (R3 == 1) {
-        stage<T, N, R1, RMAX, 1, INV, true, false>(v, tile, tw, gin, gout, lb, es, w, t, fe, flw, scale,
+        stage<T, N, R1, RMAX, 1, INV, true, false>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
                                                    a.factor, esum, want_energy);
-        stage<T, N, R2, RMAX, R1, INV, false, true>(v, tile, tw, gin, gout, lb, es, w, t, fe, flw, scale,
+        stage<T, N, R2, RMAX, R1, INV, false, true>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
                                                     a.factor, esum, want_energy);
     } else {
-        stage<T, N, R1, RMAX, 1, INV, true, false>(v, tile, tw, gin, gout, lb, es, w, t, fe, flw, scale,
+        stage<T, N, R1, RMAX, 1, INV, true, false>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
                                                    a.factor, esum, want_energy);
-        stage<T, N, R2, RMAX, R1, INV, false, false>(v, tile, tw, gin, gout, lb, es, w, t, fe, flw, scale,
+        stage<T, N, R2, RMAX, R1, INV, false, false>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
                                                      a.factor, esum, want_energy);
-        stage<T, N, R3, RMAX, R1 * R2, INV, false, true>(v, tile, tw, gin, gout, lb, es, w, t, fe, flw, scale,
+        stage<T, N, R3, RMAX, R1 * R2, INV, false, true>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
                                                          a.factor, esum, want_energy);
     }
     if (!want_energy) return;
@@ -390,6 +425,8 @@ __global__ void __launch_bounds__(512) k_fft_energy(const double *__restrict__ p
 {
     __shared__ double red[512];
     const int t = threadIdx.x;
+    launch_dependents();
+    wait_prior_grids();
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     for (int b = t; b < n; b += 4 * 512) {
         s0 += partials[b];
@@ -494,6 +531,29 @@ jac_status check_shape(int n1, int n2, int n3, jfft_prec prec)
 
 }  // namespace
 
+// A launch that may start before the stream's previous one has ended (its
+// kernel waits for it, see wait_prior_grids).
+template <typename... P, typename... A>
+jac_status launch_chained(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                          const char *what, A... args)
+{
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    if (e == cudaSuccess) return JAC_OK;
+    jac::set_thread_error(std::string(what) + ": " + cudaGetErrorString(e));
+    return JAC_ECUDA;
+}
+
 // Launch of one pass: the kernel instantiation for (T, N, INV).
 template <typename T, bool INV, bool YZ>
 jac_status launch_pass_t(int N, const PassArgs &a, unsigned grid, unsigned block, cudaStream_t st)
@@ -535,13 +595,7 @@ jac_status launch_pass_t(int N, const PassArgs &a, unsigned grid, unsigned block
             else it->second = smem;
         }
     }
-    kern<<<grid, block, smem, st>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        jac::set_thread_error(std::string("FFT pass launch: ") + cudaGetErrorString(e));
-        return JAC_ECUDA;
-    }
-    return JAC_OK;
+    return launch_chained(kern, grid, block, smem, st, "FFT pass launch", a);
 }
 
 }  // namespace jfft
@@ -584,17 +638,17 @@ jac_status run3(jfft_plan *p, const void *in, void *out, bool inv, double scale,
         if (a < b + bytes && b < a + bytes) return plan_fail(p, JAC_EINVAL, "in and out overlap without being equal");
     }
     if (factor) {
-        const int nt = p->n[0] + p->n[1] + p->n[2];
-        if (p->prec == JFFT_C32)
-            jfft::k_fft_factors<float><<<(nt + 255) / 256, 256, 0, p->stream>>>(
-                c, p->n[0], p->n[1], p->n[2], reinterpret_cast<float *>(p->ws + p->L.fac[0]),
-                reinterpret_cast<float *>(p->ws + p->L.fac[1]), reinterpret_cast<float *>(p->ws + p->L.fac[2]));
-        else
-            jfft::k_fft_factors<double><<<(nt + 255) / 256, 256, 0, p->stream>>>(
-                c, p->n[0], p->n[1], p->n[2], reinterpret_cast<double *>(p->ws + p->L.fac[0]),
-                reinterpret_cast<double *>(p->ws + p->L.fac[1]), reinterpret_cast<double *>(p->ws + p->L.fac[2]));
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return plan_fail(p, JAC_ECUDA, std::string("factor launch: ") + cudaGetErrorString(e));
+        const unsigned blocks = (unsigned)(p->n[0] + p->n[1] + p->n[2] + 255) / 256;
+        char *f[3] = {p->ws + p->L.fac[0], p->ws + p->L.fac[1], p->ws + p->L.fac[2]};
+        const jac_status s =
+            p->prec == JFFT_C32
+                ? jfft::launch_chained(jfft::k_fft_factors<float>, blocks, 256, 0, p->stream, "factor launch", c, p->n[0],
+                                       p->n[1], p->n[2], reinterpret_cast<float *>(f[0]),
+                                       reinterpret_cast<float *>(f[1]), reinterpret_cast<float *>(f[2]))
+                : jfft::launch_chained(jfft::k_fft_factors<double>, blocks, 256, 0, p->stream, "factor launch", c,
+                                       p->n[0], p->n[1], p->n[2], reinterpret_cast<double *>(f[0]),
+                                       reinterpret_cast<double *>(f[1]), reinterpret_cast<double *>(f[2]));
+        if (s != JAC_OK) return plan_from_thread(p, s);
     }
     for (int axis = 0; axis < 3; ++axis) {
         const int N = p->n[axis];
@@ -631,10 +685,9 @@ jac_status run3(jfft_plan *p, const void *in, void *out, bool inv, double scale,
                           : jfft::launch_pass_t<double, false, false>(N, a, grid, block, p->stream));
         if (s != JAC_OK) return plan_from_thread(p, s);
         if (axis == 2 && energy) {
-            jfft::k_fft_energy<<<1, 512, 0, p->stream>>>(reinterpret_cast<double *>(p->ws + p->L.partials), (int)grid,
-                                                         energy);
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return plan_fail(p, JAC_ECUDA, std::string("energy launch: ") + cudaGetErrorString(e));
+            s = jfft::launch_chained(jfft::k_fft_energy, 1, 512, 0, p->stream, "energy launch",
+                                     reinterpret_cast<const double *>(p->ws + p->L.partials), (int)grid, energy);
+            if (s != JAC_OK) return plan_from_thread(p, s);
         }
     }
     return JAC_OK;

@@ -122,3 +122,30 @@ def test_bad_arguments(pkg):
         a, b = big[:512].view(4, 8, 16), big[8:520].view(4, 8, 16)      # overlapping, not equal
         with pytest.raises(pkg.JacError):
             f.forward(a, out=b)
+
+
+@pytest.mark.parametrize("prec", ["c64", "c32"])
+@pytest.mark.parametrize("shape", [(2, 4, 8), (64, 32, 128), (512, 4, 2), (16, 256, 32)])
+def test_chained_launches_equal_separate_ones(pkg, shape, prec):
+    """Passes start before the stream's previous launch has ended and wait for
+    it themselves: a chain of transforms and steps in place gives bitwise what
+    it gives with the GPU idle before every call."""
+    import torch
+    n1, n2, n3 = shape
+    x = _dev(ji.fft_field(n1, n2, n3, seed=640 + n2), prec)
+
+    def chain(wait):
+        a, e = x.clone(), torch.zeros(1, dtype=torch.float64, device="cuda")
+        with pkg.FFT3(n1, n2, n3, prec) as f:
+            out = []
+            for k in range(6):
+                for step in (lambda: f.forward(a, out=a), lambda: f.evolve(a, 1e-4, 0.1 * k, out=a, energy=e),
+                             lambda: a.mul_(1.0 + k), lambda: f.forward(a, out=a), lambda: f.inverse(a, out=a)):
+                    step()
+                    if wait:
+                        torch.cuda.synchronize()
+                out.append((a.clone(), e.clone()))
+        return out
+
+    for (a, e), (b, g) in zip(chain(False), chain(True)):
+        assert torch.equal(torch.view_as_real(a), torch.view_as_real(b)) and torch.equal(e, g)
