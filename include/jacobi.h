@@ -133,7 +133,12 @@ typedef struct jac_grid {
  * tile that range touches, so every CTA gets the same number of planes
  * (FP64 storage only; with FP32 storage they measured slower than the
  * rule above, and the call returns JAC_EINVAL).
- * Unsupported shapes: JAC_EINVAL at launch. */
+ * Unsupported shapes: JAC_EINVAL at launch.
+ * A plan of all zeros (or NULL) leaves the kernel to the library as well:
+ * calls of three sweeps or more on grids whose coefficients fit in the shared
+ * memory of all SMs together run resident (one launch that keeps them there
+ * and exchanges only the rows between neighbouring CTAs; the state is bitwise
+ * the same).  Any non-zero field selects the kernel described above. */
 enum { JAC_KDEPTH_BALANCED = -1 };
 typedef struct jac_plan {
     int tile_j;   /* rows per work item */
@@ -165,8 +170,10 @@ typedef struct jac_plan {
  * dimensions, precision or plan entries, or a shape the kernels lack. */
 jac_status jac_resolve_plan(const jac_grid *g, const jac_plan *plan, int sm_count, jac_plan *out);
 
-/* Bytes of device workspace jac_sweep_dev needs for this grid and plan
- * (host only).  No paper counterpart (the caller-owned scratch of the
+/* Bytes of device workspace for jac_sweep_dev on this grid and plan (host
+ * only).  It includes the flags of the resident kernel where the grid can
+ * take it; jac_sweep_dev also accepts a workspace without room for them (256
+ * bytes and one double per CTA of the plan) and then never runs resident.  No paper counterpart (the caller-owned scratch of the
  * stateless form). */
 jac_status jac_sweep_workspace_size(const jac_grid *g, const jac_plan *plan, size_t *bytes);
 

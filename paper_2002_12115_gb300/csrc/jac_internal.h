@@ -19,7 +19,10 @@ void set_thread_error(const std::string &m);
 jac_status validate_grid(const jac_grid *g);
 jac_plan resolve_plan(const jac_grid *g, const jac_plan *plan);
 jac_plan resolve_plan_sms(const jac_grid *g, const jac_plan *plan, int sms);
+// Bytes of workspace a sweep with this plan needs, and the bytes with which
+// every path open to the library's own plan may run (never less).
 size_t sweep_workspace_bytes(const jac_grid *g, const jac_plan &p);
+size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p);
 // Launch options of the single-grid sweep.  wait_ns and gbar_extra are set
 // only by a test of the failure path: a shorter limit for the waits on other
 // warps and CTAs, and an offset that makes the grid barrier between sweeps
@@ -69,6 +72,20 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
 // Whether the library's plan for this grid takes two-sweep passes (fuse 0).
 bool two_sweep_default(const jac_grid *g);
 size_t sweep2_workspace_bytes(const jac_grid *g);
+// Resident sweeps (jac_resident.cu): the boxes of a small grid, one per CTA,
+// whose coefficients stay in shared memory for all sweeps of a call.
+struct ResidentShape {
+    int nj, nk;        // boxes along j and k
+    int bj, bk;        // most rows of a box along j and k
+    int ws;            // shared-memory row length (elements)
+    size_t smem;       // dynamic shared memory of a CTA
+};
+// False where the grid does not fit in the shared memory of `sms` SMs.
+bool resident_shape(int I, int J, int K, jac_prec prec, int sms, ResidentShape *out);
+size_t resident_workspace_bytes(const ResidentShape &s);
+// d_residual NULL: no residual is summed.
+jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, double *d_residual, void *workspace,
+                        cudaStream_t st);
 jac_status adjoint_step_dev(const jac_grid *g, const void *p_t, const void *lam_in, void *lam_out, double *g_wrk1,
                             double *g_a3, double *const *g_coef, int kdepth, void *workspace, size_t ws_bytes,
                             cudaStream_t st);

@@ -88,7 +88,7 @@ jac_status jac_sweep_dev_noalloc(const jac_grid *g, const jac_plan *plan, int n_
         jac::set_thread_error(std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
         return JAC_ECUDA;
     }
-    return jac::sweep_dev(g, &p, n_iter, d_residual, scratch, kNoAllocScratchBytes, stream);
+    return jac::sweep_dev(g, plan, n_iter, d_residual, scratch, kNoAllocScratchBytes, stream);
 }
 
 }  // extern "C"

@@ -428,6 +428,28 @@ size_t sweep_workspace_bytes(const jac_grid *g, const jac_plan &p)
     return std::max(single, sweep2_workspace_bytes(g));   // two-sweep passes may run
 }
 
+size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
+{
+    ResidentShape r;
+    const size_t need = sweep_workspace_bytes(g, p);
+    if (!resident_shape(g->I, g->J, g->K, g->prec, num_sms(), &r)) return need;
+    return std::max(need, resident_workspace_bytes(r));
+}
+
+// Whether a call runs resident (jac_resident.cu): the library's own plan, a
+// grid that fits in shared memory and a workspace with room for the flags (a
+// caller with a workspace sized for the streaming kernel keeps that one).
+// Measured with both kernels on every grid tried (17x17x17 to 65x65x129, all
+// precisions) a resident sweep takes 0.54-0.82 of a streaming one and the
+// launch up to 6 us more (the copy of the coefficients), so it pays from the
+// third sweep on; one or two sweeps stay with the streaming kernel.
+static bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r)
+{
+    if (n_iter < 3) return false;
+    if (plan && (plan->tile_i != 0 || plan->tile_j != 0 || plan->kdepth != 0 || plan->fuse != 0)) return false;
+    return resident_shape(g->I, g->J, g->K, g->prec, num_sms(), r) && ws_bytes >= resident_workspace_bytes(*r);
+}
+
 // Whether a call of n_iter sweeps runs as two-sweep passes.
 bool use_two_sweep_passes(const jac_grid *g, const jac_plan &p, int n_iter)
 {
@@ -451,6 +473,11 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15)) return fail(JAC_EINVAL, "bad workspace");
     const size_t need = sweep_workspace_bytes(g, p);
     if (ws_bytes < need) return fail(JAC_EINVAL, "workspace too small: need " + std::to_string(need) + " bytes");
+    ResidentShape shape;
+    if (!injected && use_resident(g, plan, n_iter, ws_bytes, &shape)) {
+        double *res = no_res ? nullptr : (d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual);
+        return resident_run(g, shape, n_iter, res, workspace, static_cast<cudaStream_t>(stream));
+    }
     if (!injected && use_two_sweep_passes(g, p, n_iter)) {
         // an even number of passes keeps the state of n sweeps in p[n % 2];
         // the remaining 0..3 sweeps run singly and give the residual if any
@@ -526,7 +553,7 @@ jac_status jac_sweep_workspace_size(const jac_grid *g, const jac_plan *plan, siz
     if (!bytes) return jac::fail(JAC_EINVAL, "bytes is NULL");
     jac_status s = jac::validate_grid(g);
     if (s != JAC_OK) return s;
-    *bytes = jac::sweep_workspace_bytes(g, jac::resolve_plan(g, plan));
+    *bytes = jac::sweep_workspace_reported(g, jac::resolve_plan(g, plan));
     return JAC_OK;
 }
 
