@@ -6,7 +6,7 @@
 // the pass and transforms them in registers and shared memory:
 //   * mixed-radix Stockham FFT of length N = R1 R2 R3 (radices 2..16):
 //     stage s reads R values at stride N / R, multiplies by the twiddles
-//     W_{Ns R}^{(j mod Ns) r} (from a table of W_N^m computed on the host in
+//     W_{Ns R}^{(j mod Ns) r} (from a table per stage computed on the host in
 //     FP64), does an R-point DFT in registers (radix-2 decimation in
 //     frequency with constant twiddles, its bit-reversed output order folded
 //     into the register indices) and writes R values at stride Ns, Ns = R1
@@ -22,6 +22,14 @@
 //     axis times one factor per line), and the last pass scales by 1/N as it
 //     stores and sums |u|^2 per CTA in FP64; a one-CTA kernel then adds the
 //     per-CTA sums in a fixed order, so the energy is bitwise reproducible.
+// What bounds a pass: FP32 passes of 512 points run at 4-5 TB/s of their own
+// reads and writes even when all of them hit L2, so instructions and latency
+// bound them, not DRAM; FP64 passes are bound by the FP64 pipe.  Hence
+// element offsets of a butterfly are constants (shared memory, twiddles) or a
+// running pointer (global), indices are 32 bits, and factors of 1 are not
+// multiplied by.  Before and after, on one GB300: x pass of 512x512x512 FP32
+// in 64 -> 48 registers; forward and one spectral step on 512^3 FP32 2.75 ->
+// 2.42 ms, on 256x256x128 FP64 2.67 -> 2.36 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -137,6 +145,10 @@ struct Radix {
     static constexpr int R3 = N <= 256 ? 1 : (N == 512 ? 8 : 16);
     static constexpr int RMAX = R1 > R2 ? (R1 > R3 ? R1 : R3) : (R2 > R3 ? R2 : R3);
     static_assert(R1 * R2 * R3 == N, "radix plan");
+    // The twiddles of the second and third stage: W^{jm r} of its length for
+    // jm < NS and r = 1 .. R-1 at [(r - 1) NS + jm], so that a butterfly reads
+    // them at constant offsets from jm.  N - R1 values in all.
+    static constexpr int TW3 = R1 * (R2 - 1), TW = N - R1;
 };
 
 // Elements of a line each thread holds.  The pass along x keeps the
@@ -169,6 +181,10 @@ __host__ __device__ constexpr int pad_idx(int e)
 {
     return sizeof(T) == 4 ? e + (e >> 4) : e + (e >> 3);
 }
+// pad_idx(a + x) = pad_idx(a) + pad_idx(x) for the indices of a stage: a lies
+// in a block of S elements that starts at a multiple of S (a power of two)
+// and x is a multiple of S, or the roles are swapped, so no carry crosses the
+// pad's digits.  The elements of a butterfly are then constants apart.
 
 // Row stride of the tile (elements): the padded line plus one, with the
 // stride odd in units of 32 bytes, so that lanes on different lines at the
@@ -183,7 +199,7 @@ __host__ __device__ constexpr int row_stride()
 struct PassArgs {
     const void *in;
     void *out;
-    const void *tw;          // W_N^m, m = 0 .. N-1, of this axis (forward sign)
+    const void *tw;          // this axis' twiddles by stage (Radix<N>; forward sign)
     int n1, n2, n3;
     int axis;                // 0: x, 1: y, 2: z
     int W;                   // lines per CTA
@@ -205,9 +221,6 @@ __device__ __forceinline__ double kbar2(int k, int n)
 // Programmatic dependent launch: a pass lets the next launch of the stream
 // start its prologue as soon as every CTA of this one runs, and waits for
 // everything before it in the stream ahead of its own first data access.
-// Small transforms are bound by their launches: 64x32x128 FP32 forward and
-// inverse 28.7 -> 22.4 us (with the twiddle copy and the data loads in flight
-// together); 512^3 gains 2.8% from overlapped tails.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_prior_grids() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -234,76 +247,64 @@ __device__ __forceinline__ void copy_async(E *smem_dst, const E *src)
                  : "memory");
 }
 
-// The first stage's inputs: radix R butterflies at stride N / R.
+// A thread's elements of a line are t + k TT, k = 0 .. RMAX-1; butterfly q of
+// a radix-R stage holds those with k = q + r RMAX / R.  The first stage's
+// inputs from `line` (this line's first element; es: its element stride).
 template <typename T, int N, int R, int RMAX>
-__device__ __forceinline__ void load_line(C2<T> (&v)[RMAX], const C2<T> *gin, long long lb, long long es, int t)
+__device__ __forceinline__ void load_line(C2<T> (&v)[RMAX], const C2<T> *line, unsigned es, int t)
 {
-    constexpr int TT = N / RMAX;
+    constexpr int TT = N / RMAX, BPT = RMAX / R;
+    const C2<T> *p = line + (unsigned)t * es;
 #pragma unroll
-    for (int q = 0; q < RMAX / R; ++q)
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[q * R + r] = gin[lb + (long long)(t + q * TT + r * (N / R)) * es];
+    for (int k = 0; k < RMAX; ++k, p += TT * es) v[(k % BPT) * R + k / BPT] = *p;
 }
 
-// One Stockham stage for the BPT = RMAX / R butterflies of this thread (the
-// first stage finds its inputs in v).
+// The last stage's outputs to `line`.
+template <typename T, int N, int R, int RMAX>
+__device__ __forceinline__ void store_line(const C2<T> (&v)[RMAX], C2<T> *line, unsigned es, int t)
+{
+    constexpr int TT = N / RMAX, BPT = RMAX / R;
+    C2<T> *p = line + (unsigned)t * es;
+#pragma unroll
+    for (int k = 0; k < RMAX; ++k, p += TT * es) *p = v[(k % BPT) * R + brev(k / BPT, R)];
+}
+
+// One Stockham stage for the BPT = RMAX / R butterflies of this thread: the
+// first finds its inputs in v, the last leaves its outputs there (the output
+// of index j + r N/R at v[q R + brev(r)]).
 template <typename T, int N, int R, int RMAX, int NS, bool INV, bool FIRST, bool LAST>
-__device__ __forceinline__ void stage(C2<T> (&v)[RMAX], C2<T> *tile, const C2<T> *tw, C2<T> *gout, long long lb, long long es, int w, int t, const T *fe, T fl, T scale,
-                                      bool factor, T &esum, bool want_energy)
+__device__ __forceinline__ void stage(C2<T> (&v)[RMAX], C2<T> *row, const C2<T> *tw, int t)
 {
     constexpr int TT = N / RMAX;       // threads per line
     constexpr int BPT = RMAX / R;      // butterflies per thread
-    constexpr int RS = row_stride<T, N>();
-    C2<T> *row = tile + w * RS;
+    if constexpr (!FIRST) {
 #pragma unroll
-    for (int q = 0; q < BPT; ++q) {
-        const int j = t + q * TT;
+        for (int q = 0; q < BPT; ++q) {
+            const C2<T> *p = row + pad_idx<T>(t + q * TT);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int e = j + r * (N / R);
-            if constexpr (FIRST) {
-                if (factor) {
-                    const T f = fe[e] * fl;
-                    v[q * R + r].x *= f;
-                    v[q * R + r].y *= f;
-                }
-            } else {
-                v[q * R + r] = row[pad_idx<T>(e)];
-            }
+            for (int r = 0; r < R; ++r) v[q * R + r] = p[pad_idx<T>(r * (N / R))];
         }
     }
     if constexpr (!FIRST && !LAST) __syncthreads();   // every read of the tile before any write
 #pragma unroll
     for (int q = 0; q < BPT; ++q) {
-        const int j = t + q * TT;
         if constexpr (NS > 1) {
-            const int jm = j & (NS - 1);
+            const C2<T> *w = tw + ((t + q * TT) & (NS - 1));
 #pragma unroll
-            for (int r = 1; r < R; ++r) v[q * R + r] = cmul<T, INV>(v[q * R + r], tw[jm * r * (N / (NS * R))]);
+            for (int r = 1; r < R; ++r) v[q * R + r] = cmul<T, INV>(v[q * R + r], w[(r - 1) * NS]);
         }
         Dif<T, R, R / 2, INV>::run(&v[q * R]);
     }
-    T e_loc = (T)0;     // this thread's |u|^2, summed in T over its outputs
+    if constexpr (!LAST) {
 #pragma unroll
-    for (int q = 0; q < BPT; ++q) {
-        const int j = t + q * TT;
-        const int idx = (j / NS) * NS * R + (j & (NS - 1));
+        for (int q = 0; q < BPT; ++q) {
+            const int j = t + q * TT;
+            C2<T> *p = row + pad_idx<T>((j / NS) * NS * R + (j & (NS - 1)));
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int e = idx + r * NS;
-            C2<T> x = v[q * R + brev(r, R)];
-            if constexpr (LAST) {
-                x.x *= scale;
-                x.y *= scale;
-                gout[lb + (long long)e * es] = x;
-                if (want_energy) e_loc = fma(x.x, x.x, fma(x.y, x.y, e_loc));
-            } else {
-                row[pad_idx<T>(e)] = x;
-            }
+            for (int r = 0; r < R; ++r) p[pad_idx<T>(r * NS)] = v[q * R + brev(r, R)];
         }
+        __syncthreads();
     }
-    if constexpr (LAST) esum += e_loc;
-    if constexpr (!LAST) __syncthreads();
 }
 
 template <typename T, int N, bool INV, bool YZ>
@@ -314,33 +315,31 @@ __global__ void __launch_bounds__(YZ ? 512 : 256, min_ctas_per_sm<T, YZ>()) k_ff
     constexpr int TT = N / RMAX;
     constexpr int RS = row_stride<T, N>();
     extern __shared__ __align__(16) unsigned char jfft_smem[];
+    constexpr int R1 = RX::R1, R2 = RX::R2, R3 = RX::R3;
     const int W = a.W;
     C2<T> *tile = reinterpret_cast<C2<T> *>(jfft_smem);
-    C2<T> *tw = tile + (RX::R2 > 1 ? W * RS : 0);
-    T *fe = reinterpret_cast<T *>(tw + N);
+    C2<T> *tw = tile + (R2 > 1 ? W * RS : 0);
+    T *fe = reinterpret_cast<T *>(tw + RX::TW);
     T *fl = fe + N;
     __shared__ double red[512];
 
-    // this thread's line and position in it
+    // This thread's line and position in it.  Element indices are at most
+    // 2^30 (three extents of 1024), so 32 bits hold them.
     int w, t;
-    if (a.axis == 0) { t = threadIdx.x % TT; w = threadIdx.x / TT; }
+    if (!YZ) { t = threadIdx.x % TT; w = threadIdx.x / TT; }
     else { w = threadIdx.x % W; t = threadIdx.x / W; }
-    const long long n1 = a.n1, n2 = a.n2;
-    long long lb, es;              // first element of the line, element stride
-    int ia, ib;                    // the line's indices on the other two axes
-    if (a.axis == 0) {
-        const long long row = (long long)blockIdx.x * W + w;     // row = z * n2 + y
+    const unsigned n1 = (unsigned)a.n1, n2 = (unsigned)a.n2;
+    unsigned lb, es = 1;           // first element of the line, element stride
+    int ia = 0, ib = 0;            // pass along x: the line's indices on the other two axes
+    if (!YZ) {
+        const unsigned row = blockIdx.x * W + w;                 // row = z * n2 + y
         lb = row * n1;
-        es = 1;
         ia = (int)(row % n2);
         ib = (int)(row / n2);
     } else {
-        const int xt = blockIdx.x % (a.n1 / W);
-        const int o = blockIdx.x / (a.n1 / W);                   // z (y pass) or y (z pass)
-        const int x = xt * W + w;
-        ia = x;
-        ib = o;
-        lb = a.axis == 1 ? (long long)o * n1 * n2 + x : (long long)o * n1 + x;
+        const unsigned xt = blockIdx.x % (n1 / W);
+        const unsigned o = blockIdx.x / (n1 / W);                // z (y pass) or y (z pass)
+        lb = (a.axis == 1 ? o * n1 * n2 : o * n1) + xt * W + w;
         es = a.axis == 1 ? n1 : n1 * n2;
     }
 
@@ -348,16 +347,16 @@ __global__ void __launch_bounds__(YZ ? 512 : 256, min_ctas_per_sm<T, YZ>()) k_ff
     // the twiddles into shared memory (constant since the plan was made, so
     // their copies need not wait for earlier launches) ...
     const C2<T> *gtw = static_cast<const C2<T> *>(a.tw);
-    if constexpr (RX::R2 > 1)
-        for (int m = threadIdx.x; m < N; m += blockDim.x) copy_async(&tw[m], &gtw[m]);
+    if constexpr (R2 > 1)
+        for (int m = threadIdx.x; m < RX::TW; m += blockDim.x) copy_async(&tw[m], &gtw[m]);
     asm volatile("cp.async.commit_group;" ::: "memory");
     wait_prior_grids();
     // ... and, with them in flight, this thread's part of its line
-    const C2<T> *gin = static_cast<const C2<T> *>(a.in);
-    C2<T> *gout = static_cast<C2<T> *>(a.out);
+    const C2<T> *gin = static_cast<const C2<T> *>(a.in) + lb;
+    C2<T> *gout = static_cast<C2<T> *>(a.out) + lb;
     C2<T> v[RMAX];
-    load_line<T, N, RX::R1, RMAX>(v, gin, lb, es, t);
-    if (a.factor) {                // the spectral factor along this axis and of this line
+    load_line<T, N, R1, RMAX>(v, gin, es, t);
+    if (!YZ && a.factor) {         // the spectral factor along this axis and of this line
         const T *gfa = static_cast<const T *>(a.fa);
         for (int m = threadIdx.x; m < N; m += blockDim.x) fe[m] = gfa[m];
         if (t == 0) fl[w] = static_cast<const T *>(a.fb)[ia] * static_cast<const T *>(a.fc)[ib];
@@ -365,26 +364,52 @@ __global__ void __launch_bounds__(YZ ? 512 : 256, min_ctas_per_sm<T, YZ>()) k_ff
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 
-    const bool want_energy = a.energy != nullptr;
-    const T scale = (T)a.scale;
-    const T flw = a.factor ? fl[w] : (T)1;
-    T esum = (T)0;
-    constexpr int R1 = RX::R1, R2 = RX::R2, R3 = RX::R3;
+    const bool want_energy = YZ && a.energy != nullptr;
+    if (!YZ && a.factor) {
+        const T flw = fl[w];
+#pragma unroll
+        for (int q = 0; q < RMAX / R1; ++q)
+#pragma unroll
+            for (int r = 0; r < R1; ++r) {
+                const T f = fe[t + q * TT + r * (N / R1)] * flw;
+                v[q * R1 + r].x *= f;
+                v[q * R1 + r].y *= f;
+            }
+    }
+    C2<T> *row = tile + w * RS;
+    constexpr int RL = R3 > 1 ? R3 : (R2 > 1 ? R2 : R1);         // radix of the last stage
     if constexpr (R2 == 1) {
-        stage<T, N, R1, RMAX, 1, INV, true, true>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
-                                                  a.factor, esum, want_energy);
-    } else if constexpr (R3 == 1) {
-        stage<T, N, R1, RMAX, 1, INV, true, false>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
-                                                   a.factor, esum, want_energy);
-        stage<T, N, R2, RMAX, R1, INV, false, true>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
-                                                    a.factor, esum, want_energy);
+        stage<T, N, R1, RMAX, 1, INV, true, true>(v, row, tw, t);
     } else {
-        stage<T, N, R1, RMAX, 1, INV, true, false>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
-                                                   a.factor, esum, want_energy);
-        stage<T, N, R2, RMAX, R1, INV, false, false>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
-                                                     a.factor, esum, want_energy);
-        stage<T, N, R3, RMAX, R1 * R2, INV, false, true>(v, tile, tw, gout, lb, es, w, t, fe, flw, scale,
-                                                         a.factor, esum, want_energy);
+        stage<T, N, R1, RMAX, 1, INV, true, false>(v, row, tw, t);
+        if constexpr (R3 == 1) {
+            stage<T, N, R2, RMAX, R1, INV, false, true>(v, row, tw, t);
+        } else {
+            stage<T, N, R2, RMAX, R1, INV, false, false>(v, row, tw, t);
+            stage<T, N, R3, RMAX, R1 * R2, INV, false, true>(v, row, tw + RX::TW3, t);
+        }
+    }
+    // Only the last pass of an inverse transform scales; elsewhere the factor
+    // is 1 and its two multiplies per point (of about 25 in FP64, which its
+    // pipe bounds) are left out.
+    if (YZ && a.scale != 1.0) {
+        const T scale = (T)a.scale;
+#pragma unroll
+        for (int q = 0; q < RMAX; ++q) { v[q].x *= scale; v[q].y *= scale; }
+    }
+    // the stride once more, opaque: without it the 16 offsets of the loads are
+    // kept in registers for the stores (and spill)
+    if (YZ) asm volatile("" : "+r"(es));
+    store_line<T, N, RL, RMAX>(v, gout, es, t);
+    T esum = (T)0;
+    if (want_energy) {             // this thread's |u|^2, summed in T over its outputs
+#pragma unroll
+        for (int q = 0; q < RMAX / RL; ++q)
+#pragma unroll
+            for (int r = 0; r < RL; ++r) {
+                const C2<T> x = v[q * RL + brev(r, RL)];
+                esum = fma(x.x, x.x, fma(x.y, x.y, esum));
+            }
     }
     if (!want_energy) return;
 
@@ -457,6 +482,16 @@ int rmax_of(int N)
 {
     if (N <= 16) return N;
     return (N == 32 || N == 64 || N == 512) ? 8 : 16;
+}
+
+// Radix<N>::R1, R2, R3 on the host.
+void radices_of(int N, int r[3])
+{
+    static const int table[11][3] = {{1, 1, 1}, {2, 1, 1},  {4, 1, 1},   {8, 1, 1}, {16, 1, 1},   {4, 8, 1},
+                                     {8, 8, 1}, {8, 16, 1}, {16, 16, 1}, {8, 8, 8}, {4, 16, 16}};
+    int e = 0;
+    while ((1 << e) < N) ++e;
+    for (int q = 0; q < 3; ++q) r[q] = table[e][q];
 }
 
 // Elements per thread (elems_per_thread<T, N, YZ> on the host).
@@ -565,7 +600,7 @@ jac_status launch_pass_t(int N, const PassArgs &a, unsigned grid, unsigned block
     case NN:                                                                                                \
         kern = k_fft_pass<T, NN, INV, YZ>;                                                                  \
         smem = (Radix<NN>::R2 > 1 ? (size_t)a.W * row_stride<T, NN>() * sizeof(C2<T>) : 0) +               \
-               (size_t)NN * sizeof(C2<T>) + (size_t)NN * sizeof(T) + (size_t)a.W * sizeof(T);               \
+               (size_t)Radix<NN>::TW * sizeof(C2<T>) + (size_t)NN * sizeof(T) + (size_t)a.W * sizeof(T);    \
         break;
         JFFT_CASE(2) JFFT_CASE(4) JFFT_CASE(8) JFFT_CASE(16) JFFT_CASE(32) JFFT_CASE(64) JFFT_CASE(128)
         JFFT_CASE(256) JFFT_CASE(512) JFFT_CASE(1024)
@@ -727,21 +762,29 @@ jac_status jfft_plan_create(jfft_plan **out, int n1, int n2, int n3, jfft_prec p
     p->stream = static_cast<cudaStream_t>(stream);
     p->ws = static_cast<char *>(workspace);
     p->L = L;
-    // twiddle tables W_N^m = exp(-2 pi i m / N), in FP64 on the host, stored in the plan's precision
+    // twiddle tables of the stages (Radix<N>), exp(-2 pi i jm r / (NS R)), in FP64 on the host, stored in the
+    // plan's precision
     std::vector<unsigned char> host(L.fac[0] - 256, 0);
     const double pi = 3.14159265358979323846264338327950288;
     for (int a = 0; a < 3; ++a) {
         unsigned char *dst = host.data() + (L.tw[a] - 256);
-        for (int m = 0; m < n[a]; ++m) {
-            const double re = std::cos(2.0 * pi * m / n[a]), im = -std::sin(2.0 * pi * m / n[a]);
-            if (prec == JFFT_C64) {
-                const double v[2] = {re, im};
-                std::memcpy(dst + (size_t)m * 16, v, 16);
-            } else {
-                const float v[2] = {(float)re, (float)im};
-                std::memcpy(dst + (size_t)m * 8, v, 8);
-            }
-        }
+        int r3[3];
+        jfft::radices_of(n[a], r3);
+        int at = 0;
+        for (int st = 1, ns = r3[0]; st < 3; ns *= r3[st], ++st)
+            for (int r = 1; r < r3[st]; ++r)
+                for (int jm = 0; jm < ns; ++jm, ++at) {
+                    const int m = jm * r;                    // of ns * r3[st] points
+                    const double ang = 2.0 * pi * m / (ns * r3[st]);
+                    const double re = std::cos(ang), im = -std::sin(ang);
+                    if (prec == JFFT_C64) {
+                        const double v[2] = {re, im};
+                        std::memcpy(dst + (size_t)at * 16, v, 16);
+                    } else {
+                        const float v[2] = {(float)re, (float)im};
+                        std::memcpy(dst + (size_t)at * 8, v, 8);
+                    }
+                }
     }
     cudaError_t e = cudaMemsetAsync(p->ws, 0, 256, p->stream);
     if (e == cudaSuccess)
