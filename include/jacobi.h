@@ -134,11 +134,13 @@ typedef struct jac_grid {
  * (FP64 storage only; with FP32 storage they measured slower than the
  * rule above, and the call returns JAC_EINVAL).
  * Unsupported shapes: JAC_EINVAL at launch.
- * A plan of all zeros (or NULL) leaves the kernel to the library as well:
- * calls of three sweeps or more on grids whose coefficients fit in the shared
- * memory of all SMs together run resident (one launch that keeps them there
- * and exchanges only the rows between neighbouring CTAs; the state is bitwise
- * the same).  Any non-zero field selects the kernel described above. */
+ * A plan of all zeros (or NULL) leaves the kernel to the library as well;
+ * the state is bitwise the same.  Calls of three sweeps or more on grids whose
+ * coefficients fit in the shared memory of all SMs together run resident (one
+ * launch that keeps them there and exchanges only the rows between
+ * neighbouring CTAs), and FP32 grids run two sweeps per pass where that is
+ * estimated to be faster, whatever the size of their state.  Any non-zero
+ * field selects the kernels as described here. */
 enum { JAC_KDEPTH_BALANCED = -1 };
 typedef struct jac_plan {
     int tile_j;   /* rows per work item */
@@ -164,16 +166,17 @@ typedef struct jac_plan {
  * measurement otherwise (Section 4).
  * The plan a sweep of this grid would run with on a device of sm_count SMs
  * (one CTA per SM; sm_count <= 0: the current device's count): the zero
- * fields of *plan (NULL: all zero) filled in by the rules above.  Only the
+ * fields of *plan (NULL: all zero) filled in by the rules above.  (A call with
+ * all zeros may choose another kernel, see jac_plan; the state is the same.)  Only the
  * dimensions and the precision of *g are read; no device memory is touched,
  * and with sm_count > 0 no GPU is needed.  Errors: JAC_EINVAL for bad
  * dimensions, precision or plan entries, or a shape the kernels lack. */
 jac_status jac_resolve_plan(const jac_grid *g, const jac_plan *plan, int sm_count, jac_plan *out);
 
 /* Bytes of device workspace for jac_sweep_dev on this grid and plan (host
- * only).  It includes the flags of the resident kernel where the grid can
- * take it; jac_sweep_dev also accepts a workspace without room for them (256
- * bytes and one double per CTA of the plan) and then never runs resident.  No paper counterpart (the caller-owned scratch of the
+ * only).  It has room for every kernel the library may choose for a plan of
+ * all zeros; jac_sweep_dev also accepts a smaller workspace (256 bytes and one
+ * double per CTA of the plan) and then keeps to that plan.  No paper counterpart (the caller-owned scratch of the
  * stateless form). */
 jac_status jac_sweep_workspace_size(const jac_grid *g, const jac_plan *plan, size_t *bytes);
 

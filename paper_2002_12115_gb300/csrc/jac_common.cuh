@@ -17,7 +17,7 @@ struct WsHeader {
     int errword;          // JAC_OK or JAC_ETIMEOUT, written by kernels
     unsigned counter;     // CTAs finished (last one reduces and resets)
     unsigned gbar;        // grid barrier between sweeps of one launch
-    unsigned pad0;
+    unsigned ticket;      // items taken from a launch's common list (two-sweep passes)
     double residual;      // default destination of the residual
 };
 constexpr size_t kWsHeaderBytes = 256;

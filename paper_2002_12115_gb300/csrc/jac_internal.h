@@ -62,8 +62,8 @@ template <bool BATCH>
 jac_status launch_sweep(jac_prec prec, int tj, const GridDesc &d0, const SweepArgs &a, unsigned nblocks,
                         cudaStream_t st);
 // Two-sweep passes (FP32 storage): n_pass passes of two sweeps each, in one
-// cooperative launch; the residual of the last sweep to d_residual (NULL:
-// none).  kdepth 0: the default depth.
+// cooperative launch (very long calls: several); the residual of the last
+// sweep to d_residual (NULL: none).  kdepth 0: the default depth.
 // Two-sweep passes (FP32 storage): pass t reads p[t & 1] and writes the other
 // buffer.  mid (one-pass calls only) also receives the state after the first
 // sweep at every interior point; its faces are left as they are.
@@ -72,6 +72,8 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
 // Whether the library's plan for this grid takes two-sweep passes (fuse 0).
 bool two_sweep_default(const jac_grid *g);
 size_t sweep2_workspace_bytes(const jac_grid *g);
+// Steps of a two-sweep pass over the grid, and its tiles along i.
+long sweep2_steps(const jac_grid *g, int *tiles_i);
 // Resident sweeps (jac_resident.cu): the boxes of a small grid, one per CTA,
 // whose coefficients stay in shared memory for all sweeps of a call.
 struct ResidentShape {

@@ -428,12 +428,19 @@ size_t sweep_workspace_bytes(const jac_grid *g, const jac_plan &p)
     return std::max(single, sweep2_workspace_bytes(g));   // two-sweep passes may run
 }
 
+// Whether a plan leaves everything to the library.
+static bool all_zero(const jac_plan *plan)
+{
+    return !plan || (plan->tile_i == 0 && plan->tile_j == 0 && plan->kdepth == 0 && plan->fuse == 0);
+}
+
 size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
 {
     ResidentShape r;
-    const size_t need = sweep_workspace_bytes(g, p);
-    if (!resident_shape(g->I, g->J, g->K, g->prec, num_sms(), &r)) return need;
-    return std::max(need, resident_workspace_bytes(r));
+    size_t need = sweep_workspace_bytes(g, p);
+    if (g->prec == JAC_F32) need = std::max(need, sweep2_workspace_bytes(g));
+    if (resident_shape(g->I, g->J, g->K, g->prec, num_sms(), &r)) need = std::max(need, resident_workspace_bytes(r));
+    return need;
 }
 
 // Whether a call runs resident (jac_resident.cu): the library's own plan, a
@@ -446,8 +453,33 @@ size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
 static bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r)
 {
     if (n_iter < 3) return false;
-    if (plan && (plan->tile_i != 0 || plan->tile_j != 0 || plan->kdepth != 0 || plan->fuse != 0)) return false;
+    if (!all_zero(plan)) return false;
     return resident_shape(g->I, g->J, g->K, g->prec, num_sms(), r) && ws_bytes >= resident_workspace_bytes(*r);
+}
+
+// Whether a call of n_iter sweeps with the library's own plan (all zero) takes
+// two-sweep passes: the faster of the two by the measured rates of both
+// kernels (16 FP32 grids, 65x200x200 to 513x513x1025).  A step of a pass's
+// busiest CTA takes 1.55 us where both state buffers stay in half the L2, 1.67
+// where they do not, and 2.0 from three tiles along i on (more of its columns
+// and rows come from DRAM twice).  A single sweep takes 2 us and 7.1 ns per
+// 1000 points in the first case and 8.5 ns per 1000 points otherwise.  What
+// decides is how well 128 columns by 8 rows tile the grid: 129x129x257 (full
+// tiles) 31.1 us a sweep against 25.6 in passes, 161x161x161 (two tiles 62%
+// full) 29.8 against 43.5.  The single sweeps after the passes are a launch of
+// their own (11 us).
+static bool two_sweeps_pay(const jac_grid *g, int n_iter)
+{
+    if (g->prec != JAC_F32 || n_iter < 4) return false;
+    int tiles_i = 1;
+    const long steps = sweep2_steps(g, &tiles_i);
+    const double state = 2.0 * (double)jac_pitch(g->I) * g->J * g->K * 4.0;
+    const bool kept = state <= 0.5 * (double)device_l2_bytes();
+    const double points = (double)(g->I - 2) * (g->J - 2) * (g->K - 2);
+    const double two = 0.5 * (kept ? 1.55 : (tiles_i > 2 ? 2.0 : 1.67)) * (double)steps;   // us a sweep
+    const double one = kept ? 2.0 + 7.1e-6 * points : 8.5e-6 * points;
+    const int in_passes = 4 * (n_iter / 4), rest = n_iter - in_passes;
+    return in_passes * two + (rest ? 11.0 + rest * one : 0.0) < n_iter * one;
 }
 
 // Whether a call of n_iter sweeps runs as two-sweep passes.
@@ -466,13 +498,15 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     if (s != JAC_OK) return s;
     if (n_iter < 0) return fail(JAC_EINVAL, "n_iter must be >= 0");
     if (n_iter == 0) return JAC_OK;
-    const jac_plan p = resolve_plan(g, plan);
+    jac_plan p = resolve_plan(g, plan);
     int rw = 0, tj = 0;
     if ((s = check_plan(g->prec, p, &rw, &tj)) != JAC_OK) return s;
     if (p.fuse < 0 || p.fuse > 2) return fail(JAC_EINVAL, "fuse must be 0, 1 or 2");
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15)) return fail(JAC_EINVAL, "bad workspace");
     const size_t need = sweep_workspace_bytes(g, p);
     if (ws_bytes < need) return fail(JAC_EINVAL, "workspace too small: need " + std::to_string(need) + " bytes");
+    if (all_zero(plan) && g->prec == JAC_F32)
+        p.fuse = two_sweeps_pay(g, n_iter) && ws_bytes >= sweep2_workspace_bytes(g) ? 2 : 1;
     ResidentShape shape;
     if (!injected && use_resident(g, plan, n_iter, ws_bytes, &shape)) {
         double *res = no_res ? nullptr : (d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual);

@@ -16,36 +16,47 @@
 //     R1 = R2 + 2 rows j0-1 .. j0+R2 and the planes kb-1 .. ke; sweep 2 over
 //     the R2 inner rows and planes kb .. ke-1.  Tiles do not overlap: sweep 2
 //     at columns i0 and i0+127 needs sweep 1 at columns i0-1 and i0+128 too;
+//   * CTAs take the items of a pass by ticket, in the order of their numbers,
+//     so that tiles next to one another are worked on at about the same time
+//     and no CTA waits for a slower one before the end of a pass; the queue
+//     entry of a CTA's next item carries its pass.  A last pass with a
+//     residual assigns items by CTA number, so that its sum has a fixed order.
+//     Before the state of pass t the producer waits until every item of the
+//     passes before is stored (a counter; each sweep-2 warp adds one per item);
 //   * warp 10 (one lane) copies, in the order they are used, the planes of
 //     p_t with a halo of 4 columns and 2 rows into a ring of 4 slots, and the
 //     twelve coefficient tiles (128 x R1) of every sweep-1 plane into a ring
-//     of 2 stages, which sweep 1 alone uses.  Before the state of pass
-//     t >= 1 it waits on the grid barrier of the pass before;
-//   * consumer warp w (0 .. R1-1) owns row j0-1+w.  At step s (plane
-//     m = kb-1+s) it computes sweep 1 there into a ring of 4 intermediate
-//     planes, then (warps 1 .. R1-2, s >= 3) sweep 2 at plane m-2 from the
-//     intermediate planes m-3 .. m-1.  Sweep 2 trails by two planes so that
-//     its wait (every row of plane m-1 written: an mbarrier per
-//     intermediate plane) is for work the other warps finished a step ago,
-//     not for the step in flight.  Its coefficients come from global memory
-//     (the tiles were copied for sweep 1 two steps earlier, so they are read
-//     from L2) into a 6 KB buffer per warp: each lane copies its own 12 x 16
-//     bytes with cp.async at the end of a step, for the next step's sweep 2,
-//     so the L2 latency is hidden behind sweep 1.  (Keeping the stages for
-//     three steps would need four 61 KB stages in flight.)
+//     of 3 stages;
+//   * warps 0 .. R1-1 compute sweep 1, one row each, into a ring of 4
+//     intermediate planes.  A row that is an output row too keeps its twelve
+//     coefficients and a3 S - 1 in tensor memory (13 values per point, three
+//     planes; tcgen05.st/ld with each lane's own points), so that sweep 2
+//     reads neither global memory nor a stage that would have to be kept;
+//   * warps 12 .. 19 compute sweep 2, one row each, a plane behind the newest
+//     intermediate plane.  A row's sweep-2 warp has the index of its sweep-1
+//     warp modulo 4, since a warp reaches only its quarter of tensor memory;
 //   * warp 11 (the edge warp, 20 lanes) computes sweep 1 at columns i0-1 and
-//     i0+128 of the R1 rows at every step, from the state ring and
-//     coefficients it loads from global memory one plane ahead (those
-//     columns belong to the neighbouring tiles, whose CTAs copy them at
-//     about the same time);
-//   * the residual of the last pass's second sweep is reduced as in the
-//     single-sweep kernel; every wait is bounded;
+//     i0+128 of the R1 rows, from the state ring and coefficients it loads
+//     from global memory one plane ahead;
+//   * both sweeps take the update in two parts (ss_axes, ss_rest), so that 96
+//     registers hold one part's coefficients and the stencil's state values;
+//   * every wait is bounded; on expiry the kernel sets the workspace error
+//     word, drains its own copies, frees its tensor memory and returns;
 //   * a one-pass call may also store sweep 1's state at the points the
 //     items own (Sweep2Args::mid): the reverse pass recomputes two
 //     checkpoint-segment states per launch that way.
 //
-// Twelve warps leave 168 registers a thread (a thirteenth would put four
-// warps on one SM sub-partition and cap them at 128).
+// What bounds it: a step of a CTA (one plane of a tile, both sweeps) takes
+// 1.65 us up to two tiles along i, whether the state stays in L2 or not
+// (latency and issue of 18 compute warps), and 1.8-2.0 us from three tiles on,
+// where it draws 5.4 TB/s from DRAM.  Kept against, on one GB300 (Gpt/s, FP32):
+//                                             257x257x513   513x513x1025
+//   both sweeps in one warp, coefficients of
+//     sweep 2 read again from L2 (41% of all
+//     L2 reads)                                    141            145
+//   ... kept in tensor memory                      150            153
+//   separate warps for the two sweeps              164            143
+//   ... and items by ticket (this kernel)          171            149
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -64,14 +75,18 @@ struct Sweep2Shape {
     static constexpr int TILE = TI * R1 * 4;                 // one coefficient tile, 5120
     static constexpr int C_BYTES = 12 * TILE;                // one stage
     static constexpr int Q_BYTES = TI * R1 * 4;              // one intermediate plane
-    static constexpr int B_BYTES = 12 * TI * 4;              // one warp's sweep-2 coefficients of one row
-    static constexpr int RP = 4, RC = 2, RQ = 4;
-    static constexpr size_t SMEM =
-        (size_t)RP * P_BYTES + (size_t)RQ * Q_BYTES + (size_t)RC * C_BYTES + (size_t)R2 * B_BYTES + 128;
+    static constexpr int RP = 4, RC = 3, RQ = 4;
+    static constexpr size_t SMEM = (size_t)RP * P_BYTES + (size_t)RQ * Q_BYTES + (size_t)RC * C_BYTES + 128;
+    static constexpr int TM_SLOT = 13 * VI;                  // tensor-memory columns of one row: 12 coefficients, a3 S - 1
+    static constexpr int TM_SLOTS = 3;                       // planes m-2 .. m
+    static constexpr int TM_COLS = 512;                      // allocated (a power of two)
     static constexpr int EDGE_WARP = R1 + 1;                 // sweep 1 at the two columns past the tile
-    static constexpr int THREADS = 32 * (R1 + 2);
-    static_assert(P_BYTES % 128 == 0 && Q_BYTES % 128 == 0 && C_BYTES % 128 == 0 && B_BYTES % 128 == 0,
-                  "slot alignment");
+    static constexpr int WARP2 = R1 + 2;                     // first of the R2 sweep-2 warps
+    static constexpr int THREADS = 32 * (R1 + 2 + R2);
+    static constexpr int NQ = 4;                             // item queue of a CTA
+    static constexpr uint32_t END = 0xffffffffu;             // no further item
+    static_assert(P_BYTES % 128 == 0 && Q_BYTES % 128 == 0 && C_BYTES % 128 == 0, "slot alignment");
+    static_assert(R2 / 4 * TM_SLOTS * TM_SLOT <= TM_COLS && WARP2 % 4 == 0 && R2 % 4 == 0, "tensor memory columns");
 };
 
 struct Sweep2Desc {
@@ -85,6 +100,7 @@ struct Sweep2Desc {
 
 struct Sweep2Args {
     int n_pass, par;           // pass t reads p[(t + par) & 1], writes the other
+    unsigned taken;            // items of the passes whose items are taken by ticket
     double omega;
     double *partials;          // gridDim.x
     double *res;               // residual of the last pass's second sweep (NULL: none)
@@ -125,14 +141,60 @@ __device__ __forceinline__ void q_ext(const float *row, int lane, float left, fl
     e[5] = (lane == 31) ? right : r;
 }
 
-// 16 bytes global -> shared without a register round trip (cached in L2
-// only); the copies of a thread complete at cp_async_wait_all.
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *src)
+// Tensor memory as a per-lane scratchpad: a warp reaches the 32 lanes of its
+// quarter (warp index mod 4); lane l of the warp owns column values of lane l.
+__device__ __forceinline__ void tmem_alloc(uint32_t *smem_addr, int cols)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(src) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_addr)),
+                 "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void tmem_dealloc(uint32_t addr, int cols)
+{
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols) : "memory");
+}
+// Four arrays of four values (one lane's) to or from 16 columns.
+__device__ __forceinline__ void tmem_st16(uint32_t addr, const float (&a)[4], const float (&b)[4], const float (&c)[4],
+                                          const float (&d)[4])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16};" ::"r"(addr),
+        "f"(a[0]), "f"(a[1]), "f"(a[2]), "f"(a[3]), "f"(b[0]), "f"(b[1]), "f"(b[2]), "f"(b[3]), "f"(c[0]), "f"(c[1]),
+        "f"(c[2]), "f"(c[3]), "f"(d[0]), "f"(d[1]), "f"(d[2]), "f"(d[3])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t addr, const float (&a)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a[0]), "f"(a[1]),
+                 "f"(a[2]), "f"(a[3])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&a)[4], float (&b)[4], float (&c)[4], float (&d)[4])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3]), "=f"(c[0]),
+          "=f"(c[1]), "=f"(c[2]), "=f"(c[3]), "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(addr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t addr, float (&a)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Ties loaded values to the wait before it: no use of them moves above it.
+__device__ __forceinline__ void tmem_loaded(float (&a)[4])
+{
+    asm volatile("" : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3])::"memory");
+}
 
 __global__ void __launch_bounds__(Sweep2Shape::THREADS, 1)
 k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
@@ -144,11 +206,12 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(dsm2_raw) + 127) & ~uintptr_t(127));
     unsigned char *ring_q = base + (size_t)RP * S::P_BYTES;
     unsigned char *ring_c = ring_q + (size_t)RQ * S::Q_BYTES;
-    unsigned char *bufs2 = ring_c + (size_t)RC * S::C_BYTES;   // per sweep-2 warp
     __shared__ __align__(8) uint64_t p_full[RP], p_empty[RP], c_full[RC], c_empty[RC], q_full[RQ], q_empty[RQ],
-        cons_bar;
+        i_full[S::NQ], i_empty[S::NQ], cons_bar;
+    __shared__ uint32_t s_item[S::NQ];
     __shared__ volatile int s_abort;
-    __shared__ double s_part[R1];
+    __shared__ uint32_t s_tmem;
+    __shared__ double s_part[S::R2];
     __shared__ float q_edge[RQ][R1][2];   // sweep-1 values at columns i0-1 and i0+128, per row
 
     const int warp = threadIdx.x >> 5;
@@ -158,12 +221,28 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
     if (threadIdx.x == 0) {
         for (int s = 0; s < RP; ++s) { mbar_init(&p_full[s], 1); mbar_init(&p_empty[s], R1 + 1); }
         for (int s = 0; s < RC; ++s) { mbar_init(&c_full[s], 1); mbar_init(&c_empty[s], R1); }
-        for (int s = 0; s < RQ; ++s) { mbar_init(&q_full[s], R1 + 1); mbar_init(&q_empty[s], R1); }
-        mbar_init(&cons_bar, R1);
+        for (int s = 0; s < RQ; ++s) { mbar_init(&q_full[s], R1 + 1); mbar_init(&q_empty[s], S::R2); }
+        for (int s = 0; s < S::NQ; ++s) { mbar_init(&i_full[s], 1); mbar_init(&i_empty[s], R1 + 1 + S::R2); }
+        mbar_init(&cons_bar, S::R2);
         s_abort = 0;
         fence_mbar_init();
     }
+    if (warp == S::EDGE_WARP) tmem_alloc(&s_tmem, S::TM_COLS);
     __syncthreads();
+
+    // The next entry of the CTA's item queue (every warp but the producer's
+    // reads each entry): pass * nitems + item, or END; false: give up.
+    uint32_t ic = 0;
+    auto next_item = [&](uint32_t &entry) -> bool {
+        bool r = mbar_wait_bounded(&i_full[ic % S::NQ], (ic / S::NQ) & 1);
+        r = __all_sync(0xffffffffu, r && !s_abort);
+        entry = s_item[ic % S::NQ];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&i_empty[ic % S::NQ]);
+        ++ic;
+        return r;
+    };
+    const uint32_t nitems = (uint32_t)d.nitems;
 
     if (warp == R1) {
         // ------------------------------------------------------------ producer
@@ -171,10 +250,10 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         // plane (twelve 128 x R1 tiles) and the state planes of p_t with a
         // halo of 4 columns and 2 rows, in the order the consumers use them:
         // state planes 0 and 1, then per step s state plane s+2 and stage
-        // s+1.  Before the state of pass t >= 1 it waits on the grid barrier
-        // of the pass before (the first stage of the pass does not need it).
+        // s+1.  Before the state of pass t >= 1 it waits until the passes
+        // before are stored (the first stage of an item does not need it).
         if (lane == 0) {
-            const uint64_t pol_c = l2_policy(0);   // sweep 2 reads the tiles again from L2
+            const uint64_t pol_c = l2_policy(a.l2_keep_state ? -1 : 0);
             const uint64_t pol_keep = l2_policy(1);
             const uint64_t pol_p = l2_policy(a.l2_keep_state ? 1 : 0);
             uint32_t pc = 0, cc = 0;
@@ -202,23 +281,44 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 ++cc;
                 return true;
             };
-            for (int t = 0; t < a.n_pass && ok; ++t) {
+            // Items in the order of their numbers, whichever CTA is free: the
+            // first one by CTA number, then by ticket, and those of a last
+            // pass with a residual by CTA number again (a fixed assignment
+            // keeps the order of its sum).
+            uint32_t ip = 0, entry = blockIdx.x, pass = 0;
+            bool by_ticket = a.taken > 0;
+            if (!by_ticket) entry += (uint32_t)(a.n_pass - 1) * nitems;
+            const uint32_t total = (uint32_t)a.n_pass * nitems;
+            while (ok) {
+                const uint32_t qslot = ip % S::NQ;
+                if (ip >= S::NQ && !(ok = mbar_wait_bounded(&i_empty[qslot], ((ip / S::NQ) - 1) & 1))) break;
+                s_item[qslot] = entry;
+                mbar_arrive(&i_full[qslot]);
+                ++ip;
+                if (entry == S::END) break;
+                uint32_t next = 0;
+                if (by_ticket) next = (uint32_t)G + atomicAdd(&a.hdr->ticket, 1u);   // used after this item
+                const uint32_t t = entry / nitems;
+                const Item2 it = decode_item2(d, (int)(entry - t * nitems));
                 pm = ((t + a.par) & 1) ? &d.p[1] : &d.p[0];
-                bool first = true;
-                for (int item = blockIdx.x; item < d.nitems && ok; item += G) {
-                    const Item2 it = decode_item2(d, item);
-                    if (!(ok = put_coef(it, 0))) break;
-                    if (t > 0 && first) {
-                        if (!(ok = wait_counter_bounded(&a.hdr->gbar, (unsigned)t * G))) break;
-                        fence_proxy_async_global();
-                    }
-                    first = false;
-                    if (!(ok = put_state(it, 0) && put_state(it, 1))) break;
-                    for (int q = 0; q < it.nout + 2 && ok; ++q) {
-                        ok = put_state(it, q + 2);
-                        if (ok && q + 1 < it.nout + 2) ok = put_coef(it, q + 1);
-                    }
+                if (!(ok = put_coef(it, 0))) break;
+                if (t > pass) {            // every item of the passes before is stored
+                    pass = t;
+                    if (!(ok = wait_counter_bounded(&a.hdr->gbar, t * nitems * S::R2))) break;
+                    fence_proxy_async_global();
                 }
+                if (!(ok = put_state(it, 0) && put_state(it, 1))) break;
+                for (int q = 0; q < it.nout + 2 && ok; ++q) {
+                    ok = put_state(it, q + 2);
+                    if (ok && q + 1 < it.nout + 2) ok = put_coef(it, q + 1);
+                }
+                if (by_ticket && next >= a.taken) {
+                    by_ticket = false;
+                    next = a.taken < total ? a.taken + blockIdx.x : S::END;
+                } else if (!by_ticket) {
+                    next = entry + (uint32_t)G < total ? entry + (uint32_t)G : S::END;
+                }
+                entry = next;
             }
             if (!ok) {
                 s_abort = 1;
@@ -247,85 +347,228 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         const int r0 = r * S::PW, r1 = (r + 1) * S::PW, r2 = (r + 2) * S::PW;
         uint32_t pc = 0, qc = 0;
         bool ok = true;
-        for (int t = 0; t < a.n_pass && ok; ++t) {
-            for (int item = blockIdx.x; item < d.nitems && ok; item += G) {
-                const Item2 it = decode_item2(d, item);
-                const int j = it.j0 - 1 + r;
-                const int ie = side ? it.i0 + TI : it.i0 - 1;
-                const bool col_in = act && (j >= 1) && (j <= J - 2) && (ie >= 1) && (ie <= I - 2);
-                float cf[12], cn[12];
-                auto load_coef = [&](int m, float (&v)[12]) {
-                    if (col_in && m >= 1 && m <= K - 2) {
-                        const size_t off = ((size_t)m * J + (size_t)j) * (size_t)pitch + (size_t)ie;
+        uint32_t entry;
+        while ((ok = next_item(entry)) && entry != S::END) {
+            const Item2 it = decode_item2(d, (int)(entry % nitems));
+            const int j = it.j0 - 1 + r;
+            const int ie = side ? it.i0 + TI : it.i0 - 1;
+            const bool col_in = act && (j >= 1) && (j <= J - 2) && (ie >= 1) && (ie <= I - 2);
+            float cf[12], cn[12];
+            auto load_coef = [&](int m, float (&v)[12]) {
+                if (col_in && m >= 1 && m <= K - 2) {
+                    const size_t off = ((size_t)m * J + (size_t)j) * (size_t)pitch + (size_t)ie;
 #pragma unroll
-                        for (int q = 0; q < 12; ++q) v[q] = __ldg(d.coef_ptr[q] + off);
-                    } else {
+                    for (int q = 0; q < 12; ++q) v[q] = __ldg(d.coef_ptr[q] + off);
+                } else {
 #pragma unroll
-                        for (int q = 0; q < 12; ++q) v[q] = 0.0f;
-                    }
-                };
-                load_coef(it.kb - 1, cf);
-                for (int s = 0; s < it.nout + 2; ++s) {
-                    const int m = it.kb - 1 + s;
-                    if (s == 0) {
-                        ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
-                             mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
-                    }
-                    const uint32_t q2 = pc + s + 2;
-                    ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
-                    const uint32_t qs = qc + s;
-                    if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
-                    ok = __all_sync(0xffffffffu, ok && !s_abort);
-                    if (!ok) break;
-                    if (s + 1 < it.nout + 2) load_coef(m + 1, cn);
-                    if (act) {
-                        const float *Pm = reinterpret_cast<const float *>(base + (size_t)((pc + s) % RP) * S::P_BYTES);
-                        const float *Pk =
-                            reinterpret_cast<const float *>(base + (size_t)((pc + s + 1) % RP) * S::P_BYTES);
-                        const float *Pp = reinterpret_cast<const float *>(base + (size_t)(q2 % RP) * S::P_BYTES);
-                        const float c = Pk[r1 + x];
-                        float out = c;
-                        if (col_in && m >= 1 && m <= K - 2) {
-                            const float bij = ((Pk[r2 + x + 1] - Pk[r0 + x + 1]) - Pk[r2 + x - 1]) + Pk[r0 + x - 1];
-                            const float bjk = ((Pp[r2 + x] - Pm[r2 + x]) - Pp[r0 + x]) + Pm[r0 + x];
-                            const float bik = ((Pp[r1 + x + 1] - Pm[r1 + x + 1]) - Pp[r1 + x - 1]) + Pm[r1 + x - 1];
-                            const float ss = ss_f32<false>(c, Pk[r1 + x + 1], Pk[r1 + x - 1], Pk[r2 + x], Pk[r0 + x],
-                                                           Pp[r1 + x], Pm[r1 + x], bij, bjk, bik, cf[0], cf[1], cf[2],
-                                                           cf[3], cf[4], cf[5], cf[6], cf[7], cf[8], cf[9], cf[10],
-                                                           cf[11]);
-                            out = fmaf(omega, ss, c);
-                        }
-                        q_edge[qs % RQ][r][side] = out;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 12; ++q) cf[q] = cn[q];
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(&q_full[qs % RQ]);            // the edge values of intermediate plane s
-                        mbar_arrive(&p_empty[(pc + s) % RP]);     // state plane m-1 is done
-                    }
+                    for (int q = 0; q < 12; ++q) v[q] = 0.0f;
                 }
+            };
+            load_coef(it.kb - 1, cf);
+            for (int s = 0; s < it.nout + 2; ++s) {
+                const int m = it.kb - 1 + s;
+                if (s == 0) {
+                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
+                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
+                }
+                const uint32_t q2 = pc + s + 2;
+                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
+                const uint32_t qs = qc + s;
+                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
+                ok = __all_sync(0xffffffffu, ok && !s_abort);
                 if (!ok) break;
+                if (s + 1 < it.nout + 2) load_coef(m + 1, cn);
+                if (act) {
+                    const float *Pm = reinterpret_cast<const float *>(base + (size_t)((pc + s) % RP) * S::P_BYTES);
+                    const float *Pk =
+                        reinterpret_cast<const float *>(base + (size_t)((pc + s + 1) % RP) * S::P_BYTES);
+                    const float *Pp = reinterpret_cast<const float *>(base + (size_t)(q2 % RP) * S::P_BYTES);
+                    const float c = Pk[r1 + x];
+                    float out = c;
+                    if (col_in && m >= 1 && m <= K - 2) {
+                        const float bij = ((Pk[r2 + x + 1] - Pk[r0 + x + 1]) - Pk[r2 + x - 1]) + Pk[r0 + x - 1];
+                        const float bjk = ((Pp[r2 + x] - Pm[r2 + x]) - Pp[r0 + x]) + Pm[r0 + x];
+                        const float bik = ((Pp[r1 + x + 1] - Pm[r1 + x + 1]) - Pp[r1 + x - 1]) + Pm[r1 + x - 1];
+                        const float ss = ss_f32<false>(c, Pk[r1 + x + 1], Pk[r1 + x - 1], Pk[r2 + x], Pk[r0 + x],
+                                                       Pp[r1 + x], Pm[r1 + x], bij, bjk, bik, cf[0], cf[1], cf[2],
+                                                       cf[3], cf[4], cf[5], cf[6], cf[7], cf[8], cf[9], cf[10],
+                                                       cf[11]);
+                        out = fmaf(omega, ss, c);
+                    }
+                    q_edge[qs % RQ][r][side] = out;
+                }
+#pragma unroll
+                for (int q = 0; q < 12; ++q) cf[q] = cn[q];
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(&p_empty[(pc + it.nout + 2) % RP]);
-                    mbar_arrive(&p_empty[(pc + it.nout + 3) % RP]);
+                    mbar_arrive(&q_full[qs % RQ]);            // the edge values of intermediate plane s
+                    mbar_arrive(&p_empty[(pc + s) % RP]);     // state plane m-1 is done
                 }
-                pc += it.nout + 4;
-                qc += it.nout + 2;
             }
+            if (!ok) break;
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&p_empty[(pc + it.nout + 2) % RP]);
+                mbar_arrive(&p_empty[(pc + it.nout + 3) % RP]);
+            }
+            pc += it.nout + 4;
+            qc += it.nout + 2;
+        }
+        if (!ok) {
+            s_abort = 1;
+            atomicExch(&a.hdr->errword, (int)JAC_ETIMEOUT);
+        }
+    } else if (warp < R1) {
+        // ------------------------------------------------------- sweep-1 warps
+        const int w = warp;                         // row j0-1+w of every item
+        const float omega = (float)a.omega;
+        const uint64_t st_pol = l2_policy(a.l2_keep_state ? 1 : 0);
+        const int I = d.I, J = d.J, K = d.K, pitch = d.pitch;
+        const bool do2 = (w >= 1) && (w <= R1 - 2);  // this warp's row is an output row too
+        const uint32_t tm = s_tmem + ((uint32_t)(w & 3) << 21) + (uint32_t)(((w - 1) >> 2) * S::TM_SLOTS * S::TM_SLOT);
+        uint32_t pc = 0, cc = 0, qc = 0;
+        bool ok = true;
+        uint32_t entry;
+        while ((ok = next_item(entry)) && entry != S::END) {
+            const Item2 it = decode_item2(d, (int)(entry % nitems));
+            const int j = it.j0 - 1 + w;
+            const int ib = it.i0 + VI * lane;
+            const bool row1_in = (j >= 1) && (j <= J - 2);
+            bool in_i[VI], owned[VI];
+            bool all_owned = true;
+#pragma unroll
+            for (int e = 0; e < VI; ++e) {
+                in_i[e] = (ib + e >= 1) && (ib + e <= I - 2);
+                owned[e] = do2 && row1_in && in_i[e];
+                all_owned = all_owned && owned[e];
+            }
+            const int r0 = w * S::PW, r1 = (w + 1) * S::PW, r2 = (w + 2) * S::PW;   // rows j-1, j, j+1
+            const int cidx = w * TI + VI * lane;
+
+            for (int s = 0; s < it.nout + 2; ++s) {
+                const int m = it.kb - 1 + s;                 // sweep-1 plane
+                const uint32_t qs = qc + s;
+                if (s == 0) {
+                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
+                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
+                }
+                const uint32_t q2 = pc + s + 2;
+                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
+                ok = ok && mbar_wait_bounded(&c_full[(cc + s) % RC], ((cc + s) / RC) & 1);
+                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
+                ok = __all_sync(0xffffffffu, ok && !s_abort);
+                if (!ok) break;
+                const float *Pm = reinterpret_cast<const float *>(base + (size_t)((pc + s) % RP) * S::P_BYTES);
+                const float *Pk =
+                    reinterpret_cast<const float *>(base + (size_t)((pc + s + 1) % RP) * S::P_BYTES);
+                const float *Pp = reinterpret_cast<const float *>(base + (size_t)(q2 % RP) * S::P_BYTES);
+                const unsigned char *cs = ring_c + (size_t)((cc + s) % RC) * S::C_BYTES;
+                float ek0[VI + 2], ek1[VI + 2], ek2[VI + 2], em1[VI + 2], ep1[VI + 2];
+                float vm0[VI], vm2[VI], vp0[VI], vp2[VI];
+                load_ext<float, VI, H>(Pk + r0, lane, 32, ek0);
+                load_ext<float, VI, H>(Pk + r1, lane, 32, ek1);
+                load_ext<float, VI, H>(Pk + r2, lane, 32, ek2);
+                load_ext<float, VI, H>(Pm + r1, lane, 32, em1);
+                load_ext<float, VI, H>(Pp + r1, lane, 32, ep1);
+                lds_vec<float, VI>(Pm + r0 + H + VI * lane, vm0);
+                lds_vec<float, VI>(Pm + r2 + H + VI * lane, vm2);
+                lds_vec<float, VI>(Pp + r0 + H + VI * lane, vp0);
+                lds_vec<float, VI>(Pp + r2 + H + VI * lane, vp2);
+                const bool in1 = row1_in && (m >= 1) && (m <= K - 2);
+                const uint32_t at = tm + (qs % S::TM_SLOTS) * S::TM_SLOT;
+                auto coef = [&](int q, float (&v)[VI]) {
+                    lds_vec<float, VI>(reinterpret_cast<const float *>(cs + (q - 1) * S::TILE) + cidx, v);
+                };
+                // The coefficients in the two parts of the update, so that
+                // only one part's are held in registers at a time; an
+                // output row keeps them for sweep 2 at this plane.
+                float dd[VI], ec[VI];
+                {
+                    float wk[VI], a0[VI], a1[VI], a2[VI], c0[VI], c1[VI], c2[VI];
+                    coef(JAC_WRK1, wk); coef(JAC_A0, a0); coef(JAC_A1, a1); coef(JAC_A2, a2);
+                    coef(JAC_C0, c0); coef(JAC_C1, c1); coef(JAC_C2, c2);
+                    if (do2) {
+                        tmem_st16(at, wk, a0, a1, a2);
+                        tmem_st4(at + 16, c0);
+                        tmem_st4(at + 20, c1);
+                        tmem_st4(at + 24, c2);
+                    }
+                    float a3[VI];
+                    coef(JAC_A3, a3);
+#pragma unroll
+                    for (int e = 0; e < VI; ++e) {
+                        dd[e] = ss_axes(ek1[e + 1], ek1[e + 2], ek1[e], ek2[e + 1], ek0[e + 1], ep1[e + 1],
+                                        em1[e + 1], a0[e], a1[e], a2[e], c0[e], c1[e], c2[e], wk[e]);
+                        ec[e] = a3s_minus_one<false>(a3[e], a0[e], a1[e], a2[e], c0[e], c1[e], c2[e]);
+                    }
+                }
+                float out[VI];
+                {
+                    float b0[VI], b1[VI], b2[VI], a3[VI], bn[VI];
+                    coef(JAC_B0, b0); coef(JAC_B1, b1); coef(JAC_B2, b2); coef(JAC_A3, a3); coef(JAC_BND, bn);
+                    if (do2) {
+                        tmem_st4(at + 28, b0);
+                        tmem_st4(at + 32, b1);
+                        tmem_st16(at + 36, b2, a3, bn, ec);
+                    }
+#pragma unroll
+                    for (int e = 0; e < VI; ++e) {
+                        const float c = ek1[e + 1];
+                        const float bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
+                        const float bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
+                        const float bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
+                        const float ss = ss_rest(dd[e], c, bij, bjk, bik, a3[e], b0[e], b1[e], b2[e], bn[e], ec[e]);
+                        out[e] = (in1 && in_i[e]) ? fmaf(omega, ss, c) : c;
+                    }
+                }
+                float *qrow = reinterpret_cast<float *>(ring_q + (size_t)(qs % RQ) * S::Q_BYTES) + w * TI;
+                *reinterpret_cast<float4 *>(qrow + VI * lane) = make_float4(out[0], out[1], out[2], out[3]);
+                if (a.mid != nullptr && m >= it.kb && m < it.kb + it.nout) {
+                    // the intermediate state at this item's own points
+                    const size_t offm = ((size_t)m * J + (size_t)j) * (size_t)pitch + (size_t)ib;
+                    if (all_owned) {
+                        store_vec<float, VI>(a.mid + offm, out, st_pol);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < VI; ++e)
+                            if (owned[e]) a.mid[offm + e] = out[e];
+                    }
+                }
+                if (do2) {
+                    tmem_wait_st();
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&q_full[qs % RQ]);            // intermediate plane s: this row written
+                    mbar_arrive(&p_empty[(pc + s) % RP]);     // state plane m-1 is done
+                    mbar_arrive(&c_empty[(cc + s) % RC]);     // stage s is done
+                }
+            }
+            if (!ok) break;
+            __syncwarp();
+            if (lane == 0) {                      // the item's last state planes
+                mbar_arrive(&p_empty[(pc + it.nout + 2) % RP]);
+                mbar_arrive(&p_empty[(pc + it.nout + 3) % RP]);
+            }
+            pc += it.nout + 4;
+            cc += it.nout + 2;
+            qc += it.nout + 2;
         }
         if (!ok) {
             s_abort = 1;
             atomicExch(&a.hdr->errword, (int)JAC_ETIMEOUT);
         }
     } else {
-        // ------------------------------------------------------------ consumers
-        const int w = warp;                         // row j0-1+w of every item
+        // ------------------------------------------------------- sweep-2 warps
+        // A row's sweep-2 warp has the index of its sweep-1 warp modulo 4: the
+        // two share a quarter of the tensor memory.
+        const int w = (warp - S::WARP2) == 0 ? S::R2 : warp - S::WARP2;   // row j0-1+w of every item
         const float omega = (float)a.omega;
         const uint64_t st_pol = l2_policy(a.l2_keep_state ? 1 : 0);
-        const int I = d.I, J = d.J, K = d.K, pitch = d.pitch;
-        uint32_t pc = 0, cc = 0, qc = 0;
+        const int I = d.I, J = d.J, pitch = d.pitch;
+        const uint32_t tm = s_tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(((w - 1) >> 2) * S::TM_SLOTS * S::TM_SLOT);
+        uint32_t qc = 0;
         bool ok = true;
         double acc = 0.0;
         uint32_t sync_phase = 0;
@@ -336,265 +579,141 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             ++sync_phase;
             return __all_sync(0xffffffffu, r);
         };
-        const bool do2 = (w >= 1) && (w <= R1 - 2);  // this warp's row is an output row too
-
-        for (int t = 0; t < a.n_pass && ok; ++t) {
-            const bool res = (t == a.n_pass - 1) && (a.res != nullptr);
+        uint32_t entry;
+        while ((ok = next_item(entry)) && entry != S::END) {
+            const uint32_t t = entry / nitems;
+            const Item2 it = decode_item2(d, (int)(entry - t * nitems));
+            const bool res = (t == (uint32_t)a.n_pass - 1) && (a.res != nullptr);
             float *p_out = static_cast<float *>(((t + 1 + a.par) & 1) ? d.p_buf[1] : d.p_buf[0]);
-            for (int item = blockIdx.x; item < d.nitems && ok; item += G) {
-                const Item2 it = decode_item2(d, item);
-                const int j = it.j0 - 1 + w;
-                const int ib = it.i0 + VI * lane;
-                const bool row1_in = (j >= 1) && (j <= J - 2);
-                bool in_i[VI], owned[VI];
+            const int j = it.j0 - 1 + w;
+            const int ib = it.i0 + VI * lane;
+            const bool row_in = j <= J - 2;
+            bool owned[VI], all_owned = true;
 #pragma unroll
-                for (int e = 0; e < VI; ++e) {
-                    in_i[e] = (ib + e >= 1) && (ib + e <= I - 2);
-                    owned[e] = do2 && row1_in && in_i[e];
+            for (int e = 0; e < VI; ++e) {
+                owned[e] = row_in && (ib + e >= 1) && (ib + e <= I - 2);
+                all_owned = all_owned && owned[e];
+            }
+            const int q0 = (w - 1) * TI, q1 = w * TI, q2r = (w + 1) * TI;
+            for (int s = 3; s < it.nout + 3; ++s) {
+                // output plane kb-3+s from intermediate planes s-3 .. s-1
+                const uint32_t qs = qc + s;
+                const size_t off = ((size_t)(it.kb - 3 + s) * J + (size_t)j) * (size_t)pitch + (size_t)ib;
+                if (s == 3)
+                    ok = mbar_wait_bounded(&q_full[qc % RQ], (qc / RQ) & 1) &&
+                         mbar_wait_bounded(&q_full[(qc + 1) % RQ], ((qc + 1) / RQ) & 1);
+                ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1);
+                ok = __all_sync(0xffffffffu, ok && !s_abort);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const float *Qm =
+                    reinterpret_cast<const float *>(ring_q + (size_t)((qs - 3) % RQ) * S::Q_BYTES);
+                const float *Qk =
+                    reinterpret_cast<const float *>(ring_q + (size_t)((qs - 2) % RQ) * S::Q_BYTES);
+                const float *Qp =
+                    reinterpret_cast<const float *>(ring_q + (size_t)((qs - 1) % RQ) * S::Q_BYTES);
+                // columns i0-1 and i0+128 come from the edge warp
+                const float(*Em)[2] = q_edge[(qs - 3) % RQ];
+                const float(*Ek)[2] = q_edge[(qs - 2) % RQ];
+                const float(*Ep)[2] = q_edge[(qs - 1) % RQ];
+                float ek0[VI + 2], ek1[VI + 2], ek2[VI + 2], em1[VI + 2], ep1[VI + 2];
+                float vm0[VI], vm2[VI], vp0[VI], vp2[VI];
+                q_ext(Qk + q0, lane, Ek[w - 1][0], Ek[w - 1][1], ek0);
+                q_ext(Qk + q1, lane, Ek[w][0], Ek[w][1], ek1);
+                q_ext(Qk + q2r, lane, Ek[w + 1][0], Ek[w + 1][1], ek2);
+                q_ext(Qm + q1, lane, Em[w][0], Em[w][1], em1);
+                q_ext(Qp + q1, lane, Ep[w][0], Ep[w][1], ep1);
+                lds_vec<float, VI>(Qm + q0 + VI * lane, vm0);
+                lds_vec<float, VI>(Qm + q2r + VI * lane, vm2);
+                lds_vec<float, VI>(Qp + q0 + VI * lane, vp0);
+                lds_vec<float, VI>(Qp + q2r + VI * lane, vp2);
+                const uint32_t at = tm + ((qs - 2) % S::TM_SLOTS) * S::TM_SLOT;
+                float dd[VI], out[VI];
+                {
+                    float wk[VI], a0[VI], a1[VI], a2[VI], c0[VI], c1[VI], c2[VI];
+                    tmem_ld16(at, wk, a0, a1, a2);
+                    tmem_ld4(at + 16, c0);
+                    tmem_ld4(at + 20, c1);
+                    tmem_ld4(at + 24, c2);
+                    tmem_wait_ld();
+                    tmem_loaded(wk); tmem_loaded(a0); tmem_loaded(a1); tmem_loaded(a2);
+                    tmem_loaded(c0); tmem_loaded(c1); tmem_loaded(c2);
+#pragma unroll
+                    for (int e = 0; e < VI; ++e)
+                        dd[e] = ss_axes(ek1[e + 1], ek1[e + 2], ek1[e], ek2[e + 1], ek0[e + 1], ep1[e + 1],
+                                        em1[e + 1], a0[e], a1[e], a2[e], c0[e], c1[e], c2[e], wk[e]);
                 }
-                bool all_owned = true, any_owned = false;
-#pragma unroll
-                for (int e = 0; e < VI; ++e) {
-                    all_owned = all_owned && owned[e];
-                    any_owned = any_owned || owned[e];
-                }
-                const int r0 = w * S::PW, r1 = (w + 1) * S::PW, r2 = (w + 2) * S::PW;   // rows j-1, j, j+1
-                const int cidx = w * TI + VI * lane;
-                float *buf2 = reinterpret_cast<float *>(bufs2 + (size_t)(do2 ? w - 1 : 0) * S::B_BYTES);
-                // a3 S - 1 of this row's points at the sweep-1 planes of the
-                // last two steps, carried to sweep 2 at those planes
-                float ec1[VI], ec2[VI];
-#pragma unroll
-                for (int e = 0; e < VI; ++e) ec1[e] = ec2[e] = 0.0f;
-
-                for (int s = 0; s < it.nout + 3; ++s) {
-                    const int m = it.kb - 1 + s;                 // sweep-1 plane
-                    const uint32_t qs = qc + s;
-                    float ec0[VI];
-#pragma unroll
-                    for (int e = 0; e < VI; ++e) ec0[e] = 0.0f;
-                    if (s < it.nout + 2) {
-                        // ---- sweep 1 at plane m, row j, into intermediate plane s
-                        if (s == 0) {
-                            ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
-                                 mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
-                        }
-                        const uint32_t q2 = pc + s + 2;
-                        ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
-                        ok = ok && mbar_wait_bounded(&c_full[(cc + s) % RC], ((cc + s) / RC) & 1);
-                        if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
-                        ok = __all_sync(0xffffffffu, ok && !s_abort);
-                        if (!ok) break;
-                        const float *Pm = reinterpret_cast<const float *>(base + (size_t)((pc + s) % RP) * S::P_BYTES);
-                        const float *Pk =
-                            reinterpret_cast<const float *>(base + (size_t)((pc + s + 1) % RP) * S::P_BYTES);
-                        const float *Pp = reinterpret_cast<const float *>(base + (size_t)(q2 % RP) * S::P_BYTES);
-                        const unsigned char *cs = ring_c + (size_t)((cc + s) % RC) * S::C_BYTES;
-                        float ek0[VI + 2], ek1[VI + 2], ek2[VI + 2], em1[VI + 2], ep1[VI + 2];
-                        float vm0[VI], vm2[VI], vp0[VI], vp2[VI];
-                        load_ext<float, VI, H>(Pk + r0, lane, 32, ek0);
-                        load_ext<float, VI, H>(Pk + r1, lane, 32, ek1);
-                        load_ext<float, VI, H>(Pk + r2, lane, 32, ek2);
-                        load_ext<float, VI, H>(Pm + r1, lane, 32, em1);
-                        load_ext<float, VI, H>(Pp + r1, lane, 32, ep1);
-                        lds_vec<float, VI>(Pm + r0 + H + VI * lane, vm0);
-                        lds_vec<float, VI>(Pm + r2 + H + VI * lane, vm2);
-                        lds_vec<float, VI>(Pp + r0 + H + VI * lane, vp0);
-                        lds_vec<float, VI>(Pp + r2 + H + VI * lane, vp2);
-                        float ca0[VI], ca1[VI], ca2[VI], ca3[VI], cb0[VI], cb1[VI], cb2[VI], cc0[VI], cc1[VI],
-                            cc2[VI], cwk[VI], cbn[VI];
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 0 * S::TILE) + cidx, ca0);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 1 * S::TILE) + cidx, ca1);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 2 * S::TILE) + cidx, ca2);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 3 * S::TILE) + cidx, ca3);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 4 * S::TILE) + cidx, cb0);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 5 * S::TILE) + cidx, cb1);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 6 * S::TILE) + cidx, cb2);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 7 * S::TILE) + cidx, cc0);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 8 * S::TILE) + cidx, cc1);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 9 * S::TILE) + cidx, cc2);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 10 * S::TILE) + cidx, cwk);
-                        lds_vec<float, VI>(reinterpret_cast<const float *>(cs + 11 * S::TILE) + cidx, cbn);
-                        const bool in1 = row1_in && (m >= 1) && (m <= K - 2);
-                        float out[VI];
-#pragma unroll
-                        for (int e = 0; e < VI; ++e) {
-                            const float c = ek1[e + 1];
-                            const float bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
-                            const float bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
-                            const float bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
-                            ec0[e] = a3s_minus_one<false>(ca3[e], ca0[e], ca1[e], ca2[e], cc0[e], cc1[e], cc2[e]);
-                            const float ss = ss_f32_ec(c, ek1[e + 2], ek1[e], ek2[e + 1], ek0[e + 1], ep1[e + 1],
-                                                       em1[e + 1], bij, bjk, bik, ca0[e], ca1[e], ca2[e], ca3[e],
-                                                       cb0[e], cb1[e], cb2[e], cc0[e], cc1[e], cc2[e], cwk[e], cbn[e],
-                                                       ec0[e]);
-                            out[e] = (in1 && in_i[e]) ? fmaf(omega, ss, c) : c;
-                        }
-                        float *qrow = reinterpret_cast<float *>(ring_q + (size_t)(qs % RQ) * S::Q_BYTES) + w * TI;
-                        *reinterpret_cast<float4 *>(qrow + VI * lane) = make_float4(out[0], out[1], out[2], out[3]);
-                        if (a.mid != nullptr && m >= it.kb && m < it.kb + it.nout) {
-                            // the intermediate state at this item's own points
-                            const size_t offm = ((size_t)m * J + (size_t)j) * (size_t)pitch + (size_t)ib;
-                            if (all_owned) {
-                                store_vec<float, VI>(a.mid + offm, out, st_pol);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < VI; ++e)
-                                    if (owned[e]) a.mid[offm + e] = out[e];
-                            }
-                        }
-                        __syncwarp();
-                        if (lane == 0) {
-                            mbar_arrive(&q_full[qs % RQ]);            // intermediate plane s: this row written
-                            mbar_arrive(&p_empty[(pc + s) % RP]);     // state plane m-1 is done
-                            mbar_arrive(&c_empty[(cc + s) % RC]);     // stage s is done
-                        }
-                    }
-
-                    if (s >= 3) {
-                        // ---- sweep 2 at plane m-2 from intermediate planes s-3 .. s-1;
-                        // its coefficients come from global memory (the stage
-                        // that held them served sweep 1 two steps ago)
-                        const int m2 = m - 2;
-                        const size_t off = ((size_t)m2 * J + (size_t)j) * (size_t)pitch + (size_t)ib;
-                        for (int qq = 0; qq < 3 && ok; ++qq) {
-                            const uint32_t qw = qc + s - 3 + qq;
-                            ok = mbar_wait_bounded(&q_full[qw % RQ], (qw / RQ) & 1);
-                        }
-                        ok = __all_sync(0xffffffffu, ok && !s_abort);
-                        if (!ok) break;
-                        if (do2) {
-                            const float *Qm =
-                                reinterpret_cast<const float *>(ring_q + (size_t)((qs - 3) % RQ) * S::Q_BYTES);
-                            const float *Qk =
-                                reinterpret_cast<const float *>(ring_q + (size_t)((qs - 2) % RQ) * S::Q_BYTES);
-                            const float *Qp =
-                                reinterpret_cast<const float *>(ring_q + (size_t)((qs - 1) % RQ) * S::Q_BYTES);
-                            const int q0 = (w - 1) * TI, q1 = w * TI, q2r = (w + 1) * TI;
-                            // columns i0-1 and i0+128 come from the edge warp
-                            const float(*Em)[2] = q_edge[(qs - 3) % RQ];
-                            const float(*Ek)[2] = q_edge[(qs - 2) % RQ];
-                            const float(*Ep)[2] = q_edge[(qs - 1) % RQ];
-                            float ek0[VI + 2], ek1[VI + 2], ek2[VI + 2], em1[VI + 2], ep1[VI + 2];
-                            float vm0[VI], vm2[VI], vp0[VI], vp2[VI];
-                            q_ext(Qk + q0, lane, Ek[w - 1][0], Ek[w - 1][1], ek0);
-                            q_ext(Qk + q1, lane, Ek[w][0], Ek[w][1], ek1);
-                            q_ext(Qk + q2r, lane, Ek[w + 1][0], Ek[w + 1][1], ek2);
-                            q_ext(Qm + q1, lane, Em[w][0], Em[w][1], em1);
-                            q_ext(Qp + q1, lane, Ep[w][0], Ep[w][1], ep1);
-                            lds_vec<float, VI>(Qm + q0 + VI * lane, vm0);
-                            lds_vec<float, VI>(Qm + q2r + VI * lane, vm2);
-                            lds_vec<float, VI>(Qp + q0 + VI * lane, vp0);
-                            lds_vec<float, VI>(Qp + q2r + VI * lane, vp2);
-                            // this lane's own copies (issued a step ago) have landed
-                            cp_async_wait_all();
-                            float ca0[VI], ca1[VI], ca2[VI], ca3[VI], cb0[VI], cb1[VI], cb2[VI], cc0[VI], cc1[VI],
-                                cc2[VI], cwk[VI], cbn[VI];
-                            lds_vec<float, VI>(buf2 + 0 * TI + VI * lane, ca0);
-                            lds_vec<float, VI>(buf2 + 1 * TI + VI * lane, ca1);
-                            lds_vec<float, VI>(buf2 + 2 * TI + VI * lane, ca2);
-                            lds_vec<float, VI>(buf2 + 3 * TI + VI * lane, ca3);
-                            lds_vec<float, VI>(buf2 + 4 * TI + VI * lane, cb0);
-                            lds_vec<float, VI>(buf2 + 5 * TI + VI * lane, cb1);
-                            lds_vec<float, VI>(buf2 + 6 * TI + VI * lane, cb2);
-                            lds_vec<float, VI>(buf2 + 7 * TI + VI * lane, cc0);
-                            lds_vec<float, VI>(buf2 + 8 * TI + VI * lane, cc1);
-                            lds_vec<float, VI>(buf2 + 9 * TI + VI * lane, cc2);
-                            lds_vec<float, VI>(buf2 + 10 * TI + VI * lane, cwk);
-                            lds_vec<float, VI>(buf2 + 11 * TI + VI * lane, cbn);
-                            float out[VI];
-                            float ss2 = 0.0f;
-#pragma unroll
-                            for (int e = 0; e < VI; ++e) {
-                                const float c = ek1[e + 1];
-                                const float bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
-                                const float bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
-                                const float bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
-                                const float ss = ss_f32_ec(c, ek1[e + 2], ek1[e], ek2[e + 1], ek0[e + 1], ep1[e + 1],
-                                                           em1[e + 1], bij, bjk, bik, ca0[e], ca1[e], ca2[e], ca3[e],
-                                                           cb0[e], cb1[e], cb2[e], cc0[e], cc1[e], cc2[e], cwk[e],
-                                                           cbn[e], ec2[e]);
-                                out[e] = owned[e] ? fmaf(omega, ss, c) : c;
-                                if (res && owned[e]) ss2 = fmaf(ss, ss, ss2);
-                            }
-                            if (res) acc += (double)ss2;
-                            if (all_owned) {
-                                store_vec<float, VI>(p_out + off, out, st_pol);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < VI; ++e)
-                                    if (owned[e]) p_out[off + e] = out[e];
-                            }
-                        }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&q_empty[(qs - 3) % RQ]);   // intermediate plane s-3 done
-                    }
-                    // the coefficients of the next step's sweep 2 (plane m-1),
-                    // into this warp's buffer, which sweep 2 above has read
-                    if (do2 && s + 1 >= 3 && s + 1 <= it.nout + 2) {   // the same for every lane
-                        __syncwarp();
-                        if (any_owned) {
-                            const size_t offn = ((size_t)(m - 1) * J + (size_t)j) * (size_t)pitch + (size_t)ib;
-#pragma unroll
-                            for (int q = 0; q < 12; ++q)
-                                cp_async16(buf2 + q * TI + VI * lane, d.coef_ptr[q] + offn);
-                        }
-                        cp_async_commit();
-                    }
+                float ss2 = 0.0f;
+                {
+                    float b0[VI], b1[VI], b2[VI], a3[VI], bn[VI], ec[VI];
+                    tmem_ld4(at + 28, b0);
+                    tmem_ld4(at + 32, b1);
+                    tmem_ld16(at + 36, b2, a3, bn, ec);
+                    tmem_wait_ld();
+                    tmem_loaded(b0); tmem_loaded(b1); tmem_loaded(b2);
+                    tmem_loaded(a3); tmem_loaded(bn); tmem_loaded(ec);
 #pragma unroll
                     for (int e = 0; e < VI; ++e) {
-                        ec2[e] = ec1[e];
-                        ec1[e] = ec0[e];
+                        const float c = ek1[e + 1];
+                        const float bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
+                        const float bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
+                        const float bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
+                        const float ss = ss_rest(dd[e], c, bij, bjk, bik, a3[e], b0[e], b1[e], b2[e], bn[e], ec[e]);
+                        out[e] = owned[e] ? fmaf(omega, ss, c) : c;
+                        if (res && owned[e]) ss2 = fmaf(ss, ss, ss2);
                     }
                 }
-                if (!ok) break;
-                // the item's last state planes and intermediate planes
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&p_empty[(pc + it.nout + 2) % RP]);
-                    mbar_arrive(&p_empty[(pc + it.nout + 3) % RP]);
-                    mbar_arrive(&q_empty[(qc + it.nout) % RQ]);
-                    mbar_arrive(&q_empty[(qc + it.nout + 1) % RQ]);
+                if (res) acc += (double)ss2;
+                if (all_owned) {
+                    store_vec<float, VI>(p_out + off, out, st_pol);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < VI; ++e)
+                        if (owned[e]) p_out[off + e] = out[e];
                 }
-                pc += it.nout + 4;
-                cc += it.nout + 2;
-                qc += it.nout + 2;
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&q_empty[(qs - 3) % RQ]);   // intermediate plane s-3 done
             }
             if (!ok) break;
-            if (res) {
-                double v = acc;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-                if (lane == 0) s_part[w] = v;
-                if (!cons_sync()) { ok = false; break; }
-                if (w == 0) {
-                    const double sum = warp_sum(lane < R1 ? s_part[lane] : 0.0, 0.0);
-                    if (lane == 0) a.partials[blockIdx.x] = sum;
-                }
-                acc = 0.0;
-                if (!cons_sync()) { ok = false; break; }
+            __syncwarp();
+            if (lane == 0) {                      // the item's last intermediate planes
+                mbar_arrive(&q_empty[(qc + it.nout) % RQ]);
+                mbar_arrive(&q_empty[(qc + it.nout + 1) % RQ]);
             }
-            if (t + 1 < a.n_pass) {
-                // publish this CTA's part of the pass to every CTA's TMA reads
+            qc += it.nout + 2;
+            if (t + 1 < (uint32_t)a.n_pass) {
+                // publish this row's part of the item to every CTA's TMA reads
                 fence_proxy_async_global();
-                if (!cons_sync()) { ok = false; break; }
-                if (threadIdx.x == 0) {
+                __syncwarp();
+                if (lane == 0) {
                     __threadfence();
                     atomicAdd(&a.hdr->gbar, 1u);
                 }
+            }
+        }
+        if (ok && a.res != nullptr) {
+            double v = acc;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) s_part[w - 1] = v;
+            ok = cons_sync();
+            if (ok && warp == S::WARP2) {
+                const double sum = warp_sum(lane < S::R2 ? s_part[lane] : 0.0, 0.0);
+                if (lane == 0) a.partials[blockIdx.x] = sum;
             }
         }
         if (!ok) {
             s_abort = 1;
             atomicExch(&a.hdr->errword, (int)JAC_ETIMEOUT);
         }
-        cp_async_wait_all();   // no copy into this CTA's shared memory outlives it
     }
 
     // CTA epilogue: the last CTA to finish sums the partials in a fixed order
     // and resets the workspace counters for the next launch.
     // If any CTA gave up a wait, the residual is written as NaN.
     __syncthreads();
+    if (warp == S::EDGE_WARP) tmem_dealloc(s_tmem, S::TM_COLS);
     __shared__ int s_last;
     if (threadIdx.x == 0) {
         __threadfence();
@@ -613,6 +732,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             if (lane == 0) {
                 a.hdr->gbar = 0u;
                 a.hdr->counter = 0u;
+                a.hdr->ticket = 0u;
                 __threadfence();
             }
         }
@@ -637,12 +757,16 @@ int sweep2_tiles_i(int I)
     return (I - 2) / S::TI + 1;
 }
 
-// Output planes per item: the depth that minimises the rounds of items over
-// `ctas` CTAs times the steps of an item (its planes, the two extra planes
-// of sweep 1 and about two steps of start-up); ties go to the shallower.
-int sweep2_kdepth(long cols, int nk, int ctas)
+// Output planes per item: the depth that minimises the steps of a pass, the
+// rounds of items over `ctas` CTAs times the steps of an item (its planes, the
+// two extra planes of sweep 1 and about two steps of start-up); ties go to the
+// shallower.  steps: that minimum.
+int sweep2_kdepth(long cols, int nk, int ctas, long *steps = nullptr)
 {
-    if (nk <= 2) return std::max(nk, 1);
+    if (nk <= 2) {
+        if (steps) *steps = ((cols + ctas - 1) / ctas) * (nk + 4);
+        return std::max(nk, 1);
+    }
     long best_cost = -1;
     int best = 2;
     int prev = -1;
@@ -658,7 +782,19 @@ int sweep2_kdepth(long cols, int nk, int ctas)
             best = kd;
         }
     }
+    if (steps) *steps = best_cost;
     return best;
+}
+
+// Steps of a pass over the grid (one tile of 1024 points, both sweeps, each)
+// and tiles along i.
+long sweep2_steps(const jac_grid *g, int *tiles_i)
+{
+    const long nti = sweep2_tiles_i(g->I), ntj = (g->J - 2 + Sweep2Shape::R2 - 1) / Sweep2Shape::R2;
+    long steps = 0;
+    sweep2_kdepth(nti * ntj, g->K - 2, device_sm_count(), &steps);
+    *tiles_i = (int)nti;
+    return steps;
 }
 
 size_t sweep2_workspace_bytes(const jac_grid *g)
@@ -707,12 +843,26 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
     Sweep2Args a;
     std::memset(&a, 0, sizeof(a));
     a.n_pass = n_pass;
+    a.taken = (unsigned)(d_residual ? n_pass - 1 : n_pass) * (unsigned)d.nitems;
     a.par = 0;
     a.omega = g->omega;
     a.partials = reinterpret_cast<double *>(static_cast<char *>(workspace) + kWsHeaderBytes);
     a.res = d_residual;
     a.mid = static_cast<float *>(mid);
     a.hdr = hdr;
+    // Items of all passes and the arrivals of the pass barrier are counted in
+    // 32 bits: longer calls take several launches of an even number of passes.
+    const long long most = (0xffff0000ll / (items * S::R2)) & ~1ll;
+    if (n_pass > most) {
+        if (most < 2) return fail2(JAC_EINVAL, "grid too large for the two-sweep launch shape");
+        for (int left = n_pass; left > 0;) {
+            const int now = (int)std::min<long long>(left, most);
+            left -= now;
+            if ((s = sweep2_run(g, kdepth, now, left == 0 ? d_residual : nullptr, workspace, ws_bytes, st)) != JAC_OK)
+                return s;
+        }
+        return JAC_OK;
+    }
     SweepArgs la;
     std::memset(&la, 0, sizeof(la));
     set_l2_policy(la, g->prec, (size_t)d.pitch * g->J * g->K);

@@ -119,10 +119,10 @@ __device__ __forceinline__ float a3s_minus_one(float a3, float a0, float a1, flo
 // single-sweep and the two-sweep kernels, so that both round alike.
 // ss_f32_ec takes ec = a3 S - 1 already formed (it depends only on the
 // coefficients, so a kernel that updates the same point twice forms it once).
-__device__ __forceinline__ float ss_f32_ec(float c, float xp, float xm, float yp, float ym, float zp, float zm,
-                                           float bij, float bjk, float bik, float a0, float a1, float a2, float a3,
-                                           float b0, float b1, float b2, float c0, float c1, float c2, float wk,
-                                           float bnd, float ec)
+// It is the six axis terms (ss_axes) followed by the rest (ss_rest), for
+// kernels that hold the coefficients of one part at a time.
+__device__ __forceinline__ float ss_axes(float c, float xp, float xm, float yp, float ym, float zp, float zm, float a0,
+                                         float a1, float a2, float c0, float c1, float c2, float wk)
 {
     float d = wk;
     d = fmaf(a0, xp - c, d);
@@ -131,10 +131,25 @@ __device__ __forceinline__ float ss_f32_ec(float c, float xp, float xm, float yp
     d = fmaf(c0, xm - c, d);
     d = fmaf(c1, ym - c, d);
     d = fmaf(c2, zm - c, d);
+    return d;
+}
+
+__device__ __forceinline__ float ss_rest(float d, float c, float bij, float bjk, float bik, float a3, float b0, float b1,
+                                         float b2, float bnd, float ec)
+{
     d = fmaf(b0, bij, d);
     d = fmaf(b1, bjk, d);
     d = fmaf(b2, bik, d);
     return fmaf(a3, d, c * ec) * bnd;
+}
+
+__device__ __forceinline__ float ss_f32_ec(float c, float xp, float xm, float yp, float ym, float zp, float zm,
+                                           float bij, float bjk, float bik, float a0, float a1, float a2, float a3,
+                                           float b0, float b1, float b2, float c0, float c1, float c2, float wk,
+                                           float bnd, float ec)
+{
+    return ss_rest(ss_axes(c, xp, xm, yp, ym, zp, zm, a0, a1, a2, c0, c1, c2, wk), c, bij, bjk, bik, a3, b0, b1, b2,
+                   bnd, ec);
 }
 
 template <bool EXACT_SUM>
