@@ -34,8 +34,12 @@
 //   * consumer warp r owns row r of the tile, VI points per lane: it forms w
 //     on rows r-1, r, r+1, takes i-neighbours by lane shuffles and the
 //     tile's halo columns from the stage (lanes 0 and 31);
-//   * the FP64 gradient arrays are read-modify-written by the consumers,
-//     loaded one plane ahead;
+//   * the FP64 gradients are added in L2 (reductions without a result): an
+//     address gets one addition per launch, so the sum does not depend on
+//     their order, and no consumer waits for an old value or spends the SM's
+//     narrow FP64 pipe on the addition.  Against loads a plane ahead, an
+//     addition and a store: all gradients of 65x65x129 FP64 140 -> 90 us a
+//     sweep, dL/dwrk1 and dL/da3 of 257x257x513 FP32 617 -> 541 us;
 //   * column i = I-1 is a face that gathers only from column I-2.  When it
 //     lies just past the last tile (I-1 a multiple of TI), lane 31 of that
 //     tile emits it, so no tile is spent on a single column;
@@ -216,6 +220,11 @@ __device__ __forceinline__ void stg_vec(T *p, const T (&v)[VI])
     else *p = v[0];
 }
 
+// A gradient term as FP64: FP32 terms are widened in integer arithmetic, since
+// the conversion instruction shares the FP64 pipe with the additions.
+__device__ __forceinline__ double term(double x) { return x; }
+__device__ __forceinline__ double term(float x) { return widen(x); }
+
 template <typename T, typename C, int TJ, int VI_, bool CGRAD>
 __global__ void __launch_bounds__(AdjGeom<T, C, TJ, VI_>::THREADS, 1)
 k_adjoint(const __grid_constant__ AdjDesc d)
@@ -318,6 +327,9 @@ k_adjoint(const __grid_constant__ AdjDesc d)
         // others the right one (only lane 31 uses it)
         const int hcol = (lane == 0) ? -1 : TI;
         const bool hin = (lane == 0) ? inI_l : inI_r;
+        // FP64, which its pipe bounds: w is 0 at both halo columns of a tile as
+        // wide as the grid, and their products are left out
+        const bool halo = sizeof(T) == 4 || inI_l || inI_r;
         bool inJ[3];
 #pragma unroll
         for (int s = 0; s < 3; ++s) inJ[s] = (j - 1 + s >= 1) && (j - 1 + s <= J - 2);
@@ -326,19 +338,6 @@ k_adjoint(const __grid_constant__ AdjDesc d)
         T Xm = T(0), Xm1 = T(0);              // the same at column I-1 (extra)
 #pragma unroll
         for (int e = 0; e < VI; ++e) Qm[e] = Qm1[e] = T(0);
-        double gw[VI], ga[VI];                // gradients of the next plane, loaded one plane ahead
-#pragma unroll
-        for (int e = 0; e < VI; ++e) gw[e] = ga[e] = 0.0;
-        auto load_grads = [&](int m) {
-            if (!(m >= it.kb && m < it.ke && m >= 1 && m <= K - 2 && row_ok && inJ[1])) return;
-            const size_t dd = ((size_t)m * J + (size_t)j) * (size_t)I + (size_t)ib;
-#pragma unroll
-            for (int e = 0; e < VI; ++e)
-                if (inI[e]) {
-                    gw[e] = __ldcg(d.g_wrk1 + dd + e);
-                    ga[e] = __ldcg(d.g_a3 + dd + e);
-                }
-        };
         int pw = 0;                           // state planes of this item waited for
         const int np = it.m_hi - it.m_lo + 1;
 
@@ -346,10 +345,6 @@ k_adjoint(const __grid_constant__ AdjDesc d)
             const int kind = (m < it.kb) ? 1 : (m >= it.ke ? 2 : 0);
             const uint32_t cs = cc;
             const int need = min(m + 1, it.m_hi) - it.m_lo + 1;
-            double gwc[VI], gac[VI];          // this plane's gradients, loaded one plane ago
-#pragma unroll
-            for (int e = 0; e < VI; ++e) { gwc[e] = gw[e]; gac[e] = ga[e]; }
-            load_grads(m + 1);
             ok = mbar_wait_bounded(&c_full[cs % RC], (cs / RC) & 1);
             while (ok && pw < need) {
                 const uint32_t q = pc + (uint32_t)pw;
@@ -373,9 +368,19 @@ k_adjoint(const __grid_constant__ AdjDesc d)
                 st_vec<G, G::A3, T, VI>(st, row, VI * lane, av);
                 st_vec<G, G::BND, T, VI>(st, row, VI * lane, bv);
                 const bool rin = inK && inJ[s];
+                // where bnd is 1 the product omega bnd is omega (FP64 only,
+                // which its pipe bounds)
+                bool masked = true;
+                if constexpr (sizeof(T) == 8) {
+                    masked = false;
+#pragma unroll
+                    for (int e = 0; e < VI; ++e) masked = masked || (inI[e] && !is_one(bv[e]));
+                    masked = __any_sync(0xffffffffu, masked);
+                }
 #pragma unroll
                 for (int e = 0; e < VI; ++e) {
-                    const T mu = (rin && inI[e]) ? omega * bv[e] * lv[e] : T(0);
+                    const T ob = masked ? omega * bv[e] : omega;
+                    const T mu = (rin && inI[e]) ? ob * lv[e] : T(0);
                     w[s][e + 1] = av[e] * mu;
                     if (s == 1) { lam_c[e] = lv[e]; mu_c[e] = mu; }
                 }
@@ -386,8 +391,11 @@ k_adjoint(const __grid_constant__ AdjDesc d)
                     // the others: right), without a divergent branch; lanes 1..30
                     // discard it
                     const T lam_h = st_one<G, G::LAM, T>(st, row, hcol);
-                    const T mu = (rin && hin) ? omega * st_one<G, G::BND, T>(st, row, hcol) * lam_h : T(0);
-                    const T wh = st_one<G, G::A3, T>(st, row, hcol) * mu;
+                    T wh = T(0);
+                    if (halo) {
+                        const T mu = (rin && hin) ? omega * st_one<G, G::BND, T>(st, row, hcol) * lam_h : T(0);
+                        wh = st_one<G, G::A3, T>(st, row, hcol) * mu;
+                    }
                     wl = (lane == 0) ? wh : wl;
                     wr = (lane == 31) ? wh : wr;
                     if (s == 1) lam_x = lam_h;        // used by lane 31 only
@@ -408,7 +416,7 @@ k_adjoint(const __grid_constant__ AdjDesc d)
                 T l2 = __shfl_up_sync(0xffffffffu, P2[VI - 1], 1);
                 T r2 = __shfl_down_sync(0xffffffffu, P2[0], 1);
                 {
-                    const T p2h = st_one<G, G::B2, T>(st, r, hcol) * (lane == 0 ? w[1][0] : w[1][VI + 1]);
+                    const T p2h = halo ? st_one<G, G::B2, T>(st, r, hcol) * (lane == 0 ? w[1][0] : w[1][VI + 1]) : T(0);
                     l2 = (lane == 0) ? p2h : l2;
                     r2 = (lane == 31) ? p2h : r2;
                 }
@@ -469,15 +477,23 @@ k_adjoint(const __grid_constant__ AdjDesc d)
                 T lbp = __shfl_up_sync(0xffffffffu, Pbp[VI - 1], 1);
                 T rbp = __shfl_down_sync(0xffffffffu, Pbp[0], 1);
                 {
-                    const T bmh = st_one<G, G::B0, T>(st, r - 1, hcol) * (lane == 0 ? w[0][0] : w[0][VI + 1]);
-                    const T bph = st_one<G, G::B0, T>(st, r + 1, hcol) * (lane == 0 ? w[2][0] : w[2][VI + 1]);
+                    T bmh = T(0), bph = T(0);
+                    if (halo) {
+                        bmh = st_one<G, G::B0, T>(st, r - 1, hcol) * (lane == 0 ? w[0][0] : w[0][VI + 1]);
+                        bph = st_one<G, G::B0, T>(st, r + 1, hcol) * (lane == 0 ? w[2][0] : w[2][VI + 1]);
+                    }
                     lbm = (lane == 0) ? bmh : lbm;
                     rbm = (lane == 31) ? bmh : rbm;
                     lbp = (lane == 0) ? bph : lbp;
                     rbp = (lane == 31) ? bph : rbp;
                 }
-                if (lane == 0) la0 = st_one<G, G::A0, T>(st, r, -1) * w[1][0];
-                if (lane == 31) rc0 = st_one<G, G::C0, T>(st, r, TI) * w[1][VI + 1];
+                if (halo) {
+                    if (lane == 0) la0 = st_one<G, G::A0, T>(st, r, -1) * w[1][0];
+                    if (lane == 31) rc0 = st_one<G, G::C0, T>(st, r, TI) * w[1][VI + 1];
+                } else {
+                    if (lane == 0) la0 = T(0);
+                    if (lane == 31) rc0 = T(0);
+                }
 #pragma unroll
                 for (int e = 0; e < VI; ++e) {
                     const T a0w = (e == 0) ? la0 : Pa0[e - 1];
@@ -542,12 +558,12 @@ k_adjoint(const __grid_constant__ AdjDesc d)
                         s0 = fma(c2c[e], zm, s0);
                         const T we = w[1][e + 1];
                         // each sweep's term is formed in T and accumulated in FP64
-                        d.g_wrk1[dd + e] = gwc[e] + (double)we;
-                        d.g_a3[dd + e] = gac[e] + (double)(mu_c[e] * s0);
+                        atomicAdd(&d.g_wrk1[dd + e], term(we));
+                        atomicAdd(&d.g_a3[dd + e], term(mu_c[e] * s0));
                         if constexpr (CGRAD) {
                             const T tv[9] = {xp, yp, zp, bij, bjk, bik, xm, ym, zm};
 #pragma unroll
-                            for (int q = 0; q < 9; ++q) d.g_coef[q][dd + e] += (double)(we * tv[q]);
+                            for (int q = 0; q < 9; ++q) atomicAdd(&d.g_coef[q][dd + e], term(we * tv[q]));
                         }
                     }
                 }

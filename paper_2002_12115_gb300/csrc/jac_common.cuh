@@ -164,6 +164,42 @@ __device__ __forceinline__ void st_v2d_hint(double *p, double a, double b, uint6
                  : "memory");
 }
 
+// FP64 to FP32, round to nearest even.  In range of the normal FP32 numbers
+// the exponent is rebased, the significand cut to 23 bits and the 29 bits cut
+// off decide the rounding, whose carry may run into the exponent (up to
+// infinity); zero keeps its sign.  FP32 subnormals, overflow, infinity and
+// NaN take the conversion instruction (it runs on GB300's narrow FP64 pipe).
+__device__ __forceinline__ float narrow(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned mag = hi & 0x7fffffffu;
+    if (mag - (897u << 20) < (254u << 20)) {                  // 2^-126 <= |x| < 2^128
+        unsigned bits = __funnelshift_l(lo, mag - (896u << 20), 3);
+        const unsigned cut = lo << 3;                         // the 29 bits cut off, left-aligned
+        bits += (cut > 0x80000000u || (cut == 0x80000000u && (bits & 1u))) ? 1u : 0u;
+        return __uint_as_float(bits | (hi & 0x80000000u));
+    }
+    if ((mag | lo) == 0u) return __uint_as_float(hi);
+    return __double2float_rn(x);
+}
+
+// FP32 to FP64 (exact): normal numbers and zeros in integers.
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
+    if (mag - 0x00800000u < 0x7f000000u) {
+        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + (896u << 20))), (int)(u << 29));
+    }
+    if (mag == 0u) return __hiloint2double((int)u, 0);
+    return (double)x;
+}
+
+// Whether x is exactly 1 (an integer test: it costs no FP64 instruction).
+__device__ __forceinline__ bool is_one(double x)
+{
+    return __double2hiint(x) == 0x3ff00000 && __double2loint(x) == 0;
+}
+
 // Storage element type of array `which` under precision `prec` (host side).
 inline size_t elem_bytes(jac_prec prec, int which)
 {

@@ -31,36 +31,6 @@ namespace jac {
 
 namespace {
 
-// FP64 to FP32, round to nearest even.  In range of the normal FP32 numbers
-// the exponent is rebased, the significand cut to 23 bits and the 29 bits cut
-// off decide the rounding, whose carry may run into the exponent (up to
-// infinity); zero keeps its sign.  FP32 subnormals, overflow, infinity and
-// NaN take the conversion instruction.
-__device__ __forceinline__ float narrow(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const unsigned mag = hi & 0x7fffffffu;
-    if (mag - (897u << 20) < (254u << 20)) {                  // 2^-126 <= |x| < 2^128
-        unsigned bits = __funnelshift_l(lo, mag - (896u << 20), 3);
-        const unsigned cut = lo << 3;                         // the 29 bits cut off, left-aligned
-        bits += (cut > 0x80000000u || (cut == 0x80000000u && (bits & 1u))) ? 1u : 0u;
-        return __uint_as_float(bits | (hi & 0x80000000u));
-    }
-    if ((mag | lo) == 0u) return __uint_as_float(hi);
-    return __double2float_rn(x);
-}
-
-// FP32 to FP64 (exact): normal numbers and zeros in integers.
-__device__ __forceinline__ double widen(float x)
-{
-    const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
-    if (mag - 0x00800000u < 0x7f000000u) {
-        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + (896u << 20))), (int)(u << 29));
-    }
-    if (mag == 0u) return __hiloint2double((int)u, 0);
-    return (double)x;
-}
-
 // FP64 -> FP32 -> BF16, each RNE; FP32 numbers keep their value in FP32 and
 // FP64 storage, so both sources give the same storage values.
 template <typename C, typename S>
