@@ -31,8 +31,8 @@
 // L2, the flag follows, is seen, and the rows come back) plus the arithmetic
 // (FP64) or the shared-memory reads of 19 state values and the coefficients
 // per point (FP32).  Measured, us a sweep, streaming -> resident:
-//   17x17x17 FP64 6.3 -> 3.4      33x33x65 FP64 6.4 -> 5.2   49x49x97 FP64 15.9 -> 10.9
-//   33x33x65 FP32 4.5 -> 3.5      77x53x101 FP32 7.0 -> 5.7  65x65x129 FP32 6.5 -> 4.7
+//   17x17x17 FP64 6.3 -> 3.7      33x33x65 FP64 6.4 -> 5.1   49x49x97 FP64 15.9 -> 10.9
+//   33x33x65 FP32 4.5 -> 3.5      77x53x101 FP32 7.0 -> 4.8  65x65x129 FP32 6.5 -> 4.7
 //   65x65x129 BF16 6.1 -> 4.2
 #include <algorithm>
 #include <cstring>
@@ -161,9 +161,10 @@ struct PointCoef<float, __nv_bfloat16> {
 };
 
 // ss of the point at P in a state with row stride W and plane stride Z; the
-// operations of the streaming kernels, in their order.
+// operations of the streaming kernels, in their order.  FP64 leaves out the
+// multiply by bnd where the whole box has bnd = 1 (not masked).
 template <typename T, typename C>
-__device__ __forceinline__ T res_ss(const T *P, int W, int Z, const PointCoef<T, C> &k)
+__device__ __forceinline__ T res_ss(const T *P, int W, int Z, const PointCoef<T, C> &k, bool masked)
 {
     const T c = P[0], xp = P[1], xm = P[-1], yp = P[W], ym = P[-W], zp = P[Z], zm = P[-Z];
     const T bij = ((P[W + 1] - P[-W + 1]) - P[W - 1]) + P[-W - 1];
@@ -183,7 +184,9 @@ __device__ __forceinline__ T res_ss(const T *P, int W, int Z, const PointCoef<T,
         s0 = fma(k.c0, xm, s0);
         s0 = fma(k.c1, ym, s0);
         s0 = fma(k.c2, zm, s0);
-        return fma(s0, k.a3, -c) * k.bn;
+        T ss = fma(s0, k.a3, -c);
+        if (masked) ss *= k.bn;
+        return ss;
     }
 }
 
@@ -194,6 +197,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
     constexpr int TV = 16 / (int)sizeof(T);            // elements of a 16-byte vector
     extern __shared__ __align__(16) unsigned char res_smem[];
     __shared__ volatile int s_abort;
+    __shared__ int s_masked;
     __shared__ double s_part[kWarps];
     __shared__ int s_last;
 
@@ -214,6 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
 
     if (tid == 0) {
         s_abort = 0;
+        s_masked = 0;
         __stcg(a.flags + (size_t)b * kFlagStride, 0u);
         __threadfence();
         atomicAdd(&a.hdr->gbar, 1u);                   // every flag is zero once all G arrived
@@ -245,9 +250,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
     __syncthreads();
     for (int u = tid; u < units; u += kThreads) {
         const int r = u / bi;
-        PC::put(coefs + u, a.ucap, a.coef, (size_t)rowtab[r].y + 1 + (u - r * bi));
+        const size_t off = (size_t)rowtab[r].y + 1 + (u - r * bi);
+        PC::put(coefs + u, a.ucap, a.coef, off);
+        if constexpr (sizeof(T) == 8)
+            if (__ldg(static_cast<const double *>(a.coef[JAC_BND - 1]) + off) != 1.0) s_masked = 1;
     }
     __syncthreads();
+    const bool masked = s_masked != 0;
 
     const T omega = (T)a.omega;
     const bool compute = warp < kComputeWarps;
@@ -263,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
             PC k;
             k.get(coefs + u, a.ucap);
             const T *P = old + row.x + 1 + i;
-            const T ss = res_ss<T, C>(P, W, Z, k);
+            const T ss = res_ss<T, C>(P, W, Z, k, masked);
             const T v = fma(omega, ss, P[0]);
             nxt[row.x + 1 + i] = res ? ss : v;
             if (out) out[(size_t)row.y + 1 + i] = v;
@@ -438,30 +447,39 @@ jac_status launch_resident(const ResArgs &a, unsigned nblocks, size_t smem, cuda
 }  // namespace
 
 // The boxes of a grid over at most `sms` CTAs, and whether they fit in shared
-// memory.  Among the splits of the J-2 x K-2 rows into nj x nk boxes the one
-// with the fewest points in its largest box wins (in turns of the compute
-// warps for FP64, whose narrow pipe works in whole warps), then the one with
-// the fewest halo rows to collect.
+// memory: of the splits of the J-2 x K-2 rows into nj x nk boxes the one whose
+// largest box takes the least time by this model of a sweep, in ns: the rows
+// next to other boxes at tu per point (128 points at a time: one per lane of
+// a warp on each of the SM's four FP64 pipes), then the exchange, which the
+// inner rows overlap, and the halo rows it collects.  tu and the exchange are
+// measured (33x33x65 FP64, 77x53x101 FP32).  Against the split with the fewest
+// points in its largest box, which left 77x53x101 FP32 no inner rows (17 x 2
+// instead of 9 x 4): 5.7 -> 4.8 us a sweep.
 bool resident_shape(int I, int J, int K, jac_prec prec, int sms, ResidentShape *out)
 {
     const int nji = J - 2, nki = K - 2, bi = I - 2;
     const int ws = (int)round_up((size_t)I, prec == JAC_F64 ? 2 : 4);
+    const long long pts = (long long)nji * nki * bi;
+    // more points than all shared memory holds, or more than 32-bit offsets
+    if (pts * vectors_per_point(prec) * 16 > (long long)sms * (long long)kSmemBudget) return false;
     if ((long long)jac_pitch(I) * J * K > 0x7fffffffLL) return false;
-    long long best = -1;
+    const double tu = prec == JAC_F64 ? 5.7 : 0.47, exchange = 3000.0;
+    auto time_of = [&](long long rows) { return tu * (double)((rows * bi + 127) / 128 * 128); };
+    double best = -1.0;
     for (int nj = 1; nj <= std::min(nji, sms); ++nj) {
         const int nk = std::min(nki, sms / nj);
         const int bj = (nji + nj - 1) / nj, bk = (nki + nk - 1) / nk;
-        const long long units = (long long)bj * bk * bi;
-        if (units > 65536) continue;                   // far past any shared memory
-        const size_t smem = resident_smem(prec, (int)units, bj * bk, ws, bj, bk);
+        const long long rows = (long long)bj * bk;
+        if (rows * bi > 65536) continue;               // far past any shared memory
+        const long long edge = (bj <= 2 || bk <= 2) ? rows : 2LL * (bj + bk) - 4;
+        const double cost = time_of(edge) + std::max(exchange, time_of(rows - edge)) + 2.0 * (2 * (bj + bk) + 4);
+        if (best >= 0.0 && cost >= best) continue;
+        const size_t smem = resident_smem(prec, (int)(rows * bi), (int)rows, ws, bj, bk);
         if (smem > kSmemBudget) continue;
-        const long long turns = (units + 127) / 128 * 128;
-        const long long cost = turns * 4096 + std::min(2 * (bj + bk), 4095);
-        if (best >= 0 && cost >= best) continue;
         best = cost;
         *out = ResidentShape{nj, nk, bj, bk, ws, smem};
     }
-    return best >= 0;
+    return best >= 0.0;
 }
 
 size_t resident_workspace_bytes(const ResidentShape &s)
