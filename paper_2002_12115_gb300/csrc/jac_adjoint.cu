@@ -248,7 +248,9 @@ k_adjoint(const __grid_constant__ AdjDesc d)
         s_abort = 0;
         fence_mbar_init();
     }
+    launch_dependents();       // the next adjoint sweep's CTAs start as this one's end
     __syncthreads();
+    wait_prior_grids();        // lambda, the gradients and the states of earlier launches
 
     if (warp == TJ) {
         // ---------------------------------------------------------- producer
@@ -618,8 +620,18 @@ jac_status launch_adj(const AdjDesc &d, unsigned nblocks, cudaStream_t st)
                                    (int)G::SMEM);
     });
     if (err != cudaSuccess) return adj_fail(JAC_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(err));
-    k_adjoint<T, C, TJ, VI, CGRAD><<<nblocks, G::THREADS, G::SMEM, st>>>(d);
-    cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(nblocks);
+    cfg.blockDim = dim3(G::THREADS);
+    cfg.dynamicSmemBytes = G::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_adjoint<T, C, TJ, VI, CGRAD>, d);
     if (e != cudaSuccess) return adj_fail(JAC_ECUDA, std::string("adjoint launch: ") + cudaGetErrorString(e));
     return JAC_OK;
 }

@@ -684,7 +684,18 @@ jac_status jac_sweep_adjoint(jac_ctx *c, const double *lam_T, double *g_wrk1, do
         // recompute the segment's states: where the plan takes two-sweep
         // passes, one pass gives two states (the intermediate one stored on
         // the way), bitwise those of single sweeps
-        for (int m = 1; m < len;) {
+        jac::ResidentShape shape;
+        int m1 = 1;
+        if (jac::use_resident(&g, &c->plan, len - 1, c->ws_bytes, &shape)) {
+            // one launch, every state to its slot (a segment of 8 on 65x60x97
+            // FP32: 7 launches of 18 us -> one of 40 us)
+            g.p[0] = state(0);
+            g.p[1] = tp.seg(1);
+            s = jac::resident_run(&g, shape, len - 1, nullptr, c->ws, c->stream, tp.seg(1), tp.state_bytes);
+            if (s != JAC_OK) return ctx_from_thread(c, s);
+            m1 = len;
+        }
+        for (int m = m1; m < len;) {
             g.p[0] = state(m - 1);
             if (pairs && m + 1 < len) {
                 g.p[1] = tp.seg(m + 1);

@@ -85,9 +85,13 @@ struct ResidentShape {
 // False where the grid does not fit in the shared memory of `sms` SMs.
 bool resident_shape(int I, int J, int K, jac_prec prec, int sms, ResidentShape *out);
 size_t resident_workspace_bytes(const ResidentShape &s);
-// d_residual NULL: no residual is summed.
+// d_residual NULL: no residual is summed.  hist not NULL: state t + 1 goes
+// whole to hist + t * hist_stride (bytes; faces and padding already there)
+// and p[1] is not used.
 jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, double *d_residual, void *workspace,
-                        cudaStream_t st);
+                        cudaStream_t st, void *hist = nullptr, size_t hist_stride = 0);
+// Whether a call of n_iter sweeps with this plan and workspace runs resident.
+bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r);
 jac_status adjoint_step_dev(const jac_grid *g, const void *p_t, const void *lam_in, void *lam_out, double *g_wrk1,
                             double *g_a3, double *const *g_coef, int kdepth, void *workspace, size_t ws_bytes,
                             cudaStream_t st);

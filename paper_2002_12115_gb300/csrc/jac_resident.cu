@@ -22,6 +22,9 @@
 //   * Safety of the two state buffers: a box stores sweep t+2's rows over
 //     sweep t's only after every neighbour released sweep t+1's flag, which
 //     it does after it copied sweep t's halo.
+//   * With a history every state of the call is stored whole, each to its own
+//     array (the reverse pass recomputes a checkpoint segment that way, in one
+//     launch instead of one per sweep).
 //   * The update is the streaming kernels' arithmetic in the same order, so
 //     the state is bitwise theirs.  The last sweep stores the whole box; its ss
 //     values, left in shared memory, give the residual (one partial per CTA).
@@ -65,6 +68,8 @@ struct ResArgs {
     double *partials;          // one per CTA
     double *res;
     unsigned *flags;           // one per CTA, kFlagStride words apart
+    char *hist;                // not NULL: state t + 1 whole at hist + t * hist_stride
+    size_t hist_stride;        // instead of in p_buf[(t + 1) & 1]
     WsHeader *hdr;
 };
 
@@ -296,7 +301,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
     for (int t = 0; t < a.n_iter; ++t) {
         const T *old = (t & 1) ? st1 : st0;
         T *nxt = (t & 1) ? st0 : st1;
-        T *out = static_cast<T *>(a.p_buf[(t + 1) & 1]);
+        T *out = a.hist ? reinterpret_cast<T *>(a.hist + (size_t)t * a.hist_stride)
+                        : static_cast<T *>(a.p_buf[(t + 1) & 1]);
         const bool last = t == a.n_iter - 1;
         if (last) {
             if (compute) update(0, units, old, nxt, out, a.res != nullptr);
@@ -305,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
         if (compute) update(0, edge_rows * bi, old, nxt, out, false);
         __syncthreads();                               // the box's outer rows are stored
         if (compute) {
-            update(edge_rows * bi, units, old, nxt, nullptr, false);
+            update(edge_rows * bi, units, old, nxt, a.hist ? out : nullptr, false);
         } else {
             if (publisher && lane == 0) {
                 // orders the box's stores (before the barrier) ahead of the flag
@@ -489,7 +495,7 @@ size_t resident_workspace_bytes(const ResidentShape &s)
 }
 
 jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, double *d_residual, void *workspace,
-                        cudaStream_t st)
+                        cudaStream_t st, void *hist, size_t hist_stride)
 {
     const unsigned ctas = (unsigned)(s.nj * s.nk);
     ResArgs a;
@@ -511,6 +517,8 @@ jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, d
     a.partials = reinterpret_cast<double *>(w + kWsHeaderBytes);
     a.flags = reinterpret_cast<unsigned *>(w + kWsHeaderBytes + round_up(ctas * sizeof(double), 256));
     a.res = d_residual;
+    a.hist = static_cast<char *>(hist);
+    a.hist_stride = hist_stride;
     switch (g->prec) {
     case JAC_F64: return launch_resident<double, double>(a, ctas, s.smem, st);
     case JAC_F32: return launch_resident<float, float>(a, ctas, s.smem, st);

@@ -450,7 +450,7 @@ size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
 // precisions) a resident sweep takes 0.54-0.82 of a streaming one and the
 // launch up to 6 us more (the copy of the coefficients), so it pays from the
 // third sweep on; one or two sweeps stay with the streaming kernel.
-static bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r)
+bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r)
 {
     if (n_iter < 3) return false;
     if (!all_zero(plan)) return false;

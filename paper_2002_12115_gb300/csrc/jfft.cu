@@ -41,6 +41,7 @@
 #include <vector>
 
 #include "../../include/jfft.h"
+#include "jac_common.cuh"
 #include "jac_internal.h"
 
 namespace jfft {
@@ -221,8 +222,8 @@ __device__ __forceinline__ double kbar2(int k, int n)
 // Programmatic dependent launch: a pass lets the next launch of the stream
 // start its prologue as soon as every CTA of this one runs, and waits for
 // everything before it in the stream ahead of its own first data access.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_prior_grids() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+using jac::launch_dependents;
+using jac::wait_prior_grids;
 
 // The spectral factor along each axis, exp(c kbar^2) for every index of
 // n1, then n2, then n3 (FP64 exp, stored as T): one small launch per step,
