@@ -525,12 +525,11 @@ jac_status jac_residual(jac_ctx *c, double *out)
 {
     if (!c || !out) return ctx_fail(c, JAC_EINVAL, "NULL argument");
     if (!c->has_res) return ctx_fail(c, JAC_ESTATE, "no sweep since the last upload");
-    jac_status s = jac::workspace_check(c->ws, c->stream);
+    // the error word and the residual are in the same header: one copy
+    jac::WsHeader h;
+    jac_status s = jac::workspace_read(c->ws, c->stream, &h);
     if (s != JAC_OK) return ctx_from_thread(c, s);
-    jac::WsHeader *hdr = static_cast<jac::WsHeader *>(c->ws);
-    cudaError_t e = cudaMemcpyAsync(out, &hdr->residual, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return ctx_cuda(c, e, "residual copy");
+    *out = h.residual;
     return JAC_OK;
 }
 

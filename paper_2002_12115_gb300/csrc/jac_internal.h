@@ -12,6 +12,7 @@ namespace jac {
 
 struct GridDesc;
 struct SweepArgs;
+struct WsHeader;
 
 const char *thread_last_error();
 void set_thread_error(const std::string &m);
@@ -49,6 +50,7 @@ jac_status unpack_dev(int I, int J, int K, jac_prec prec, int which, const void 
 jac_status unpack_dev_f32(int I, int J, int K, jac_prec prec, int which, const void *src, float *dst,
                           cudaStream_t st);
 jac_status workspace_check(void *workspace, cudaStream_t st);
+jac_status workspace_read(void *workspace, cudaStream_t st, WsHeader *out);
 int device_sm_count();
 size_t device_l2_bytes();
 void set_l2_policy(SweepArgs &a, jac_prec prec, size_t points);

@@ -557,7 +557,9 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     return launch_sweep<false>(g->prec, tj, d0, a, nblocks, static_cast<cudaStream_t>(stream));
 }
 
-jac_status workspace_check(void *workspace, cudaStream_t st)
+// The workspace header, once the stream has passed; an error word set by a
+// kernel is reported and cleared.
+jac_status workspace_read(void *workspace, cudaStream_t st, WsHeader *out)
 {
     if (!workspace) return fail(JAC_EINVAL, "workspace is NULL");
     WsHeader h;
@@ -570,8 +572,11 @@ jac_status workspace_check(void *workspace, cudaStream_t st)
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         return fail((jac_status)h.errword, "a bounded device wait gave up");
     }
+    if (out) *out = h;
     return JAC_OK;
 }
+
+jac_status workspace_check(void *workspace, cudaStream_t st) { return workspace_read(workspace, st, nullptr); }
 
 }  // namespace jac
 
