@@ -521,7 +521,10 @@ jac_status jac_batch_grid_plan(const jac_batch *b, int g, jac_plan *out);
 
 /* Paper: the Himeno loop (Section 5.1.1) for many grids at once.
  * n_iter sweeps of every grid in one persistent launch (captured in a CUDA
- * graph on first use for this n_iter and buffer parity, then replayed).
+ * graph on first use for this n_iter and buffer parity, then replayed).  A
+ * FP32 batch without a plan whose state leaves L2 runs all but the last one to
+ * four sweeps in two launches instead: its wide grids in two-sweep passes, the
+ * others singly; the state is bitwise the same.
  * If res_host is not NULL it receives the n residuals of the last sweep.
  * Synchronises.  JAC_ETIMEOUT if a bounded device wait gave up. */
 jac_status jac_batch_sweep(jac_batch *b, int n_iter, double *res_host);

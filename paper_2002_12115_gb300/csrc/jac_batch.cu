@@ -6,7 +6,9 @@
 // depth) and first work item -- in a device table.  The forward kernel of
 // jac_sweep_kernel.cuh walks the concatenated work items of all grids; a
 // bounded grid barrier separates sweeps across the whole batch and the
-// residual of each grid is reduced deterministically.  Tile widths and
+// residual of each grid is reduced deterministically.  Without a plan, wide
+// grids of a FP32 batch that leaves L2 take two-sweep passes (jac_sweep2.cu)
+// for all but a call's last sweeps.  Tile widths and
 // k-block depths come per grid from a plan (an autotuner chooses them per
 // size class by measurement).
 #include <cuda_runtime.h>
@@ -40,6 +42,14 @@ struct jac_batch {
     size_t ws_bytes = 0;
     int warps = 8;
     std::vector<int> tile_i, kdepth;       // per grid, 0 = default
+    bool own_plan = true;                  // no plan set: the library's own choice per grid
+    // Grids whose sweeps (all but the last few of a call) run as two-sweep
+    // passes, and the others, each with its own tables; empty unless own_plan.
+    struct Part {
+        void *descs = nullptr;
+        int *item_base = nullptr;
+        int ngrids = 0, nitems = 0;
+    } passes, singles;
     bool tables_ok = false;
     int nitems = 0;
     unsigned nblocks = 0;
@@ -86,6 +96,11 @@ void drop_tables(jac_batch *b)
     if (b->d_descs) cudaFree(b->d_descs);
     if (b->d_item_base) cudaFree(b->d_item_base);
     if (b->ws) cudaFree(b->ws);
+    for (jac_batch::Part *p : {&b->passes, &b->singles}) {
+        if (p->descs) cudaFree(p->descs);
+        if (p->item_base) cudaFree(p->item_base);
+        *p = jac_batch::Part();
+    }
     b->d_descs = nullptr;
     b->d_item_base = nullptr;
     b->ws = nullptr;
@@ -106,6 +121,77 @@ jac_plan grid_plan(const jac_batch *b, int g)
         p.kdepth = std::max(2, std::min(b->K[g] - 2, 16));
     }
     return p;
+}
+
+// Device copies of a part's descriptors and first items.
+jac_status upload_part(jac_batch::Part *p, const void *descs, size_t desc_bytes, const std::vector<int> &base, int items)
+{
+    p->ngrids = (int)base.size();
+    p->nitems = items;
+    cudaError_t e = cudaMalloc(&p->descs, desc_bytes * base.size());
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&p->item_base), sizeof(int) * base.size());
+    if (e == cudaSuccess) e = cudaMemcpy(p->descs, descs, desc_bytes * base.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(p->item_base, base.data(), sizeof(int) * base.size(), cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? JAC_OK : JAC_ENOMEM;
+}
+
+// Which grids take two-sweep passes, and both parts' tables.  A batch whose
+// state stays in L2 keeps single sweeps; elsewhere those are bound by DRAM
+// (8.55 ns per 1000 stored points, measured on the 512-grid batch), and a pass
+// takes 1.67 us per step on one of the SMs, so a grid's width decides: 129
+// columns fill the passes' 128-column tiles, 97 three quarters of them, and
+// narrower grids are faster in single sweeps with folded rows.  Items of up to
+// 32 planes (16, 24, 48, 64, 128 planes: 1.4, 0.5, 1.1, 1.3, 5% slower).  The
+// 512 grids, 40 sweeps: 51.3 -> 47.0 ms.
+jac_status build_parts(jac_batch *b)
+{
+    if (!b->own_plan || b->prec != JAC_F32 || b->warps != 8) return JAC_OK;
+    size_t points = 0;
+    for (int g = 0; g < b->n; ++g) points += (size_t)jac_pitch(b->I[g]) * b->J[g] * b->K[g];
+    if (2 * points * sizeof(float) <= jac::device_l2_bytes() / 2) return JAC_OK;
+    const int sms = jac::device_sm_count();
+    std::vector<int> wide, narrow, depth;
+    double saved = 0.0, steps_all = 0.0;      // us a sweep; steps of a pass
+    for (int g = 0; g < b->n; ++g) {
+        const int nk = b->K[g] - 2, blocks = (nk + 31) / 32, kd = (nk + blocks - 1) / blocks;
+        const double steps = (double)((b->I[g] - 2) / 128 + 1) * ((b->J[g] - 2 + 7) / 8) * (nk + 3.0 * blocks);
+        const double one = 8.55e-6 * (double)jac_pitch(b->I[g]) * b->J[g] * b->K[g];
+        const double two = 0.5 * 1.67 * steps / sms;
+        if (two < 0.95 * one) {
+            wide.push_back(g);
+            depth.push_back(std::max(kd, 1));
+            saved += one - two;
+            steps_all += steps;
+        } else {
+            narrow.push_back(g);
+        }
+    }
+    // a pass ends with part of an item's time on most SMs idle (up to 35 steps)
+    if (wide.empty() || saved < 0.5 * 1.67 * 35.0 || steps_all < 4.0 * 35.0 * sms) return JAC_OK;
+    std::vector<char> d2(jac::sweep2_desc_bytes() * wide.size());
+    std::vector<int> base2, base1;
+    long long items2 = 0, items1 = 0;
+    for (size_t q = 0; q < wide.size(); ++q) {
+        int items = 0;
+        base2.push_back((int)items2);
+        const jac_status s = jac::sweep2_batch_desc(d2.data() + q * jac::sweep2_desc_bytes(), &b->grids[wide[q]],
+                                                    depth[q], &items);
+        if (s != JAC_OK) return bthread(b, s);
+        items2 += items;
+    }
+    std::vector<jac::GridDesc> d1;
+    for (int g : narrow) {
+        base1.push_back((int)items1);
+        d1.push_back(b->host_descs[g]);
+        d1.back().item_base = (int)items1;
+        items1 += b->host_descs[g].nitems;
+    }
+    if (items2 > 0x3fffffffLL) return JAC_OK;
+    jac_status s = upload_part(&b->passes, d2.data(), jac::sweep2_desc_bytes(), base2, (int)items2);
+    if (s == JAC_OK && !narrow.empty())
+        s = upload_part(&b->singles, d1.data(), sizeof(jac::GridDesc), base1, (int)items1);
+    return s == JAC_OK ? JAC_OK : bfail(b, JAC_ENOMEM, "batch table allocation failed");
 }
 
 // Descriptors, item bases and workspace for the current plan.
@@ -144,6 +230,11 @@ jac_status build_tables(jac_batch *b)
         drop_tables(b);
         return bcuda(b, e, "batch table upload");
     }
+    const jac_status s = build_parts(b);
+    if (s != JAC_OK) {
+        drop_tables(b);
+        return s;
+    }
     b->tables_ok = true;
     return JAC_OK;
 }
@@ -166,6 +257,34 @@ jac::SweepArgs batch_args(const jac_batch *b, int n_iter)
     for (int g = 0; g < b->n; ++g) points += (size_t)jac_pitch(b->I[g]) * b->J[g] * b->K[g];
     jac::set_l2_policy(a, b->prec, points);
     return a;
+}
+
+// The n_iter sweeps of every grid, on stream st.  With parts, all but the last
+// one to four sweeps run part by part (passes come in even numbers, so every
+// grid's state stays in the same buffer); the last ones, with the residuals,
+// over the whole batch.
+jac_status enqueue_sweeps(jac_batch *b, int n_iter, cudaStream_t st)
+{
+    jac::SweepArgs a = batch_args(b, n_iter);
+    const int n_pass = b->passes.ngrids ? ((n_iter - 1) / 2) & ~1 : 0;
+    if (n_pass > 0) {
+        jac_status s = jac::sweep2_batch_run(b->passes.descs, b->passes.item_base, b->passes.ngrids, b->passes.nitems,
+                                             n_pass, b->par, b->omega, b->ws, st);
+        if (s != JAC_OK) return s;
+        if (b->singles.ngrids) {
+            jac::SweepArgs p = a;
+            p.descs = static_cast<const jac::GridDesc *>(b->singles.descs);
+            p.item_base = b->singles.item_base;
+            p.ngrids = b->singles.ngrids;
+            p.nitems = b->singles.nitems;
+            p.n_iter = 2 * n_pass;
+            p.res = nullptr;
+            const unsigned nblocks = (unsigned)std::min<long long>(p.nitems, jac::device_sm_count());
+            if ((s = jac::launch_sweep<true>(b->prec, b->warps, b->host_descs[0], p, nblocks, st)) != JAC_OK) return s;
+        }
+        a.n_iter = n_iter - 2 * n_pass;
+    }
+    return jac::launch_sweep<true>(b->prec, b->warps, b->host_descs[0], a, b->nblocks, st);
 }
 
 jac_status read_residuals(jac_batch *b, double *res_host)
@@ -298,10 +417,12 @@ jac_status jac_batch_set_plan(jac_batch *b, int warps, const int *tile_i, const 
     if (!b) return bfail(b, JAC_EINVAL, "batch is NULL");
     if (warps != 0 && !jac::warps_supported(b->prec, warps)) return bfail(b, JAC_EINVAL, "unsupported warp count");
     b->warps = warps ? warps : 8;
+    b->own_plan = warps == 0;
     for (int g = 0; g < b->n; ++g) {
         b->tile_i[g] = tile_i ? tile_i[g] : 0;
         b->kdepth[g] = kdepth ? kdepth[g] : 0;
         if (b->tile_i[g] < 0 || b->kdepth[g] < 0) return bfail(b, JAC_EINVAL, "negative plan entry");
+        if (b->tile_i[g] != 0 || b->kdepth[g] != 0) b->own_plan = false;
     }
     drop_tables(b);
     return JAC_OK;
@@ -326,8 +447,7 @@ jac_status jac_batch_sweep(jac_batch *b, int n_iter, double *res_host)
             cudaStreamDestroy(cap);
             return bcuda(b, e, "cudaStreamBeginCapture");
         }
-        const jac::SweepArgs a = batch_args(b, n_iter);
-        s = jac::launch_sweep<true>(b->prec, b->warps, b->host_descs[0], a, b->nblocks, cap);
+        s = enqueue_sweeps(b, n_iter, cap);
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(cap, &graph);
         cudaStreamDestroy(cap);

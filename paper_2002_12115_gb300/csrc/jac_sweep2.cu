@@ -42,6 +42,9 @@
 //     registers hold one part's coefficients and the stencil's state values;
 //   * every wait is bounded; on expiry the kernel sets the workspace error
 //     word, drains its own copies, frees its tensor memory and returns;
+//   * batched (BATCH): the items of many grids in one list, each grid with its
+//     own descriptor in device memory; no residual (a batch ends with single
+//     sweeps);
 //   * a one-pass call may also store sweep 1's state at the points the
 //     items own (Sweep2Args::mid): the reverse pass recomputes two
 //     checkpoint-segment states per launch that way.
@@ -99,6 +102,10 @@ struct Sweep2Desc {
 };
 
 struct Sweep2Args {
+    const Sweep2Desc *descs;   // batched: one per grid
+    const int *item_base;      // batched: first item of each grid (ascending)
+    int ngrids, nitems;        // grids and items of a pass
+
     int n_pass, par;           // pass t reads p[(t + par) & 1], writes the other
     unsigned taken;            // items of the passes whose items are taken by ticket
     double omega;
@@ -127,6 +134,20 @@ __device__ __forceinline__ Item2 decode_item2(const Sweep2Desc &d, int item)
     it.kb = 1 + kk * d.kdepth;
     it.nout = min(d.K - 1, it.kb + d.kdepth) - it.kb;
     return it;
+}
+
+// Batched: the grid of an item, the last one whose first item is not past it;
+// `item` becomes its number within the grid.
+__device__ __forceinline__ const Sweep2Desc *find_grid(const Sweep2Args &a, int &item)
+{
+    int lo = 0, hi = a.ngrids - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(&a.item_base[mid]) <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    item -= __ldg(&a.item_base[lo]);
+    return a.descs + lo;
 }
 
 // VI values of an intermediate-plane row (no halo) with the left and right
@@ -196,6 +217,7 @@ __device__ __forceinline__ void tmem_loaded(float (&a)[4])
     asm volatile("" : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3])::"memory");
 }
 
+template <bool BATCH>
 __global__ void __launch_bounds__(Sweep2Shape::THREADS, 1)
 k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
 {
@@ -242,7 +264,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         ++ic;
         return r;
     };
-    const uint32_t nitems = (uint32_t)d.nitems;
+    const uint32_t nitems = (uint32_t)(BATCH ? a.nitems : d.nitems);
 
     if (warp == R1) {
         // ------------------------------------------------------------ producer
@@ -258,7 +280,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             const uint64_t pol_p = l2_policy(a.l2_keep_state ? 1 : 0);
             uint32_t pc = 0, cc = 0;
             bool ok = true;
-            const CUtensorMap *pm = nullptr;
+            const CUtensorMap *pm = nullptr, *cm = d.coef;
             auto put_state = [&](const Item2 &it, int q) -> bool {
                 const uint32_t slot = pc % RP, use = pc / RP;
                 if (use > 0 && !mbar_wait_bounded(&p_empty[slot], (use - 1) & 1)) return false;
@@ -276,7 +298,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 unsigned char *st = ring_c + (size_t)slot * S::C_BYTES;
                 mbar_arrive_expect_tx(&c_full[slot], (uint32_t)S::C_BYTES);
                 for (int k = JAC_A0; k <= JAC_BND; ++k)
-                    tma_load_3d_hint(st + (size_t)(k - 1) * S::TILE, &d.coef[k - 1], &c_full[slot], it.i0,
+                    tma_load_3d_hint(st + (size_t)(k - 1) * S::TILE, (BATCH ? cm : d.coef) + (k - 1), &c_full[slot], it.i0,
                                      it.j0 - 1, it.kb - 1 + q, ((a.l2_keep_coef >> k) & 1u) ? pol_keep : pol_c);
                 ++cc;
                 return true;
@@ -299,8 +321,17 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 uint32_t next = 0;
                 if (by_ticket) next = (uint32_t)G + atomicAdd(&a.hdr->ticket, 1u);   // used after this item
                 const uint32_t t = entry / nitems;
-                const Item2 it = decode_item2(d, (int)(entry - t * nitems));
-                pm = ((t + a.par) & 1) ? &d.p[1] : &d.p[0];
+                Item2 it;
+                if constexpr (BATCH) {
+                    int item = (int)(entry - t * nitems);
+                    const Sweep2Desc *g = find_grid(a, item);
+                    it = decode_item2(*g, item);
+                    pm = &g->p[(t + a.par) & 1];
+                    cm = g->coef;
+                } else {
+                    it = decode_item2(d, (int)(entry - t * nitems));
+                    pm = ((t + a.par) & 1) ? &d.p[1] : &d.p[0];
+                }
                 if (!(ok = put_coef(it, 0))) break;
                 if (t > pass) {            // every item of the passes before is stored
                     pass = t;
@@ -342,14 +373,23 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         const int r = lane >> 1, side = lane & 1;
         const bool act = lane < 2 * R1;
         const float omega = (float)a.omega;
-        const int I = d.I, J = d.J, K = d.K, pitch = d.pitch;
+        int I = d.I, J = d.J, K = d.K, pitch = d.pitch;
+        [[maybe_unused]] const Sweep2Desc *g = nullptr;
         const int x = side ? H + TI : H - 1;             // the column in the state box
         const int r0 = r * S::PW, r1 = (r + 1) * S::PW, r2 = (r + 2) * S::PW;
         uint32_t pc = 0, qc = 0;
         bool ok = true;
         uint32_t entry;
         while ((ok = next_item(entry)) && entry != S::END) {
-            const Item2 it = decode_item2(d, (int)(entry % nitems));
+            Item2 it;
+            if constexpr (BATCH) {
+                int item = (int)(entry % nitems);
+                g = find_grid(a, item);
+                it = decode_item2(*g, item);
+                I = g->I; J = g->J; K = g->K; pitch = g->pitch;
+            } else {
+                it = decode_item2(d, (int)(entry % nitems));
+            }
             const int j = it.j0 - 1 + r;
             const int ie = side ? it.i0 + TI : it.i0 - 1;
             const bool col_in = act && (j >= 1) && (j <= J - 2) && (ie >= 1) && (ie <= I - 2);
@@ -358,7 +398,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 if (col_in && m >= 1 && m <= K - 2) {
                     const size_t off = ((size_t)m * J + (size_t)j) * (size_t)pitch + (size_t)ie;
 #pragma unroll
-                    for (int q = 0; q < 12; ++q) v[q] = __ldg(d.coef_ptr[q] + off);
+                    for (int q = 0; q < 12; ++q) v[q] = __ldg((BATCH ? g->coef_ptr[q] : d.coef_ptr[q]) + off);
                 } else {
 #pragma unroll
                     for (int q = 0; q < 12; ++q) v[q] = 0.0f;
@@ -423,14 +463,23 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         const int w = warp;                         // row j0-1+w of every item
         const float omega = (float)a.omega;
         const uint64_t st_pol = l2_policy(a.l2_keep_state ? 1 : 0);
-        const int I = d.I, J = d.J, K = d.K, pitch = d.pitch;
+        int I = d.I, J = d.J, K = d.K, pitch = d.pitch;
+        [[maybe_unused]] const Sweep2Desc *g = nullptr;
         const bool do2 = (w >= 1) && (w <= R1 - 2);  // this warp's row is an output row too
         const uint32_t tm = s_tmem + ((uint32_t)(w & 3) << 21) + (uint32_t)(((w - 1) >> 2) * S::TM_SLOTS * S::TM_SLOT);
         uint32_t pc = 0, cc = 0, qc = 0;
         bool ok = true;
         uint32_t entry;
         while ((ok = next_item(entry)) && entry != S::END) {
-            const Item2 it = decode_item2(d, (int)(entry % nitems));
+            Item2 it;
+            if constexpr (BATCH) {
+                int item = (int)(entry % nitems);
+                g = find_grid(a, item);
+                it = decode_item2(*g, item);
+                I = g->I; J = g->J; K = g->K; pitch = g->pitch;
+            } else {
+                it = decode_item2(d, (int)(entry % nitems));
+            }
             const int j = it.j0 - 1 + w;
             const int ib = it.i0 + VI * lane;
             const bool row1_in = (j >= 1) && (j <= J - 2);
@@ -566,7 +615,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         const int w = (warp - S::WARP2) == 0 ? S::R2 : warp - S::WARP2;   // row j0-1+w of every item
         const float omega = (float)a.omega;
         const uint64_t st_pol = l2_policy(a.l2_keep_state ? 1 : 0);
-        const int I = d.I, J = d.J, pitch = d.pitch;
+        int I = d.I, J = d.J, pitch = d.pitch;
         const uint32_t tm = s_tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(((w - 1) >> 2) * S::TM_SLOTS * S::TM_SLOT);
         uint32_t qc = 0;
         bool ok = true;
@@ -582,9 +631,19 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         uint32_t entry;
         while ((ok = next_item(entry)) && entry != S::END) {
             const uint32_t t = entry / nitems;
-            const Item2 it = decode_item2(d, (int)(entry - t * nitems));
-            const bool res = (t == (uint32_t)a.n_pass - 1) && (a.res != nullptr);
-            float *p_out = static_cast<float *>(((t + 1 + a.par) & 1) ? d.p_buf[1] : d.p_buf[0]);
+            Item2 it;
+            float *p_out;
+            if constexpr (BATCH) {
+                int item = (int)(entry - t * nitems);
+                const Sweep2Desc *g = find_grid(a, item);
+                it = decode_item2(*g, item);
+                I = g->I; J = g->J; pitch = g->pitch;
+                p_out = static_cast<float *>(g->p_buf[(t + 1 + a.par) & 1]);
+            } else {
+                it = decode_item2(d, (int)(entry - t * nitems));
+                p_out = static_cast<float *>(((t + 1 + a.par) & 1) ? d.p_buf[1] : d.p_buf[0]);
+            }
+            const bool res = !BATCH && (t == (uint32_t)a.n_pass - 1) && (a.res != nullptr);
             const int j = it.j0 - 1 + w;
             const int ib = it.i0 + VI * lane;
             const bool row_in = j <= J - 2;
@@ -692,7 +751,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 }
             }
         }
-        if (ok && a.res != nullptr) {
+        if (!BATCH && ok && a.res != nullptr) {
             double v = acc;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -807,89 +866,135 @@ size_t sweep2_workspace_bytes(const jac_grid *g)
     return kWsHeaderBytes + round_up((size_t)std::min<long long>(items, sms) * sizeof(double), 256);
 }
 
+namespace {
+
+// Descriptor of one grid: tensor maps, tiling and item count.
+jac_status build_desc2(Sweep2Desc *d, const jac_grid *g, int kdepth)
+{
+    using S = Sweep2Shape;
+    std::memset(d, 0, sizeof(*d));
+    d->I = g->I; d->J = g->J; d->K = g->K;
+    d->pitch = jac_pitch(g->I);
+    d->nti = sweep2_tiles_i(g->I);
+    d->ntj = (g->J - 2 + S::R2 - 1) / S::R2;
+    d->kdepth = kdepth;
+    d->nkb = (g->K - 2 + kdepth - 1) / kdepth;
+    const long long items = (long long)d->nti * d->ntj * d->nkb;
+    if (items > 0x3fffffffLL) return fail2(JAC_EINVAL, "grid too large for the two-sweep launch shape");
+    d->nitems = (int)items;
+    d->p_buf[0] = g->p[0];
+    d->p_buf[1] = g->p[1];
+    jac_status s;
+    for (int b = 0; b < 2; ++b)
+        if ((s = encode_box_map(&d->p[b], g->p[b], 4, d->pitch, d->pitch, g->J, g->K, S::PW, S::PH)) != JAC_OK)
+            return s;
+    for (int q = JAC_A0; q <= JAC_BND; ++q) {
+        if ((s = encode_box_map(&d->coef[q - 1], g->coef[q], 4, d->pitch, d->pitch, g->J, g->K, S::TI, S::R1)) !=
+            JAC_OK)
+            return s;
+        d->coef_ptr[q - 1] = static_cast<const float *>(g->coef[q]);
+    }
+    return JAC_OK;
+}
+
+// All passes of a call.  Items of all passes and the arrivals of the pass
+// barrier are counted in 32 bits: very long calls take several launches, each
+// of an even number of passes.
+template <bool BATCH>
+jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStream_t st)
+{
+    using S = Sweep2Shape;
+    static std::once_flag attr_once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(attr_once, [] {
+        attr_err = cudaFuncSetAttribute(k_sweep2<BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    });
+    if (attr_err != cudaSuccess)
+        return fail2(JAC_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(attr_err));
+    const int most = (int)std::min<long long>(0x7ffffffe, (0xffff0000ll / ((long long)a.nitems * S::R2)) & ~1ll);
+    if (most < 2 && a.n_pass > most) return fail2(JAC_EINVAL, "grid too large for the two-sweep launch shape");
+    double *const res = a.res;
+    for (int left = a.n_pass; left > 0;) {
+        a.n_pass = std::min(left, most);
+        left -= a.n_pass;
+        a.res = left == 0 ? res : nullptr;
+        a.taken = (unsigned)(a.res ? a.n_pass - 1 : a.n_pass) * (unsigned)a.nitems;
+        cudaLaunchConfig_t cfg;
+        std::memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3(nblocks);
+        cfg.blockDim = dim3(S::THREADS);
+        cfg.dynamicSmemBytes = S::SMEM;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep2<BATCH>, d, a);
+        if (e != cudaSuccess) return fail2(JAC_ECUDA, std::string("two-sweep launch: ") + cudaGetErrorString(e));
+    }
+    return JAC_OK;
+}
+
+}  // namespace
+
 jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_residual, void *workspace,
                       size_t ws_bytes, cudaStream_t st, void *mid)
 {
-    using S = Sweep2Shape;
     if (mid != nullptr && n_pass != 1) return fail2(JAC_EINVAL, "the intermediate state needs a one-pass call");
-    Sweep2Desc d;
-    std::memset(&d, 0, sizeof(d));
-    d.I = g->I; d.J = g->J; d.K = g->K;
-    d.pitch = jac_pitch(g->I);
-    d.nti = sweep2_tiles_i(g->I);
-    d.ntj = (g->J - 2 + S::R2 - 1) / S::R2;
+    const long cols = (long)sweep2_tiles_i(g->I) * ((g->J - 2 + Sweep2Shape::R2 - 1) / Sweep2Shape::R2);
     const int sms = device_sm_count();
-    d.kdepth = kdepth > 0 ? kdepth : sweep2_kdepth((long)d.nti * d.ntj, g->K - 2, sms);
-    d.nkb = (g->K - 2 + d.kdepth - 1) / d.kdepth;
-    const long long items = (long long)d.nti * d.ntj * d.nkb;
-    if (items > 0x3fffffffLL) return fail2(JAC_EINVAL, "grid too large for the two-sweep launch shape");
-    d.nitems = (int)items;
-    d.p_buf[0] = g->p[0];
-    d.p_buf[1] = g->p[1];
-    jac_status s;
-    for (int b = 0; b < 2; ++b)
-        if ((s = encode_box_map(&d.p[b], g->p[b], 4, d.pitch, d.pitch, g->J, g->K, S::PW, S::PH)) != JAC_OK)
-            return s;
-    for (int q = JAC_A0; q <= JAC_BND; ++q) {
-        if ((s = encode_box_map(&d.coef[q - 1], g->coef[q], 4, d.pitch, d.pitch, g->J, g->K, S::TI, S::R1)) !=
-            JAC_OK)
-            return s;
-        d.coef_ptr[q - 1] = static_cast<const float *>(g->coef[q]);
-    }
-    const unsigned nblocks = (unsigned)std::min<long long>(items, sms);
+    Sweep2Desc d;
+    jac_status s = build_desc2(&d, g, kdepth > 0 ? kdepth : sweep2_kdepth(cols, g->K - 2, sms));
+    if (s != JAC_OK) return s;
+    const unsigned nblocks = (unsigned)std::min(d.nitems, sms);
     if (ws_bytes < kWsHeaderBytes + (size_t)nblocks * sizeof(double))
         return fail2(JAC_EINVAL, "workspace too small for the two-sweep launch");
-    WsHeader *hdr = static_cast<WsHeader *>(workspace);
     Sweep2Args a;
     std::memset(&a, 0, sizeof(a));
+    a.ngrids = 1;
+    a.nitems = d.nitems;
     a.n_pass = n_pass;
-    a.taken = (unsigned)(d_residual ? n_pass - 1 : n_pass) * (unsigned)d.nitems;
-    a.par = 0;
     a.omega = g->omega;
     a.partials = reinterpret_cast<double *>(static_cast<char *>(workspace) + kWsHeaderBytes);
     a.res = d_residual;
     a.mid = static_cast<float *>(mid);
-    a.hdr = hdr;
-    // Items of all passes and the arrivals of the pass barrier are counted in
-    // 32 bits: longer calls take several launches of an even number of passes.
-    const long long most = (0xffff0000ll / (items * S::R2)) & ~1ll;
-    if (n_pass > most) {
-        if (most < 2) return fail2(JAC_EINVAL, "grid too large for the two-sweep launch shape");
-        for (int left = n_pass; left > 0;) {
-            const int now = (int)std::min<long long>(left, most);
-            left -= now;
-            if ((s = sweep2_run(g, kdepth, now, left == 0 ? d_residual : nullptr, workspace, ws_bytes, st)) != JAC_OK)
-                return s;
-        }
-        return JAC_OK;
-    }
+    a.hdr = static_cast<WsHeader *>(workspace);
     SweepArgs la;
     std::memset(&la, 0, sizeof(la));
     set_l2_policy(la, g->prec, (size_t)d.pitch * g->J * g->K);
     a.l2_keep_state = la.l2_keep_state;
     a.l2_keep_coef = la.l2_keep_coef;
+    return launch2<false>(d, a, nblocks, st);
+}
 
-    static std::once_flag attr_once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(attr_once, [] {
-        attr_err = cudaFuncSetAttribute(k_sweep2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    });
-    if (attr_err != cudaSuccess)
-        return fail2(JAC_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(attr_err));
-    cudaLaunchConfig_t cfg;
-    std::memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(nblocks);
-    cfg.blockDim = dim3(S::THREADS);
-    cfg.dynamicSmemBytes = S::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep2, d, a);
-    if (e != cudaSuccess) return fail2(JAC_ECUDA, std::string("two-sweep launch: ") + cudaGetErrorString(e));
-    return JAC_OK;
+// ---- batches: the descriptors of many grids in device memory
+size_t sweep2_desc_bytes() { return sizeof(Sweep2Desc); }
+
+jac_status sweep2_batch_desc(void *desc, const jac_grid *g, int kdepth, int *items)
+{
+    Sweep2Desc *d = static_cast<Sweep2Desc *>(desc);
+    const jac_status s = build_desc2(d, g, kdepth);
+    if (s == JAC_OK) *items = d->nitems;
+    return s;
+}
+
+jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids, int nitems, int n_pass, int par,
+                            double omega, void *workspace, cudaStream_t st)
+{
+    Sweep2Args a;
+    std::memset(&a, 0, sizeof(a));
+    a.descs = static_cast<const Sweep2Desc *>(descs);
+    a.item_base = item_base;
+    a.ngrids = ngrids;
+    a.nitems = nitems;
+    a.n_pass = n_pass;
+    a.par = par;
+    a.omega = omega;
+    a.hdr = static_cast<WsHeader *>(workspace);
+    Sweep2Desc unused;
+    std::memset(&unused, 0, sizeof(unused));
+    return launch2<true>(unused, a, (unsigned)std::min(nitems, device_sm_count()), st);
 }
 
 }  // namespace jac

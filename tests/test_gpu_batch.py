@@ -186,3 +186,42 @@ def test_config4_full_batch():
     print(f"512 grids against the oracle: worst p err {worst[0]:.2e}, residual err {worst[1]:.2e}")
     b1.close()
     b2.close()
+
+
+@pytest.mark.parametrize("n", [5, 6, 12])
+def test_two_sweep_passes_of_a_batch(n):
+    """Without a plan the wide grids of a FP32 batch that leaves L2 run in
+    two-sweep passes for all but a call's last sweeps: state bitwise that of
+    per-grid launches and of the same batch with an explicit plan (single
+    sweeps), in both buffer parities; residuals to 1e-9 (their FP32 squares are
+    summed in the same groups, the FP64 sums in another order)."""
+    import torch
+
+    from paper_2002_12115_gb300 import JacobiBatch
+    dims = [(129, 129, 129)] * 17 + [(17, 33, 49), (97, 65, 30), (129, 20, 17), (65, 65, 65), (200, 40, 33)]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    fields = []
+    for I, J, K in dims:
+        f = {q: 0.95 + 0.1 * torch.rand((K, J, I), generator=g, dtype=torch.float64, device="cuda")
+             for q in ("a0", "a1", "a2", "c0", "c1", "c2")}
+        f.update({q: 0.02 * torch.rand((K, J, I), generator=g, dtype=torch.float64, device="cuda")
+                  for q in ("b0", "b1", "b2", "wrk1", "p")})
+        f["a3"] = 1.0 / (f["a0"] + f["a1"] + f["a2"] + f["c0"] + f["c1"] + f["c2"])
+        f["bnd"] = torch.zeros_like(f["p"])
+        f["bnd"][1:-1, 1:-1, 1:-1] = 1.0
+        fields.append(f)
+    got = []
+    for how in ("passes", "plan", "loop"):
+        with JacobiBatch(dims, "f32") as b:
+            for k, f in enumerate(fields):
+                b.upload_tensors(k, f)
+            if how == "plan":
+                b.set_plan(8)
+            sweep = b.sweep_loop if how == "loop" else b.sweep
+            res = [sweep(n), sweep(n + 3)]
+            got.append((res, [b.download_tensor(k) for k in range(len(dims))]))
+    for res, p in got[1:]:
+        for k in range(len(dims)):
+            assert torch.equal(p[k], got[0][1][k]), (k, dims[k])
+        for r0, r1 in zip(got[0][0], res):
+            assert np.all(np.abs(r1 - r0) <= 1e-9 * r0)
