@@ -38,28 +38,33 @@
 //   * warp 11 (the edge warp, 20 lanes) computes sweep 1 at columns i0-1 and
 //     i0+128 of the R1 rows, from the state ring and coefficients it loads
 //     from global memory one plane ahead;
-//   * both sweeps take the update in two parts (ss_axes, ss_rest), so that 96
-//     registers hold one part's coefficients and the stencil's state values;
+//   * both sweeps take the update in two parts (ss_axes, ss_rest), and sweep 1
+//     forms the b brackets before it loads a coefficient, so that 96 registers
+//     hold one part's coefficients and the state values still needed.  Spilled
+//     registers went through an L1 of a few KB, behind the copies' traffic;
+//   * two points share an instruction (f32x2) where both operands lie in
+//     aligned register pairs: a3 S - 1 and the axis terms;
 //   * every wait is bounded; on expiry the kernel sets the workspace error
 //     word, drains its own copies, frees its tensor memory and returns;
 //   * batched (BATCH): the items of many grids in one list, each grid with its
 //     own descriptor in device memory; no residual (a batch ends with single
 //     sweeps);
 //   * a one-pass call may also store sweep 1's state at the points the
-//     items own (Sweep2Args::mid): the reverse pass recomputes two
+//     items own (MID, Sweep2Args::mid): the reverse pass recomputes two
 //     checkpoint-segment states per launch that way.
 //
-// What bounds it: a step of a CTA (one plane of a tile, both sweeps) takes
-// 1.65 us up to two tiles along i, whether the state stays in L2 or not
-// (latency and issue of 18 compute warps), and 1.8-2.0 us from three tiles on,
-// where it draws 5.4 TB/s from DRAM.  Kept against, on one GB300 (Gpt/s, FP32):
-//                                             257x257x513   513x513x1025
+// What bounds it: latency and issue of 18 compute warps where the state stays in
+// L2 (a step of a CTA, one plane of a tile, both sweeps, takes 1.36 us), DRAM
+// elsewhere, which delivers 5.8 TB/s but 1.2-1.3 times the bytes a pass needs.
+// Kept against, on one GB300 (Gpt/s, FP32):
+//                                             129x129x257   257x257x513   513x513x1025
 //   both sweeps in one warp, coefficients of
 //     sweep 2 read again from L2 (41% of all
-//     L2 reads)                                    141            145
-//   ... kept in tensor memory                      150            153
-//   separate warps for the two sweeps              164            143
-//   ... and items by ticket (this kernel)          171            149
+//     L2 reads)                                                   141            145
+//   ... kept in tensor memory                                     150            153
+//   separate warps for the two sweeps                             164            143
+//   ... and items by ticket                        161            171            150
+//   barriers tested together, no spills, f32x2     189            172            158
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -217,7 +222,87 @@ __device__ __forceinline__ void tmem_loaded(float (&a)[4])
     asm volatile("" : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3])::"memory");
 }
 
-template <bool BATCH>
+// Two FP32 numbers in one register pair: one instruction for two points where
+// both operands lie in aligned pairs.  Each half rounds like the single
+// instruction, so the values are bitwise the same.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ void fast_two_sum_acc2(f32x2 &hi, f32x2 &lo, f32x2 b)
+{
+    const f32x2 s = add2(hi, b);
+    lo = add2(lo, sub2(b, sub2(s, hi)));
+    hi = s;
+}
+
+// a3s_minus_one<false> of four points.
+__device__ __forceinline__ void a3s_minus_one4(const float (&a3)[4], const float (&a0)[4], const float (&a1)[4],
+                                               const float (&a2)[4], const float (&c0)[4], const float (&c1)[4],
+                                               const float (&c2)[4], float (&ec)[4])
+{
+#pragma unroll
+    for (int e = 0; e < 4; e += 2) {
+        f32x2 hi = pack2(fmaxf(a0[e], c0[e]), fmaxf(a0[e + 1], c0[e + 1])), lo = pack2(0.0f, 0.0f);
+        fast_two_sum_acc2(hi, lo, pack2(fminf(a0[e], c0[e]), fminf(a0[e + 1], c0[e + 1])));
+        fast_two_sum_acc2(hi, lo, pack2(a1[e], a1[e + 1]));
+        fast_two_sum_acc2(hi, lo, pack2(c1[e], c1[e + 1]));
+        fast_two_sum_acc2(hi, lo, pack2(a2[e], a2[e + 1]));
+        fast_two_sum_acc2(hi, lo, pack2(c2[e], c2[e + 1]));
+        const f32x2 s = pack2(a3[e], a3[e + 1]);
+        unpack2(fma2(s, lo, fma2(s, hi, pack2(-1.0f, -1.0f))), ec[e], ec[e + 1]);
+    }
+}
+
+// ss_axes of four points; x, yp, ym, zp, zm with one value past each end.  The
+// differences along i, whose operands are shifted by one point, are formed
+// singly, into aligned pairs.
+__device__ __forceinline__ void ss_axes4(const float (&x)[6], const float (&yp)[6], const float (&ym)[6],
+                                         const float (&zp)[6], const float (&zm)[6], const float (&a0)[4],
+                                         const float (&a1)[4], const float (&a2)[4], const float (&c0)[4],
+                                         const float (&c1)[4], const float (&c2)[4], const float (&wk)[4],
+                                         float (&d)[4])
+{
+#pragma unroll
+    for (int e = 0; e < 4; e += 2) {
+        const f32x2 c = pack2(x[e + 1], x[e + 2]);
+        f32x2 s = pack2(wk[e], wk[e + 1]);
+        s = fma2(pack2(a0[e], a0[e + 1]), pack2(x[e + 2] - x[e + 1], x[e + 3] - x[e + 2]), s);
+        s = fma2(pack2(a1[e], a1[e + 1]), sub2(pack2(yp[e + 1], yp[e + 2]), c), s);
+        s = fma2(pack2(a2[e], a2[e + 1]), sub2(pack2(zp[e + 1], zp[e + 2]), c), s);
+        s = fma2(pack2(c0[e], c0[e + 1]), pack2(x[e] - x[e + 1], x[e + 1] - x[e + 2]), s);
+        s = fma2(pack2(c1[e], c1[e + 1]), sub2(pack2(ym[e + 1], ym[e + 2]), c), s);
+        s = fma2(pack2(c2[e], c2[e + 1]), sub2(pack2(zm[e + 1], zm[e + 2]), c), s);
+        unpack2(s, d[e], d[e + 1]);
+    }
+}
+
+template <bool BATCH, bool MID>
 __global__ void __launch_bounds__(Sweep2Shape::THREADS, 1)
 k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
 {
@@ -407,6 +492,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             load_coef(it.kb - 1, cf);
             for (int s = 0; s < it.nout + 2; ++s) {
                 const int m = it.kb - 1 + s;
+                const bool gone = s_abort;
                 if (s == 0) {
                     ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
                          mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
@@ -415,7 +501,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
                 const uint32_t qs = qc + s;
                 if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
-                ok = __all_sync(0xffffffffu, ok && !s_abort);
+                ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
                 if (s + 1 < it.nout + 2) load_coef(m + 1, cn);
                 if (act) {
@@ -467,7 +553,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         [[maybe_unused]] const Sweep2Desc *g = nullptr;
         const bool do2 = (w >= 1) && (w <= R1 - 2);  // this warp's row is an output row too
         const uint32_t tm = s_tmem + ((uint32_t)(w & 3) << 21) + (uint32_t)(((w - 1) >> 2) * S::TM_SLOTS * S::TM_SLOT);
-        uint32_t pc = 0, cc = 0, qc = 0;
+        uint32_t pc = 0, qc = 0;
         bool ok = true;
         uint32_t entry;
         while ((ok = next_item(entry)) && entry != S::END) {
@@ -497,21 +583,31 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             for (int s = 0; s < it.nout + 2; ++s) {
                 const int m = it.kb - 1 + s;                 // sweep-1 plane
                 const uint32_t qs = qc + s;
+                const bool gone = s_abort;
                 if (s == 0) {
                     ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
                          mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
                 }
                 const uint32_t q2 = pc + s + 2;
-                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
-                ok = ok && mbar_wait_bounded(&c_full[(cc + s) % RC], ((cc + s) / RC) & 1);
-                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
-                ok = __all_sync(0xffffffffu, ok && !s_abort);
+                // The newest state plane, the stage and a free intermediate
+                // plane (whose phase before the first use counts as
+                // complete), tested together: one latency when all are there.
+                const bool got_p = mbar_try_wait(&p_full[q2 % RP], (q2 / RP) & 1);
+                const bool got_c = mbar_try_wait(&c_full[qs % RC], (qs / RC) & 1);
+                const bool got_q = mbar_try_wait(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
+                ok = ok && !gone;
+                if (!__all_sync(0xffffffffu, ok && got_p && got_c && got_q)) {
+                    ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1) &&
+                         mbar_wait_bounded(&c_full[qs % RC], (qs / RC) & 1) &&
+                         mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
+                    ok = __all_sync(0xffffffffu, ok);
+                }
                 if (!ok) break;
                 const float *Pm = reinterpret_cast<const float *>(base + (size_t)((pc + s) % RP) * S::P_BYTES);
                 const float *Pk =
                     reinterpret_cast<const float *>(base + (size_t)((pc + s + 1) % RP) * S::P_BYTES);
                 const float *Pp = reinterpret_cast<const float *>(base + (size_t)(q2 % RP) * S::P_BYTES);
-                const unsigned char *cs = ring_c + (size_t)((cc + s) % RC) * S::C_BYTES;
+                const unsigned char *cs = ring_c + (size_t)(qs % RC) * S::C_BYTES;
                 float ek0[VI + 2], ek1[VI + 2], ek2[VI + 2], em1[VI + 2], ep1[VI + 2];
                 float vm0[VI], vm2[VI], vp0[VI], vp2[VI];
                 load_ext<float, VI, H>(Pk + r0, lane, 32, ek0);
@@ -531,6 +627,15 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 // The coefficients in the two parts of the update, so that
                 // only one part's are held in registers at a time; an
                 // output row keeps them for sweep 2 at this plane.
+                float bij[VI], bjk[VI], bik[VI];
+#pragma unroll
+                for (int e = 0; e < VI; ++e) {
+                    bij[e] = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
+                    bjk[e] = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
+                    bik[e] = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
+                }
+                // formed before the coefficients are loaded: nothing is spilled
+                tmem_loaded(bij); tmem_loaded(bjk); tmem_loaded(bik);
                 float dd[VI], ec[VI];
                 {
                     float wk[VI], a0[VI], a1[VI], a2[VI], c0[VI], c1[VI], c2[VI];
@@ -544,12 +649,8 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                     }
                     float a3[VI];
                     coef(JAC_A3, a3);
-#pragma unroll
-                    for (int e = 0; e < VI; ++e) {
-                        dd[e] = ss_axes(ek1[e + 1], ek1[e + 2], ek1[e], ek2[e + 1], ek0[e + 1], ep1[e + 1],
-                                        em1[e + 1], a0[e], a1[e], a2[e], c0[e], c1[e], c2[e], wk[e]);
-                        ec[e] = a3s_minus_one<false>(a3[e], a0[e], a1[e], a2[e], c0[e], c1[e], c2[e]);
-                    }
+                    ss_axes4(ek1, ek2, ek0, ep1, em1, a0, a1, a2, c0, c1, c2, wk, dd);
+                    a3s_minus_one4(a3, a0, a1, a2, c0, c1, c2, ec);
                 }
                 float out[VI];
                 {
@@ -563,16 +664,14 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
 #pragma unroll
                     for (int e = 0; e < VI; ++e) {
                         const float c = ek1[e + 1];
-                        const float bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
-                        const float bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
-                        const float bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
-                        const float ss = ss_rest(dd[e], c, bij, bjk, bik, a3[e], b0[e], b1[e], b2[e], bn[e], ec[e]);
+                        const float ss = ss_rest(dd[e], c, bij[e], bjk[e], bik[e], a3[e], b0[e], b1[e], b2[e],
+                                                 bn[e], ec[e]);
                         out[e] = (in1 && in_i[e]) ? fmaf(omega, ss, c) : c;
                     }
                 }
                 float *qrow = reinterpret_cast<float *>(ring_q + (size_t)(qs % RQ) * S::Q_BYTES) + w * TI;
                 *reinterpret_cast<float4 *>(qrow + VI * lane) = make_float4(out[0], out[1], out[2], out[3]);
-                if (a.mid != nullptr && m >= it.kb && m < it.kb + it.nout) {
+                if (MID && m >= it.kb && m < it.kb + it.nout) {
                     // the intermediate state at this item's own points
                     const size_t offm = ((size_t)m * J + (size_t)j) * (size_t)pitch + (size_t)ib;
                     if (all_owned) {
@@ -591,7 +690,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 if (lane == 0) {
                     mbar_arrive(&q_full[qs % RQ]);            // intermediate plane s: this row written
                     mbar_arrive(&p_empty[(pc + s) % RP]);     // state plane m-1 is done
-                    mbar_arrive(&c_empty[(cc + s) % RC]);     // stage s is done
+                    mbar_arrive(&c_empty[qs % RC]);     // stage s is done
                 }
             }
             if (!ok) break;
@@ -601,7 +700,6 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 mbar_arrive(&p_empty[(pc + it.nout + 3) % RP]);
             }
             pc += it.nout + 4;
-            cc += it.nout + 2;
             qc += it.nout + 2;
         }
         if (!ok) {
@@ -658,11 +756,12 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 // output plane kb-3+s from intermediate planes s-3 .. s-1
                 const uint32_t qs = qc + s;
                 const size_t off = ((size_t)(it.kb - 3 + s) * J + (size_t)j) * (size_t)pitch + (size_t)ib;
+                const bool gone = s_abort;
                 if (s == 3)
                     ok = mbar_wait_bounded(&q_full[qc % RQ], (qc / RQ) & 1) &&
                          mbar_wait_bounded(&q_full[(qc + 1) % RQ], ((qc + 1) / RQ) & 1);
                 ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1);
-                ok = __all_sync(0xffffffffu, ok && !s_abort);
+                ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const float *Qm =
@@ -697,10 +796,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                     tmem_wait_ld();
                     tmem_loaded(wk); tmem_loaded(a0); tmem_loaded(a1); tmem_loaded(a2);
                     tmem_loaded(c0); tmem_loaded(c1); tmem_loaded(c2);
-#pragma unroll
-                    for (int e = 0; e < VI; ++e)
-                        dd[e] = ss_axes(ek1[e + 1], ek1[e + 2], ek1[e], ek2[e + 1], ek0[e + 1], ep1[e + 1],
-                                        em1[e + 1], a0[e], a1[e], a2[e], c0[e], c1[e], c2[e], wk[e]);
+                    ss_axes4(ek1, ek2, ek0, ep1, em1, a0, a1, a2, c0, c1, c2, wk, dd);
                 }
                 float ss2 = 0.0f;
                 {
@@ -900,14 +996,15 @@ jac_status build_desc2(Sweep2Desc *d, const jac_grid *g, int kdepth)
 // All passes of a call.  Items of all passes and the arrivals of the pass
 // barrier are counted in 32 bits: very long calls take several launches, each
 // of an even number of passes.
-template <bool BATCH>
+template <bool BATCH, bool MID>
 jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStream_t st)
 {
     using S = Sweep2Shape;
     static std::once_flag attr_once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(attr_once, [] {
-        attr_err = cudaFuncSetAttribute(k_sweep2<BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        attr_err = cudaFuncSetAttribute(k_sweep2<BATCH, MID>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)S::SMEM);
     });
     if (attr_err != cudaSuccess)
         return fail2(JAC_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(attr_err));
@@ -930,7 +1027,7 @@ jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStre
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep2<BATCH>, d, a);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep2<BATCH, MID>, d, a);
         if (e != cudaSuccess) return fail2(JAC_ECUDA, std::string("two-sweep launch: ") + cudaGetErrorString(e));
     }
     return JAC_OK;
@@ -965,7 +1062,8 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
     set_l2_policy(la, g->prec, (size_t)d.pitch * g->J * g->K);
     a.l2_keep_state = la.l2_keep_state;
     a.l2_keep_coef = la.l2_keep_coef;
-    return launch2<false>(d, a, nblocks, st);
+    return mid != nullptr ? launch2<false, true>(d, a, nblocks, st)
+                          : launch2<false, false>(d, a, nblocks, st);
 }
 
 // ---- batches: the descriptors of many grids in device memory
@@ -994,7 +1092,7 @@ jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids,
     a.hdr = static_cast<WsHeader *>(workspace);
     Sweep2Desc unused;
     std::memset(&unused, 0, sizeof(unused));
-    return launch2<true>(unused, a, (unsigned)std::min(nitems, device_sm_count()), st);
+    return launch2<true, false>(unused, a, (unsigned)std::min(nitems, device_sm_count()), st);
 }
 
 }  // namespace jac
