@@ -139,11 +139,11 @@ jac_status upload_part(jac_batch::Part *p, const void *descs, size_t desc_bytes,
 // Which grids take two-sweep passes, and both parts' tables.  A batch whose
 // state stays in L2 keeps single sweeps; elsewhere those are bound by DRAM
 // (8.55 ns per 1000 stored points, measured on the 512-grid batch), and a pass
-// takes 1.67 us per step on one of the SMs, so a grid's width decides: 129
+// takes 1.45 us per step on one of the SMs, so a grid's width decides: 129
 // columns fill the passes' 128-column tiles, 97 three quarters of them, and
 // narrower grids are faster in single sweeps with folded rows.  Items of up to
 // 32 planes (16, 24, 48, 64, 128 planes: 1.4, 0.5, 1.1, 1.3, 5% slower).  The
-// 512 grids, 40 sweeps: 51.3 -> 47.0 ms.
+// 512 grids, 40 sweeps: 51.3 -> 43.1 ms.
 jac_status build_parts(jac_batch *b)
 {
     if (!b->own_plan || b->prec != JAC_F32 || b->warps != 8) return JAC_OK;
@@ -157,7 +157,7 @@ jac_status build_parts(jac_batch *b)
         const int nk = b->K[g] - 2, blocks = (nk + 31) / 32, kd = (nk + blocks - 1) / blocks;
         const double steps = (double)((b->I[g] - 2) / 128 + 1) * ((b->J[g] - 2 + 7) / 8) * (nk + 3.0 * blocks);
         const double one = 8.55e-6 * (double)jac_pitch(b->I[g]) * b->J[g] * b->K[g];
-        const double two = 0.5 * 1.67 * steps / sms;
+        const double two = 0.5 * 1.45 * steps / sms;
         if (two < 0.95 * one) {
             wide.push_back(g);
             depth.push_back(std::max(kd, 1));
@@ -168,7 +168,7 @@ jac_status build_parts(jac_batch *b)
         }
     }
     // a pass ends with part of an item's time on most SMs idle (up to 35 steps)
-    if (wide.empty() || saved < 0.5 * 1.67 * 35.0 || steps_all < 4.0 * 35.0 * sms) return JAC_OK;
+    if (wide.empty() || saved < 0.5 * 1.45 * 35.0 || steps_all < 4.0 * 35.0 * sms) return JAC_OK;
     std::vector<char> d2(jac::sweep2_desc_bytes() * wide.size());
     std::vector<int> base2, base1;
     long long items2 = 0, items1 = 0;

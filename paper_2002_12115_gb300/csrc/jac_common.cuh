@@ -17,7 +17,8 @@ struct WsHeader {
     int errword;          // JAC_OK or JAC_ETIMEOUT, written by kernels
     unsigned counter;     // CTAs finished (last one reduces and resets)
     unsigned gbar;        // grid barrier between sweeps of one launch
-    unsigned ticket;      // items taken from a launch's common list (two-sweep passes)
+    unsigned ticket;      // items taken from a launch's common list (batched two-sweep passes)
+    unsigned clock;       // progress of all CTAs of a launch (two-sweep passes)
     double residual;      // default destination of the residual
 };
 constexpr size_t kWsHeaderBytes = 256;
@@ -92,6 +93,13 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p)
 {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ unsigned ld_relaxed_gpu(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 

@@ -74,8 +74,8 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
 // Whether the library's plan for this grid takes two-sweep passes (fuse 0).
 bool two_sweep_default(const jac_grid *g);
 size_t sweep2_workspace_bytes(const jac_grid *g);
-// Steps of a two-sweep pass over the grid, and its tiles along i.
-long sweep2_steps(const jac_grid *g, int *tiles_i);
+// Steps of a two-sweep pass over the grid.
+long sweep2_steps(const jac_grid *g);
 // Two-sweep passes of a batch: descriptors (sweep2_desc_bytes each, built on
 // the host, used from device memory) and first items of its grids.  No
 // residual; n_pass even; pass t reads p[(t + par) & 1].

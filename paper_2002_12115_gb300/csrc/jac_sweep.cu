@@ -459,24 +459,21 @@ bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws
 
 // Whether a call of n_iter sweeps with the library's own plan (all zero) takes
 // two-sweep passes: the faster of the two by the measured rates of both
-// kernels (16 FP32 grids, 65x200x200 to 513x513x1025).  A step of a pass's
-// busiest CTA takes 1.55 us where both state buffers stay in half the L2, 1.67
-// where they do not, and 2.0 from three tiles along i on (more of its columns
-// and rows come from DRAM twice).  A single sweep takes 2 us and 7.1 ns per
-// 1000 points in the first case and 8.5 ns per 1000 points otherwise.  What
-// decides is how well 128 columns by 8 rows tile the grid: 129x129x257 (full
-// tiles) 31.1 us a sweep against 25.6 in passes, 161x161x161 (two tiles 62%
-// full) 29.8 against 43.5.  The single sweeps after the passes are a launch of
-// their own (11 us).
+// kernels (21 FP32 grids, 65x200x200 to 513x513x1025).  A step of a pass's
+// busiest CTA takes 1.30-1.43 us on 16 of them and up to 1.7 on the others.
+// A single sweep takes 2 us and 7.1 ns per 1000 points where both state buffers
+// stay in half the L2 and 8.5 ns per 1000 points otherwise.  What decides is
+// how well 128 columns by 8 rows tile the grid: 129x129x257 (full tiles) 31.0
+// us a sweep against 21.5 in passes, 161x161x161 (two tiles 62% full) 29.3
+// against 35.2, 300x205x399 (three tiles 78% full) 207 against 182.  The
+// single sweeps after the passes are a launch of their own (11 us).
 static bool two_sweeps_pay(const jac_grid *g, int n_iter)
 {
     if (g->prec != JAC_F32 || n_iter < 4) return false;
-    int tiles_i = 1;
-    const long steps = sweep2_steps(g, &tiles_i);
     const double state = 2.0 * (double)jac_pitch(g->I) * g->J * g->K * 4.0;
     const bool kept = state <= 0.5 * (double)device_l2_bytes();
     const double points = (double)(g->I - 2) * (g->J - 2) * (g->K - 2);
-    const double two = 0.5 * (kept ? 1.55 : (tiles_i > 2 ? 2.0 : 1.67)) * (double)steps;   // us a sweep
+    const double two = 0.5 * 1.45 * (double)sweep2_steps(g);   // us a sweep
     const double one = kept ? 2.0 + 7.1e-6 * points : 8.5e-6 * points;
     const int in_passes = 4 * (n_iter / 4), rest = n_iter - in_passes;
     return in_passes * two + (rest ? 11.0 + rest * one : 0.0) < n_iter * one;

@@ -16,11 +16,17 @@
 //     R1 = R2 + 2 rows j0-1 .. j0+R2 and the planes kb-1 .. ke; sweep 2 over
 //     the R2 inner rows and planes kb .. ke-1.  Tiles do not overlap: sweep 2
 //     at columns i0 and i0+127 needs sweep 1 at columns i0-1 and i0+128 too;
-//   * CTAs take the items of a pass by ticket, in the order of their numbers,
-//     so that tiles next to one another are worked on at about the same time
-//     and no CTA waits for a slower one before the end of a pass; the queue
-//     entry of a CTA's next item carries its pass.  A last pass with a
-//     residual assigns items by CTA number, so that its sum has a fixed order.
+//   * items are numbered along i, then j, then k, and CTA b takes items b,
+//     b + G, ... of every pass (a fixed assignment also keeps the order of the
+//     residual's sum).  A tile shares two columns (whole sectors, in twelve
+//     arrays) and two rows with its neighbours along i and j: 1.32 times the
+//     bytes where each reads them from DRAM.  They are in L2 when the tiles
+//     are worked on at the same time, so the producers keep in step by a clock:
+//     the sum of all CTAs' planes / 4.  None starts a plane more than 8 planes
+//     ahead of the average (it waits 20 us at most, then goes on); the CTA
+//     furthest behind never waits.  Batched, the grids' items differ in size:
+//     they are taken by ticket, whichever CTA is free, without the clock;
+//   * the queue entry of a CTA's next item carries its pass.
 //     Before the state of pass t the producer waits until every item of the
 //     passes before is stored (a counter; each sweep-2 warp adds one per item);
 //   * warp 10 (one lane) copies, in the order they are used, the planes of
@@ -54,9 +60,9 @@
 //     checkpoint-segment states per launch that way.
 //
 // What bounds it: latency and issue of 18 compute warps where the state stays in
-// L2 (a step of a CTA, one plane of a tile, both sweeps, takes 1.36 us), DRAM
-// elsewhere, which delivers 5.8 TB/s but 1.2-1.3 times the bytes a pass needs.
-// Kept against, on one GB300 (Gpt/s, FP32):
+// L2 (a step of a CTA, one plane of a tile, both sweeps, takes 1.34 us), and
+// DRAM elsewhere: 513x513x1025 reads and writes 1.06 times the bytes a pass
+// needs at 6.1 TB/s.  Kept against, on one GB300 (Gpt/s, FP32):
 //                                             129x129x257   257x257x513   513x513x1025
 //   both sweeps in one warp, coefficients of
 //     sweep 2 read again from L2 (41% of all
@@ -65,6 +71,10 @@
 //   separate warps for the two sweeps                             164            143
 //   ... and items by ticket                        161            171            150
 //   barriers tested together, no spills, f32x2     189            172            158
+//   i-neighbours first, all CTAs in step
+//     (this kernel)                                192            216            208
+// The order alone (by ticket) ran at 184 and 157, the clock alone at 174 and
+// 160; the clock's lead of 1 to 8 ticks made 1% of difference.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -93,6 +103,9 @@ struct Sweep2Shape {
     static constexpr int THREADS = 32 * (R1 + 2 + R2);
     static constexpr int NQ = 4;                             // item queue of a CTA
     static constexpr uint32_t END = 0xffffffffu;             // no further item
+    static constexpr uint32_t TICK = 4;                      // planes of a tick of the clock
+    static constexpr uint32_t LEAD = 2;                      // ticks a CTA may be ahead of the average
+    static constexpr unsigned long long CLOCK_WAIT_NS = 20000;   // then it goes on all the same
     static_assert(P_BYTES % 128 == 0 && Q_BYTES % 128 == 0 && C_BYTES % 128 == 0, "slot alignment");
     static_assert(R2 / 4 * TM_SLOTS * TM_SLOT <= TM_COLS && WARP2 % 4 == 0 && R2 % 4 == 0, "tensor memory columns");
 };
@@ -112,7 +125,6 @@ struct Sweep2Args {
     int ngrids, nitems;        // grids and items of a pass
 
     int n_pass, par;           // pass t reads p[(t + par) & 1], writes the other
-    unsigned taken;            // items of the passes whose items are taken by ticket
     double omega;
     double *partials;          // gridDim.x
     double *res;               // residual of the last pass's second sweep (NULL: none)
@@ -130,10 +142,10 @@ __device__ __forceinline__ Item2 decode_item2(const Sweep2Desc &d, int item)
 {
     using S = Sweep2Shape;
     Item2 it;
-    const int tj = item % d.ntj;
-    const int r = item / d.ntj;
-    it.ti = r % d.nti;
-    const int kk = r / d.nti;
+    it.ti = item % d.nti;
+    const int r = item / d.nti;
+    const int tj = r % d.ntj;
+    const int kk = r / d.ntj;
     it.i0 = it.ti * S::TI;
     it.j0 = 1 + tj * S::R2;
     it.kb = 1 + kk * d.kdepth;
@@ -360,7 +372,11 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         // s+1.  Before the state of pass t >= 1 it waits until the passes
         // before are stored (the first stage of an item does not need it).
         if (lane == 0) {
-            const uint64_t pol_c = l2_policy(a.l2_keep_state ? -1 : 0);
+            // Coefficients make way for a state that stays in L2, but not
+            // before a neighbour along i has read the columns it shares
+            // (129x129x257, one tile: 22.6 -> 21.6 us a sweep; 250x129x257,
+            // two: 44.6 -> 54.0 if they did).
+            const uint64_t pol_c = l2_policy(a.l2_keep_state && (BATCH || d.nti == 1) ? -1 : 0);
             const uint64_t pol_keep = l2_policy(1);
             const uint64_t pol_p = l2_policy(a.l2_keep_state ? 1 : 0);
             uint32_t pc = 0, cc = 0;
@@ -388,14 +404,16 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 ++cc;
                 return true;
             };
-            // Items in the order of their numbers, whichever CTA is free: the
-            // first one by CTA number, then by ticket, and those of a last
-            // pass with a residual by CTA number again (a fixed assignment
-            // keeps the order of its sum).
+            // Items by CTA number in every pass (batched: in the order of
+            // their numbers, whichever CTA is free, by ticket).  The clock
+            // counts the ticks of all CTAs; one that takes part in fewer
+            // items or planes than others adds the rest when it is done.
             uint32_t ip = 0, entry = blockIdx.x, pass = 0;
-            bool by_ticket = a.taken > 0;
-            if (!by_ticket) entry += (uint32_t)(a.n_pass - 1) * nitems;
             const uint32_t total = (uint32_t)a.n_pass * nitems;
+            const uint32_t ticks = BATCH ? 0 : ((uint32_t)d.kdepth + 2 + S::TICK - 1) / S::TICK;   // of an item
+            const uint32_t rounds = (nitems + (uint32_t)G - 1) / (uint32_t)G;   // items of a CTA in a pass
+            uint32_t round = 0;
+            [[maybe_unused]] uint32_t clock = 0;      // as last read
             while (ok) {
                 const uint32_t qslot = ip % S::NQ;
                 if (ip >= S::NQ && !(ok = mbar_wait_bounded(&i_empty[qslot], ((ip / S::NQ) - 1) & 1))) break;
@@ -403,8 +421,8 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 mbar_arrive(&i_full[qslot]);
                 ++ip;
                 if (entry == S::END) break;
-                uint32_t next = 0;
-                if (by_ticket) next = (uint32_t)G + atomicAdd(&a.hdr->ticket, 1u);   // used after this item
+                [[maybe_unused]] uint32_t ticket = 0;
+                if constexpr (BATCH) ticket = (uint32_t)G + atomicAdd(&a.hdr->ticket, 1u);   // used after this item
                 const uint32_t t = entry / nitems;
                 Item2 it;
                 if constexpr (BATCH) {
@@ -425,16 +443,35 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 }
                 if (!(ok = put_state(it, 0) && put_state(it, 1))) break;
                 for (int q = 0; q < it.nout + 2 && ok; ++q) {
+                    if (!BATCH && q % S::TICK == 0) {
+                        // not far ahead of the average: rows and columns that
+                        // tiles share are then still in L2
+                        atomicAdd(&a.hdr->clock, 1u);
+                        const uint32_t mine = ((t * rounds + round) * ticks + q / S::TICK - S::LEAD) * (uint32_t)G;
+                        if ((int)(mine - clock) > 0) {
+                            const unsigned long long t0 = globaltimer_ns();
+                            do {
+                                clock = ld_relaxed_gpu(&a.hdr->clock);
+                            } while ((int)(mine - clock) > 0 && globaltimer_ns() - t0 < S::CLOCK_WAIT_NS);
+                        }
+                    }
                     ok = put_state(it, q + 2);
                     if (ok && q + 1 < it.nout + 2) ok = put_coef(it, q + 1);
                 }
-                if (by_ticket && next >= a.taken) {
-                    by_ticket = false;
-                    next = a.taken < total ? a.taken + blockIdx.x : S::END;
-                } else if (!by_ticket) {
-                    next = entry + (uint32_t)G < total ? entry + (uint32_t)G : S::END;
+                if constexpr (BATCH) {
+                    entry = ticket < total ? ticket : S::END;
+                } else {
+                    uint32_t rest = ticks - ((uint32_t)it.nout + 2 + S::TICK - 1) / S::TICK;
+                    ++round;
+                    if (entry - t * nitems + (uint32_t)G < nitems) {
+                        entry += (uint32_t)G;
+                    } else {
+                        rest += (rounds - round) * ticks;
+                        round = 0;
+                        entry = t + 1 < (uint32_t)a.n_pass ? (t + 1) * nitems + blockIdx.x : S::END;
+                    }
+                    if (rest > 0) atomicAdd(&a.hdr->clock, rest);
                 }
-                entry = next;
             }
             if (!ok) {
                 s_abort = 1;
@@ -888,6 +925,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 a.hdr->gbar = 0u;
                 a.hdr->counter = 0u;
                 a.hdr->ticket = 0u;
+                a.hdr->clock = 0u;
                 __threadfence();
             }
         }
@@ -941,14 +979,12 @@ int sweep2_kdepth(long cols, int nk, int ctas, long *steps = nullptr)
     return best;
 }
 
-// Steps of a pass over the grid (one tile of 1024 points, both sweeps, each)
-// and tiles along i.
-long sweep2_steps(const jac_grid *g, int *tiles_i)
+// Steps of a pass over the grid (one tile of 1024 points, both sweeps, each).
+long sweep2_steps(const jac_grid *g)
 {
     const long nti = sweep2_tiles_i(g->I), ntj = (g->J - 2 + Sweep2Shape::R2 - 1) / Sweep2Shape::R2;
     long steps = 0;
     sweep2_kdepth(nti * ntj, g->K - 2, device_sm_count(), &steps);
-    *tiles_i = (int)nti;
     return steps;
 }
 
@@ -1015,7 +1051,6 @@ jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStre
         a.n_pass = std::min(left, most);
         left -= a.n_pass;
         a.res = left == 0 ? res : nullptr;
-        a.taken = (unsigned)(a.res ? a.n_pass - 1 : a.n_pass) * (unsigned)a.nitems;
         cudaLaunchConfig_t cfg;
         std::memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3(nblocks);

@@ -76,12 +76,12 @@ def test_default_plan_takes_passes_where_the_state_leaves_l2():
     assert abs(g0 - g1) <= 1e-9 * abs(g1), (g0, g1)
 
 
-@pytest.mark.parametrize("dims,n", [((129, 129, 140), 16), ((257, 65, 70), 12), ((385, 40, 33), 21)])
+@pytest.mark.parametrize("dims,n", [((129, 129, 140), 16), ((257, 65, 70), 12), ((385, 40, 33), 21), ((300, 205, 61), 14)])
 def test_passes_by_ticket_are_repeatable_and_equal_single_sweeps(dims, n):
-    """Several passes with more items than CTAs, or with a shared pass barrier
-    over few items: which CTA takes an item differs from run to run, the state
-    and the residual do not.  Also the library's own choice on grids whose
-    state stays in L2."""
+    """Several passes with more items than CTAs (the last rounds of a pass and
+    of planes not full), or with a shared pass barrier over few items: which
+    CTA is ahead differs from run to run, the state and the residual do not.
+    Also the library's own choice on grids whose state stays in L2."""
     I, J, K = dims
     f = ji.himeno_fields(I, J, K, seed=800 + I + n)
     p1, g1 = gpu_run(f, n, "f32", SINGLE)
