@@ -318,10 +318,13 @@ __device__ __forceinline__ Item decode_item(const SweepArgs &a, const GridDesc *
     }
     const GridDesc *D = it.D;
     const int ntj = D->ntj, nti = D->nti;
-    const int tj = local % ntj;
-    const int r = local / ntj;
-    const int ti = r % nti;
-    const int kk = r / nti;
+    // i-neighbours first: tiles that share the state's columns and rows are
+    // worked on at about the same time (513x513x1025, items of 8 planes: BF16
+    // 1454 -> 1416 us a sweep, FP32 2320 -> 2215; one round of items: the same)
+    const int ti = local % nti;
+    const int r = local / nti;
+    const int tj = r % ntj;
+    const int kk = r / ntj;
     it.i0 = ti * D->ti;
     it.j0 = 1 + tj * D->rows;
     it.kb = 1 + kk * D->kdepth;
