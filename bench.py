@@ -146,13 +146,26 @@ def variant_roofline(prec: str, gpts: float) -> dict:
 SWEEP2_FILES = ("jac_sweep2.cu", "jac_sweep_kernel.cuh", "jac_common.cuh")
 
 
+def passes_pay(w, n):
+    """Whether a call of n FP32 sweeps without a plan takes two-sweep passes:
+    the rule of csrc/jac_sweep.cu (two_sweeps_pay), restated for a device with
+    152 SMs and 128 MiB of L2 to name the kernel and its bytes."""
+    I, J, K = w["I"], w["J"], w["K"]
+    cols = ((I - 2) // 128 + 1) * ((J - 2 + 7) // 8)
+    steps = min(-(-cols * -(-(K - 2) // kd) // GB300_SMS) * (kd + 4)
+                for kd in {max(2, -(-(K - 2) // b)) for b in range(1, K - 1)})
+    points = (I - 2) * (J - 2) * (K - 2)
+    kept = 2 * 4 * (-(-I // 4) * 4) * J * K <= 64 * 2**20
+    one = 2.0 + 7.1e-6 * points if kept else 8.5e-6 * points
+    rest = n % 4
+    return 4 * (n // 4) * 0.5 * 1.45 * steps + (11.0 + rest * one if rest else 0.0) < n * one
+
+
 def sweep_split(w, prec, n, fuse=0):
-    """(two-sweep passes, single sweeps) of a call of n sweeps under the
-    library's plan for this grid (fuse 0: the library's choice): an even
-    number of passes when the resolved plan takes them and n >= 4."""
-    from paper_2002_12115_gb300.binding import resolve_plan
-    f = resolve_plan(w["I"], w["J"], w["K"], prec, fuse=fuse)["fuse"]
-    if prec != "f32" or f != 2 or n < 4:
+    """(two-sweep passes, single sweeps) of a call of n sweeps: an even number
+    of passes where they are taken (fuse 2, or fuse 0 and the library's choice)
+    and n >= 4."""
+    if prec != "f32" or n < 4 or fuse == 1 or (fuse == 0 and not passes_pay(w, n)):
         return 0, n
     n_pass = (n // 2) & ~1
     return n_pass, n - 2 * n_pass
@@ -171,7 +184,8 @@ def sweep_roofline(w, prec, n, ms, fuse=0) -> dict:
     key = f"{w['I']}x{w['J']}x{w['K']} {prec}"
     if n_pass == 0:
         r = variant_roofline(prec, gpts)
-        r.update({"kernel": "k_sweep", "algorithmic_bytes_per_launch": BYTES_PER_POINT[prec] * npts * n})
+        r.update({"kernel": "k_sweep" if fuse else "k_sweep (k_resident where the grid fits in shared memory)",
+                  "algorithmic_bytes_per_launch": BYTES_PER_POINT[prec] * npts * n})
         per_sweep = profiled_traffic(key)
         traffic = per_sweep * n if per_sweep else None
     else:
@@ -186,9 +200,9 @@ def sweep_roofline(w, prec, n, ms, fuse=0) -> dict:
                                       "reading": "the rate single sweeps would reach at the full measured HBM "
                                                  "bandwidth (56 B per point-update)"},
              "reading": "a pass reads every array once per two point-updates; frac counts those bytes "
-                        "(28 B per point-update) against the copy peak, and the pass is bound by latency, "
-                        "not DRAM; the bandwidth fraction of single sweeps on the same grid (56 B per "
-                        "point-update) is compare." + prec + "_single_sweeps"}
+                        "(28 B per point-update) against the copy peak; above 1 the state and part of the "
+                        "coefficients stay in L2; the bandwidth fraction of single sweeps on the same grid "
+                        "(56 B per point-update) is compare." + prec + "_single_sweeps"}
         per_pass = profiled_traffic(key + " two-sweep pass", SWEEP2_FILES)
         traffic = per_pass * n_pass if (per_pass and rest == 0) else None
     r["traffic"] = traffic
@@ -668,9 +682,11 @@ def residual_vs_f64(w, dev, stream, sweeps):
 
 def bench_batch(args, stream, sweeps=100, steps=3, autotune=True, loops=True, tuner="cd", prec="f32",
                 n_grids=512):
-    """512 grids, dims drawn from {17, .., 129}: one graph-replayed persistent
-    launch per step against loops of per-grid launches.  The plan search runs
-    for FP32 storage; other precisions take the library's default plan.
+    """512 grids, dims drawn from {17, .., 129}: one graph launch per step
+    (without a plan the wide FP32 grids in two-sweep passes, then single sweeps)
+    against loops of per-grid launches.  The plan search runs for FP32 storage,
+    and its plan is used if it is faster than none; other precisions take the
+    library's default plan.
     n_grids < 512: the first n_grids of the same draw (a profiling subset)."""
     import torch
 
@@ -684,10 +700,21 @@ def bench_batch(args, stream, sweeps=100, steps=3, autotune=True, loops=True, tu
     plan = None
     if autotune and prec == "f32":
         from paper_2002_12115_gb300 import autotune as at
+
+        def ms_per_call():
+            b.sweep(sweeps, residuals=False)
+            return at.time_call(lambda: b.sweep(sweeps, residuals=False), 3, stream) * 1e3
+        default_ms = ms_per_call()
         if tuner == "ga":
             plan = at.ga_tune_batch(b, M=10, T=10, n_sweeps=10, reps=2)
         else:
             plan = at.tune_batch(b, n_sweeps=10, reps=2, passes=1)
+        # a plan asks for single sweeps; without one the wide grids sweep in passes
+        tuned_ms = ms_per_call()
+        if default_ms <= tuned_ms:
+            b.set_plan(0, None, None)
+        plan = {"plan": plan, "ms_per_step": tuned_ms, "default_ms_per_step": default_ms,
+                "used": "default" if default_ms <= tuned_ms else "plan"}
     b.sweep(sweeps)          # capture + warm-up
     b.sweep(sweeps)
     a, e = events()
@@ -700,7 +727,7 @@ def bench_batch(args, stream, sweeps=100, steps=3, autotune=True, loops=True, tu
     out = {"value": npts * sweeps / (ms * 1e-3) / 1e9, "unit": UNIT, "ms_per_step": ms,
            "grids": len(dims), "points": npts, "sweeps": sweeps,
            "gbs": BYTES_PER_POINT[prec] * npts * sweeps / (ms * 1e-3) / 1e9,
-           "launches_per_step": 1, "plan": plan, "info": b.info()}
+           "launches_per_step": 1, "plan_search": plan, "info": b.info()}
     if loops:
         for key, per_sweep, launches in (("per_grid_launches", False, len(dims)),
                                          ("per_grid_per_sweep_launches", True, len(dims) * sweeps)):
@@ -1034,11 +1061,11 @@ def run_native(args, w, wname):
                      "warmup": 2, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
                      "vs_baseline": None, "dtype": DTYPE[w["prec"]], "data": "synthetic",
                      "config": {"workload": f"{w['n_grids']} grids, dims drawn from {{17,33,49,65,97,129}}, {w['prec']}, 100 "
-                                            "sweeps per step in one graph-replayed persistent launch",
+                                            "sweeps per step in one graph launch",
                                 "l2": f"inputs larger than L2 ({BYTES_PER_POINT[w['prec']] * r['points'] / 1e9:.1f} GB "
                                       "of interior-point bytes swept per sweep)"},
                      "roofline": dict(variant_roofline(w["prec"], r["value"]), traffic=None,
-                                      kernel="k_sweep (batched)"),
+                                      kernel="k_sweep and k_sweep2 (batched)"),
                      "batch": r, "gpu_launches": args.steps})
     if wname == "tuners":
         r = bench_tuners(stream, sweeps=w["sweeps"])
@@ -1165,7 +1192,7 @@ def run_native(args, w, wname):
                     f"{'FP32' if f32_host else 'FP64'} arrays (the inputs of the {prec} problem), jac_sweep, "
                     f"jac_download_{'f32_' if f32_host else ''}async of the state and the residual, jac_sync; "
                     "two contexts on two streams take the steps in turn")},
-        "gpu_launches": args.steps * 15,
+        "gpu_launches": args.steps * (2 + sum(1 for q in sweep_split(w, prec, n, args.fuse) if q)),
         "clocks": s["clocks"],
         "residual": gosa,
         "compare": compare,
