@@ -106,10 +106,10 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-# FP64 operations (DADD, DMUL, DFMA, each one issue of the FP64 pipe) per
-# interior point of a non-residual FP64 sweep: 9 in the three b-brackets, 9
-# fused terms of s0, one fused and one plain product for ss, one fused update.
-F64_OPS_PER_POINT = 21
+# FP64 operations (DADD, DFMA, each one issue of the FP64 pipe) per interior
+# point of a non-residual FP64 sweep where bnd = 1: 5 for the three b-brackets
+# (the resident kernel: 9), 9 fused terms of s0, one for ss, one fused update.
+F64_OPS_PER_POINT = 16
 # GB300 issues two FP64 thread operations per SM per clock (the ncu peak of
 # sm__sass_thread_inst_executed_op_dfma_pred_on is 2 per SM per cycle).
 F64_OPS_PER_SM_CLK = 2

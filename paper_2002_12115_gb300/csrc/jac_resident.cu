@@ -172,13 +172,16 @@ template <typename T, typename C>
 __device__ __forceinline__ T res_ss(const T *P, int W, int Z, const PointCoef<T, C> &k, bool masked)
 {
     const T c = P[0], xp = P[1], xm = P[-1], yp = P[W], ym = P[-W], zp = P[Z], zm = P[-Z];
-    const T bij = ((P[W + 1] - P[-W + 1]) - P[W - 1]) + P[-W - 1];
-    const T bjk = ((P[Z + W] - P[-Z + W]) - P[Z - W]) + P[-Z - W];
-    const T bik = ((P[Z + 1] - P[-Z + 1]) - P[Z - 1]) + P[-Z - 1];
     if constexpr (sizeof(T) == 4) {
+        const T bij = ((P[W + 1] - P[-W + 1]) - P[W - 1]) + P[-W - 1];
+        const T bjk = ((P[Z + W] - P[-Z + W]) - P[Z - W]) + P[-Z - W];
+        const T bik = ((P[Z + 1] - P[-Z + 1]) - P[Z - 1]) + P[-Z - 1];
         return ss_f32<sizeof(C) == 2>(c, xp, xm, yp, ym, zp, zm, bij, bjk, bik, k.a0, k.a1, k.a2, k.a3, k.b0, k.b1,
                                       k.b2, k.c0, k.c1, k.c2, k.wk, k.bn);
     } else {
+        const T bij = (P[W + 1] - P[-W + 1]) - (P[W - 1] - P[-W - 1]);
+        const T bjk = (P[Z + W] - P[Z - W]) - (P[-Z + W] - P[-Z - W]);
+        const T bik = (P[Z + 1] - P[Z - 1]) - (P[-Z + 1] - P[-Z - 1]);
         T s0 = k.wk;
         s0 = fma(k.a0, xp, s0);
         s0 = fma(k.a1, yp, s0);

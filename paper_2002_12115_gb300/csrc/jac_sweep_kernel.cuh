@@ -224,9 +224,12 @@ struct SweepShape {
     static constexpr uint32_t C_TX = (uint32_t)(11 * TILE_C + TILE_T);
     static constexpr int C_STRIDE = (int)((C_TX + 127) / 128 * 128);
     static constexpr int BUDGET = (DEEP ? 226 : 220) * 1024;
-    static constexpr int RC_FIT = (BUDGET - RP * P_STRIDE - 1024) / C_STRIDE;
+    // FP64: a warp's differences along j (with a halo) and along i, two planes
+    static constexpr int D1 = TI + 2 * RW_MAX, D_PLANE = D1 + TI;
+    static constexpr int DIFF = sizeof(T) == 8 ? TJ * 2 * D_PLANE * (int)sizeof(T) : 0;   // bytes
+    static constexpr int RC_FIT = (BUDGET - RP * P_STRIDE - DIFF - 1024) / C_STRIDE;
     static constexpr int RC = RC_FIT > 8 ? 8 : RC_FIT;     // coefficient stages
-    static constexpr size_t SMEM = (size_t)RP * P_STRIDE + (size_t)RC * C_STRIDE + 128;
+    static constexpr size_t SMEM = (size_t)RP * P_STRIDE + (size_t)RC * C_STRIDE + DIFF + 128;
     static constexpr int THREADS = 32 * (TJ + 2);          // TJ consumers, state and coefficient producers
     static __host__ __device__ constexpr int tile_off(int q)
     {
@@ -245,6 +248,13 @@ __device__ __forceinline__ void lds_vec(const T *p, T (&v)[VI])
         const double2 x = *reinterpret_cast<const double2 *>(p);
         v[0] = x.x; v[1] = x.y;
     }
+}
+
+template <typename T, int VI>
+__device__ __forceinline__ void sts_vec(T *p, const T (&v)[VI])
+{
+    static_assert(sizeof(T) == 8 && VI == 2, "unsupported vector shape");
+    *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
 }
 
 // VI coefficient values of one lane from a shared-memory tile, as T.
@@ -535,6 +545,18 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
                 size_t off = ((size_t)it.kb * J + (size_t)j) * (size_t)pitch + (size_t)ib;
                 const int cidx = row * D->ti + VI * lin;        // element index in a coefficient tile
                 const int r0 = row * W, r1 = (row + 1) * W, r2 = (row + 2) * W;   // rows j-1, j, j+1
+                // FP64: the warp's differences, a segment's row of D1 followed by
+                // its left and right halo; the halo is formed by the lanes at a
+                // segment's ends where a point of the grid needs it
+                [[maybe_unused]] T *diff = reinterpret_cast<T *>(ring_c + (size_t)RC * S::C_STRIDE) +
+                                           (size_t)wy * 2 * S::D_PLANE;
+                [[maybe_unused]] const int dseg = rin * (VI * seg + 2), down = dseg + VI * lin;
+                [[maybe_unused]] const bool dhalo =
+                    (lin == 0 || lin == seg - 1) && (it.i0 > 0 || it.i0 + D->ti <= I - 1);
+                [[maybe_unused]] const int dhi = dseg + VI * seg + (lin == 0 ? 0 : 1);
+                [[maybe_unused]] const int dcol = lin == 0 ? H - 1 : H + VI * lin + VI;
+                [[maybe_unused]] const int dli = lin == 0 ? dseg + VI * seg : down - 1;
+                [[maybe_unused]] const int dri = lin == seg - 1 ? dseg + VI * seg + 1 : down + VI;
 
                 for (int m = 0; m < it.nout; ++m, off += plane) {
                     if (m == 0) {
@@ -554,15 +576,82 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
 
                     T ek0[VI + 2], ek1[VI + 2], ek2[VI + 2], em1[VI + 2], ep1[VI + 2];
                     T vm0[VI], vm2[VI], vp0[VI], vp2[VI];
-                    load_ext<T, VI, H>(Pk + r0, lin, seg, ek0);
-                    load_ext<T, VI, H>(Pk + r1, lin, seg, ek1);
-                    load_ext<T, VI, H>(Pk + r2, lin, seg, ek2);
-                    load_ext<T, VI, H>(Pm + r1, lin, seg, em1);
-                    load_ext<T, VI, H>(Pp + r1, lin, seg, ep1);
-                    lds_vec<T, VI>(Pm + r0 + H + VI * lin, vm0);
-                    lds_vec<T, VI>(Pm + r2 + H + VI * lin, vm2);
-                    lds_vec<T, VI>(Pp + r0 + H + VI * lin, vp0);
-                    lds_vec<T, VI>(Pp + r2 + H + VI * lin, vp2);
+                    [[maybe_unused]] T dij[VI], djk[VI], dik[VI];      // FP64: the three b brackets
+                    if constexpr (sizeof(T) == 4) {
+                        load_ext<T, VI, H>(Pk + r0, lin, seg, ek0);
+                        load_ext<T, VI, H>(Pk + r1, lin, seg, ek1);
+                        load_ext<T, VI, H>(Pk + r2, lin, seg, ek2);
+                        load_ext<T, VI, H>(Pm + r1, lin, seg, em1);
+                        load_ext<T, VI, H>(Pp + r1, lin, seg, ep1);
+                        lds_vec<T, VI>(Pm + r0 + H + VI * lin, vm0);
+                        lds_vec<T, VI>(Pm + r2 + H + VI * lin, vm2);
+                        lds_vec<T, VI>(Pp + r0 + H + VI * lin, vp0);
+                        lds_vec<T, VI>(Pp + r2 + H + VI * lin, vp2);
+                    } else {
+                        // Each bracket is a difference of two differences along
+                        // j (D1) or along i (D2) that neighbouring points and
+                        // planes share: bij = D1(i+1) - D1(i-1) in plane k,
+                        // bjk = D1(k+1) - D1(k-1), bik = D2(k+1) - D2(k-1).
+                        // Only plane k+1's are formed here; the others lie in
+                        // the warp's shared memory: 5 FP64 operations instead of
+                        // 9 (16 instead of 20 a point), and fewer state values
+                        // in registers.  The narrow FP64 pipe bounds this path:
+                        // 129x129x257 177.8 -> 149.7 us a sweep, 257x257x257
+                        // 674.9 -> 565.2, 200x150x100 152.6 -> 118.2, 65x65x129
+                        // 26.7 -> 22.9, against one coefficient stage less (3).
+                        // The error against 80-bit arithmetic is that of the
+                        // brackets summed left to right (rms ratio 0.99-1.00).
+                        load_ext<T, VI, H>(Pk + r1, lin, seg, ek1);
+                        T *dm = diff + (m & 1) * S::D_PLANE, *dk = diff + ((m + 1) & 1) * S::D_PLANE;
+                        auto d1_of = [&](const T *P, T *d, T(&u)[VI]) {
+                            T v[VI];
+                            lds_vec<T, VI>(P + r0 + H + VI * lin, u);
+                            lds_vec<T, VI>(P + r2 + H + VI * lin, v);
+#pragma unroll
+                            for (int e = 0; e < VI; ++e) u[e] = v[e] - u[e];
+                            sts_vec<T, VI>(d + down, u);
+                            if (dhalo) d[dhi] = P[r2 + dcol] - P[r0 + dcol];
+                        };
+                        auto d2_of = [&](const T(&x)[VI + 2], T *d, T(&u)[VI]) {
+#pragma unroll
+                            for (int e = 0; e < VI; ++e) u[e] = x[e + 2] - x[e];
+                            sts_vec<T, VI>(d + S::D1 + VI * lane, u);
+                        };
+                        if (m == 0) {
+                            T x[VI + 2], u[VI];
+                            load_ext<T, VI, H>(Pm + r1, lin, seg, x);
+                            d1_of(Pm, dm, u);
+                            d2_of(x, dm, u);
+                            d1_of(Pk, dk, u);
+                            d2_of(ek1, dk, u);
+                            __syncwarp();
+                        }
+                        T d1m[VI], d2m[VI], d1k[VI], d1p[VI], d2p[VI];
+                        load_ext<T, VI, H>(Pp + r1, lin, seg, ep1);
+                        lds_vec<T, VI>(dm + down, d1m);
+                        lds_vec<T, VI>(dm + S::D1 + VI * lane, d2m);
+                        lds_vec<T, VI>(dk + down, d1k);
+                        const T left = dk[dli], right = dk[dri];
+                        d1_of(Pp, dm, d1p);
+                        d2_of(ep1, dm, d2p);
+#pragma unroll
+                        for (int e = 0; e < VI; ++e) {
+                            dij[e] = (e == VI - 1 ? right : d1k[e + 1 < VI ? e + 1 : e]) -
+                                     (e == 0 ? left : d1k[e > 0 ? e - 1 : e]);
+                            djk[e] = d1p[e] - d1m[e];
+                            dik[e] = d2p[e] - d2m[e];
+                        }
+                        T v[VI];
+                        lds_vec<T, VI>(Pk + r0 + H + VI * lin, v);
+#pragma unroll
+                        for (int e = 0; e < VI; ++e) ek0[e + 1] = v[e];
+                        lds_vec<T, VI>(Pk + r2 + H + VI * lin, v);
+#pragma unroll
+                        for (int e = 0; e < VI; ++e) ek2[e + 1] = v[e];
+                        lds_vec<T, VI>(Pm + r1 + H + VI * lin, v);
+#pragma unroll
+                        for (int e = 0; e < VI; ++e) em1[e + 1] = v[e];
+                    }
 
                     T ca0[VI], ca1[VI], ca2[VI], ca3[VI], cb0[VI], cb1[VI], cb2[VI], cc0[VI], cc1[VI], cc2[VI],
                         cwk[VI], cbn[VI];
@@ -580,8 +669,8 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
                     smem_coef<T, C, VI>(cs + S::tile_off(JAC_BND), cidx, cbn);
 
                     // bnd is 1 at every point of most rows: there the multiply
-                    // by it changes nothing and is left out (one of 21 FP64
-                    // operations a point: 129x129x257 181.5 -> 178.9 us a sweep)
+                    // by it changes nothing and is left out (one of 17 FP64
+                    // operations a point)
                     bool masked = false;
                     if constexpr (sizeof(T) == 8) {
 #pragma unroll
@@ -594,9 +683,14 @@ k_sweep(const __grid_constant__ GridDesc d0, const SweepArgs a)
 #pragma unroll
                     for (int e = 0; e < VI; ++e) {
                         const T c = ek1[e + 1];
-                        const T bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
-                        const T bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
-                        const T bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
+                        T bij, bjk, bik;
+                        if constexpr (sizeof(T) == 4) {
+                            bij = ((ek2[e + 2] - ek0[e + 2]) - ek2[e]) + ek0[e];
+                            bjk = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
+                            bik = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
+                        } else {
+                            bij = dij[e]; bjk = djk[e]; bik = dik[e];
+                        }
                         T ss;
                         if constexpr (sizeof(T) == 4) {
                             // difference form with an exact a3*S - 1
