@@ -644,13 +644,33 @@ jac_status launch_adj(const AdjDesc &d, unsigned nblocks, cudaStream_t st)
 // one sub-partition and cap every thread at 96).  FP64: 8 rows of 64 points.
 constexpr int kAdjRowsF32 = 15, kAdjVIF32 = 2, kAdjRowsF64 = 8;
 
-// Output planes per item: 32, fewer while the grid has too few items to give
-// every SM two.
+// Output planes per item, at most 32 (48 to 128 measured the same or slower on
+// 513x513x1025): those with the least time of the CTA with the most to do.  An
+// item takes its planes plus 1.2 (its planes kb-1 and ke, with cross-plane
+// products only, and the ring's first fill); the last block of planes may be
+// shorter, and plane K-1 is a face.  The model's order is that of the measured
+// times, within 2%, on 10 grids of 33x33x65 to 257x257x513.  Against halving 32
+// until every SM has two items, us a sweep: 17x17x17 FP64 46.1 -> 17.7, 65x65x129
+// FP64 90.8 -> 85.0, 97x90x80 FP64 177 -> 153, 90x60x100 BF16 20.9 -> 15.4,
+// 200x150x120 FP32 82.5 -> 72.7, 257x257x513 FP32 536 -> 518; 513x513x257 FP32
+// 1045 -> 1052.
 int adj_kdepth(int K, long long tiles_ij, int sms)
 {
-    int kd = 32;
-    while (kd > 4 && tiles_ij * ((K + kd - 1) / kd) < 2LL * sms) kd /= 2;
-    return kd;
+    constexpr double extra = 1.2;
+    int best = 1;
+    double least = -1.0;
+    for (int kd = std::min(32, K); kd >= 1; --kd) {
+        const long long blocks = (K + kd - 1) / kd, items = tiles_ij * blocks;
+        const long long before = (items - 1) / sms;               // rounds before the last
+        const bool is_short = before * sms >= items - tiles_ij;   // the last round has last blocks only
+        const double last = is_short ? (double)(K - (blocks - 1) * kd - 1) + 0.5 * extra : kd + extra;
+        const double time = (double)before * (kd + extra) + last;
+        if (least < 0.0 || time < least) {
+            least = time;
+            best = kd;
+        }
+    }
+    return best;
 }
 
 // TJ consumer warps (tile rows) of VI points per lane.

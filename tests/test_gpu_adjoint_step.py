@@ -139,6 +139,20 @@ def test_kdepth_does_not_change_the_result():
             assert np.array_equal(got[k], ref[k]), (kd, k)
 
 
+@pytest.mark.parametrize("prec,dims", [("f64", (65, 65, 129)), ("f64", (33, 17, 3)), ("f32", (65, 60, 97)),
+                                       ("bf16", (90, 31, 100)), ("f32", (64, 16, 33))])
+def test_default_kdepth_gives_the_same_bits(prec, dims):
+    """The library's own depth (one round of items, several, a last block of
+    one plane) against items of 32 planes."""
+    I, J, K = dims
+    f = ji.himeno_fields(I, J, K, seed=41 + I)
+    target = ji.target_field(I, J, K)
+    ref, _ = one_step(f, prec, target, 32, coef_grads=True)
+    got, _ = one_step(f, prec, target, 0, coef_grads=True)
+    for k in ref:
+        assert np.array_equal(got[k], ref[k]), k
+
+
 def test_entry_point_rejects_bad_arguments():
     import torch
 
