@@ -8,8 +8,9 @@
 // Kernel design (2.5-D blocking, k-streaming, persistent, warp-specialised):
 //   * one cooperative launch runs all n sweeps of a call, one CTA per SM;
 //   * a work item is a tile of ti x rows points in (i, j) of one grid over
-//     `kdepth` consecutive k-planes.  Consumer warp w owns rows w*rw .. w*rw +
-//     rw-1 of the tile; each of its rw row segments has 32/rw lanes of VI
+//     `kdepth` consecutive k-planes, numbered along i, then j, then k.
+//     Consumer warp w owns rows w*rw .. w*rw + rw-1 of the tile; each of its
+//     rw row segments has 32/rw lanes of VI
 //     points (i-folding: narrow grids use narrow, tall tiles, so no lane
 //     idles on a 17-point row);  CTA b takes items b, b + G, b + 2G, ...;
 //   * warp TJ (one lane) issues the state-plane TMA copies -- the plane with
@@ -26,7 +27,8 @@
 //       ss = a3 * (sum_d coef_d (p_nb - p) + b-terms + wrk1) + p (a3 S - 1),
 //     with S = a0 + a1 + a2 + c0 + c1 + c2 summed exactly (Fast2Sum, or a
 //     plain sum for BF16 coefficients): algebraically the definition, without
-//     cancelling s0*a3 against p.  FP64 uses the written form with FMAs;
+//     cancelling s0*a3 against p.  FP64 uses the written form with FMAs and
+//     forms the b brackets from differences that points and planes share;
 //   * the last sweep sums each lane's squares of one step in FP32 and
 //     accumulates them in FP64; at every change of grid in a CTA's item list
 //     the consumer warps reduce (shuffles, compensated) into one partial per
