@@ -347,14 +347,24 @@ k_adjoint(const __grid_constant__ AdjDesc d)
             const int kind = (m < it.kb) ? 1 : (m >= it.ke ? 2 : 0);
             const uint32_t cs = cc;
             const int need = min(m + 1, it.m_hi) - it.m_lo + 1;
-            ok = mbar_wait_bounded(&c_full[cs % RC], (cs / RC) & 1);
-            while (ok && pw < need) {
-                const uint32_t q = pc + (uint32_t)pw;
-                ok = mbar_wait_bounded(&p_full[q % RP], (q / RP) & 1);
-                ++pw;
+            const bool gone = s_abort;
+            // The stage and the one plane that most steps wait for, tested
+            // together (200x150x120 FP32 72.4 -> 70.7 us a sweep, 90x60x100
+            // BF16 15.4 -> 14.8, 257x257x513 FP32 524 -> 519).
+            const uint32_t qn = pc + (uint32_t)(need - 1);
+            const bool got_c = mbar_try_wait(&c_full[cs % RC], (cs / RC) & 1);
+            const bool got_p = need - pw <= 1 && (need == pw || mbar_try_wait(&p_full[qn % RP], (qn / RP) & 1));
+            if (!__all_sync(0xffffffffu, got_c && got_p && !gone)) {
+                ok = !gone && mbar_wait_bounded(&c_full[cs % RC], (cs / RC) & 1);
+                while (ok && pw < need) {
+                    const uint32_t q = pc + (uint32_t)pw;
+                    ok = mbar_wait_bounded(&p_full[q % RP], (q / RP) & 1);
+                    ++pw;
+                }
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
             }
-            ok = __all_sync(0xffffffffu, ok && !s_abort);
-            if (!ok) break;
+            pw = need;
             const unsigned char *st = ring_s + (size_t)(cs % RC) * G::STAGE;
             const bool inK = (m >= 1) && (m <= K - 2);
 
