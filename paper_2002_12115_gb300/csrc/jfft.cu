@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(YZ ? 512 : 256, min_ctas_per_sm<T, YZ>()) k_ff
 // Sum of the n per-CTA energy partials of the last pass, in a fixed order:
 // thread t adds the partials t, t + 512, ... (four independent loads in
 // flight), then a pairwise tree over the 512 threads.  One CTA of 512
-// threads.
-__global__ void __launch_bounds__(512) k_fft_energy(const double *__restrict__ partials, int n, double *energy)
+// threads.  It may start while that pass still writes the partials, so the
+// pointer is not __restrict__ and they are read through L2, after the wait.
+__global__ void __launch_bounds__(512) k_fft_energy(const double *partials, int n, double *energy)
 {
     __shared__ double red[512];
     const int t = threadIdx.x;
@@ -455,10 +456,10 @@ __global__ void __launch_bounds__(512) k_fft_energy(const double *__restrict__ p
     wait_prior_grids();
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     for (int b = t; b < n; b += 4 * 512) {
-        s0 += partials[b];
-        if (b + 512 < n) s1 += partials[b + 512];
-        if (b + 1024 < n) s2 += partials[b + 1024];
-        if (b + 1536 < n) s3 += partials[b + 1536];
+        s0 += __ldcg(partials + b);
+        if (b + 512 < n) s1 += __ldcg(partials + b + 512);
+        if (b + 1024 < n) s2 += __ldcg(partials + b + 1024);
+        if (b + 1536 < n) s3 += __ldcg(partials + b + 1536);
     }
     red[t] = (s0 + s1) + (s2 + s3);
     __syncthreads();
