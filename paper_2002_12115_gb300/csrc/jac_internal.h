@@ -77,8 +77,9 @@ size_t sweep2_workspace_bytes(const jac_grid *g);
 // Steps of a two-sweep pass over the grid.
 long sweep2_steps(const jac_grid *g);
 // Two-sweep passes of a batch: descriptors (sweep2_desc_bytes each, built on
-// the host, used from device memory) and first items of its grids.  No
-// residual; n_pass even; pass t reads p[(t + par) & 1].
+// the host at any address, used from device memory at a multiple of 64) and
+// first items of its grids.  No residual; n_pass even; pass t reads
+// p[(t + par) & 1].
 size_t sweep2_desc_bytes();
 jac_status sweep2_batch_desc(void *desc, const jac_grid *g, int kdepth, int *items);
 jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids, int nitems, int n_pass, int par,

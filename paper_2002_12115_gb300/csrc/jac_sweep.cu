@@ -73,28 +73,17 @@ CUtensorMapDataType map_type(size_t elem)
                      : (elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
 }
 
-// 3-D tensor map of one storage-layout array with a (bx, by, 1) box.
-jac_status encode_map(CUtensorMap *m, const void *base, size_t elem, int pitch, int J, int K, int bx, int by)
-{
-    const cuuint64_t dims[3] = {(cuuint64_t)pitch, (cuuint64_t)J, (cuuint64_t)K};
-    const cuuint64_t strides[2] = {(cuuint64_t)pitch * elem, (cuuint64_t)pitch * J * elem};
-    const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    CUresult r = g_encode(m, map_type(elem), 3, const_cast<void *>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(JAC_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
-    return JAC_OK;
-}
-
 // SM count of the current device (148 if it cannot be queried).
 int num_sms() { return device_attr<int>(g_num_sms, cudaDevAttrMultiProcessorCount, 148); }
 
 }  // namespace
 
+// 3-D tensor map of one storage-layout array with a (bx, by, 1) box.  The
+// driver asks for a map at a multiple of 64.
 jac_status encode_box_map(CUtensorMap *m, const void *base, size_t elem, int extent_i, int pitch, int J, int K,
                           int bx, int by)
 {
+    if (reinterpret_cast<uintptr_t>(m) & 63) return fail(JAC_EINVAL, "a tensor map must lie at a multiple of 64");
     jac_status s = ensure_encode();
     if (s != JAC_OK) return s;
     const cuuint64_t dims[3] = {(cuuint64_t)extent_i, (cuuint64_t)J, (cuuint64_t)K};
@@ -321,11 +310,12 @@ jac_status build_desc(GridDesc *d, const jac_grid *g, const jac_plan &p, int ite
     d->p_buf[0] = g->p[0];
     d->p_buf[1] = g->p[1];
     for (int b = 0; b < 2; ++b)
-        if ((s = encode_map(&d->p[b], g->p[b], et, d->pitch, g->J, g->K, d->ti + 2 * H, d->rows + 2)) != JAC_OK)
+        if ((s = encode_box_map(&d->p[b], g->p[b], et, d->pitch, d->pitch, g->J, g->K, d->ti + 2 * H, d->rows + 2)) !=
+            JAC_OK)
             return s;
     for (int q = JAC_A0; q <= JAC_BND; ++q)
-        if ((s = encode_map(&d->coef[q - 1], g->coef[q], q == JAC_WRK1 ? et : ec, d->pitch, g->J, g->K, d->ti,
-                            d->rows)) != JAC_OK)
+        if ((s = encode_box_map(&d->coef[q - 1], g->coef[q], q == JAC_WRK1 ? et : ec, d->pitch, d->pitch, g->J, g->K,
+                                d->ti, d->rows)) != JAC_OK)
             return s;
     return JAC_OK;
 }

@@ -1106,10 +1106,12 @@ size_t sweep2_desc_bytes() { return sizeof(Sweep2Desc); }
 
 jac_status sweep2_batch_desc(void *desc, const jac_grid *g, int kdepth, int *items)
 {
-    Sweep2Desc *d = static_cast<Sweep2Desc *>(desc);
-    const jac_status s = build_desc2(d, g, kdepth);
-    if (s == JAC_OK) *items = d->nitems;
-    return s;
+    Sweep2Desc d;                  // tensor maps are encoded at multiples of 64; desc may lie anywhere
+    const jac_status s = build_desc2(&d, g, kdepth);
+    if (s != JAC_OK) return s;
+    std::memcpy(desc, &d, sizeof(d));
+    *items = d.nitems;
+    return JAC_OK;
 }
 
 jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids, int nitems, int n_pass, int par,
