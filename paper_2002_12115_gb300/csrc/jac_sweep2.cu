@@ -226,6 +226,10 @@ __device__ __forceinline__ void tmem_ld4(uint32_t addr, float (&a)[4])
                  : "r"(addr)
                  : "memory");
 }
+// Order this warp's tensor-memory accesses before a barrier that it arrives
+// at, and after one that it waited for.
+__device__ __forceinline__ void tmem_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Ties loaded values to the wait before it: no use of them moves above it.
@@ -640,6 +644,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                     ok = __all_sync(0xffffffffu, ok);
                 }
                 if (!ok) break;
+                if (do2) tmem_after_sync();                  // sweep 2 is done with the slot of plane s-3
                 const float *Pm = reinterpret_cast<const float *>(base + (size_t)((pc + s) % RP) * S::P_BYTES);
                 const float *Pk =
                     reinterpret_cast<const float *>(base + (size_t)((pc + s + 1) % RP) * S::P_BYTES);
@@ -721,7 +726,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 }
                 if (do2) {
                     tmem_wait_st();
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    tmem_before_sync();
                 }
                 __syncwarp();
                 if (lane == 0) {
@@ -800,7 +805,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1);
                 ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tmem_after_sync();
                 const float *Qm =
                     reinterpret_cast<const float *>(ring_q + (size_t)((qs - 3) % RQ) * S::Q_BYTES);
                 const float *Qk =
@@ -863,7 +868,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                     for (int e = 0; e < VI; ++e)
                         if (owned[e]) p_out[off + e] = out[e];
                 }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                tmem_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&q_empty[(qs - 3) % RQ]);   // intermediate plane s-3 done
             }
@@ -905,7 +910,10 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
     // and resets the workspace counters for the next launch.
     // If any CTA gave up a wait, the residual is written as NaN.
     __syncthreads();
-    if (warp == S::EDGE_WARP) tmem_dealloc(s_tmem, S::TM_COLS);
+    if (warp == S::EDGE_WARP) {
+        tmem_after_sync();
+        tmem_dealloc(s_tmem, S::TM_COLS);
+    }
     __shared__ int s_last;
     if (threadIdx.x == 0) {
         __threadfence();

@@ -27,3 +27,29 @@ def test_dependent_launches_read_coherently():
         # and every kernel waits for the launches before it
         kernels = re.findall(r"__global__.*?\n}", text, flags=re.S)
         assert kernels and all("wait_prior_grids()" in k for k in kernels), f
+
+
+AFTER, BEFORE = "tmem_after_sync();", "tmem_before_sync();"
+
+
+def test_tensor_memory_is_fenced_on_both_sides():
+    """Every hand-over of tensor memory through a barrier is fenced by the
+    warp that used it last and by the one that uses it next: sweep 1's stores
+    to sweep 2's loads, sweep 2's loads to the stores that reuse a slot, and
+    both to the deallocation."""
+    text = code("jac_sweep2.cu")
+    assert 'void tmem_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;"' in text
+    assert 'void tmem_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;"' in text
+    kernel = text[text.index("k_sweep2("):]
+    sweep1 = kernel[kernel.index("const bool got_q"):]
+    sweep2 = sweep1[sweep1.index("float *p_out;"):]
+    sweep1 = sweep1[:sweep1.index("float *p_out;")]
+    # sweep 1: the slot was read by sweep 2 before q_empty completed
+    assert AFTER in sweep1[:sweep1.index("tmem_st16(")]
+    assert BEFORE in sweep1[sweep1.index("tmem_wait_st()"):sweep1.index("mbar_arrive(&q_full")]
+    # sweep 2
+    assert AFTER in sweep2[:sweep2.index("tmem_ld16(")]
+    assert BEFORE in sweep2[sweep2.rindex("tmem_wait_ld()"):sweep2.index("mbar_arrive(&q_empty")]
+    # the deallocation, behind the CTA's last barrier
+    end = sweep2[sweep2.index("__syncthreads();"):]
+    assert AFTER in end[:end.index("tmem_dealloc(")]
