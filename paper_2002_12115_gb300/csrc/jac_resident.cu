@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
                     if (!got) s_abort = 1;
                 }
                 got = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
+                __syncwarp();                          // the other lanes' loads follow lane 0's acquire
                 if (got) {
                     const int vpr = W / TV, n = hnj * hnk * vpr;
                     const int drow = 32 / vpr, dcol = 32 - drow * vpr;

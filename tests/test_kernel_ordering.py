@@ -53,3 +53,13 @@ def test_tensor_memory_is_fenced_on_both_sides():
     # the deallocation, behind the CTA's last barrier
     end = sweep2[sweep2.index("__syncthreads();"):]
     assert AFTER in end[:end.index("tmem_dealloc(")]
+
+
+def test_resident_halo_loads_follow_the_flag():
+    """One lane of a communication warp acquires the neighbour's flag; the
+    shuffle that tells the others does not order memory, so a warp barrier
+    stands between it and their loads."""
+    text = code("jac_resident.cu")
+    wait = text[text.index("ld_acquire_gpu(nb_flag)"):]
+    wait = wait[wait.index("__shfl_sync("):]
+    assert "__syncwarp();" in wait[:wait.index("__ldcg(")]
