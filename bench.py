@@ -146,32 +146,16 @@ def variant_roofline(prec: str, gpts: float) -> dict:
 SWEEP2_FILES = ("jac_sweep2.cu", "jac_sweep_kernel.cuh", "jac_common.cuh")
 
 
-def passes_pay(w, n):
-    """Whether a call of n FP32 sweeps without a plan takes two-sweep passes:
-    the rule of csrc/jac_sweep.cu (two_sweeps_pay), restated for a device with
-    152 SMs and 128 MiB of L2 to name the kernel and its bytes."""
-    I, J, K = w["I"], w["J"], w["K"]
-    cols = ((I - 2) // 128 + 1) * ((J - 2 + 7) // 8)
-    steps = min(-(-cols * -(-(K - 2) // kd) // GB300_SMS) * (kd + 4)
-                for kd in {max(2, -(-(K - 2) // b)) for b in range(1, K - 1)})
-    points = (I - 2) * (J - 2) * (K - 2)
-    kept = 2 * 4 * (-(-I // 4) * 4) * J * K <= 64 * 2**20
-    one = 2.0 + 7.1e-6 * points if kept else 8.5e-6 * points
-    rest = n % 4
-    return 4 * (n // 4) * 0.5 * 1.45 * steps + (11.0 + rest * one if rest else 0.0) < n * one
+def sweep_route(w, prec, n, fuse=0, **tiles) -> dict:
+    """What a call of n sweeps runs with this plan, as the library says (on this
+    GPU; without one, on a GB300's 152 SMs)."""
+    import torch
+    from paper_2002_12115_gb300 import sweep_route as route
+    return route(w["I"], w["J"], w["K"], prec, n, sm_count=0 if torch.cuda.is_available() else GB300_SMS, fuse=fuse,
+                 **tiles)
 
 
-def sweep_split(w, prec, n, fuse=0):
-    """(two-sweep passes, single sweeps) of a call of n sweeps: an even number
-    of passes where they are taken (fuse 2, or fuse 0 and the library's choice)
-    and n >= 4."""
-    if prec != "f32" or n < 4 or fuse == 1 or (fuse == 0 and not passes_pay(w, n)):
-        return 0, n
-    n_pass = (n // 2) & ~1
-    return n_pass, n - 2 * n_pass
-
-
-def sweep_roofline(w, prec, n, ms, fuse=0) -> dict:
+def sweep_roofline(w, prec, n, ms, fuse=0, **tiles) -> dict:
     """Roofline of one call of n sweeps that took ms: HBM (FP32, BF16) or the
     FP64 ALU for single sweeps; for two-sweep passes HBM at the pass's own
     algorithmic bytes (every array read once and the state written once per
@@ -179,12 +163,13 @@ def sweep_roofline(w, prec, n, ms, fuse=0) -> dict:
     that single sweeps' 56 B per point-update put on the same bandwidth."""
     npts = n_interior(w)
     gpts = npts * n / (ms * 1e-3) / 1e9
-    n_pass, rest = sweep_split(w, prec, n, fuse)
+    route = sweep_route(w, prec, n, fuse, **tiles)
+    n_pass, rest = route["passes"], route["single_sweeps"]
     peak, kind = measured_peak()
     key = f"{w['I']}x{w['J']}x{w['K']} {prec}"
     if n_pass == 0:
         r = variant_roofline(prec, gpts)
-        r.update({"kernel": "k_sweep" if fuse else "k_sweep (k_resident where the grid fits in shared memory)",
+        r.update({"kernel": "k_resident" if route["resident_sweeps"] else "k_sweep",
                   "algorithmic_bytes_per_launch": BYTES_PER_POINT[prec] * npts * n})
         per_sweep = profiled_traffic(key)
         traffic = per_sweep * n if per_sweep else None
@@ -727,7 +712,7 @@ def bench_batch(args, stream, sweeps=100, steps=3, autotune=True, loops=True, tu
     out = {"value": npts * sweeps / (ms * 1e-3) / 1e9, "unit": UNIT, "ms_per_step": ms,
            "grids": len(dims), "points": npts, "sweeps": sweeps,
            "gbs": BYTES_PER_POINT[prec] * npts * sweeps / (ms * 1e-3) / 1e9,
-           "launches_per_step": 1, "plan_search": plan, "info": b.info()}
+           "launches_per_step": b.route(sweeps)["launches"], "plan_search": plan, "info": b.info()}
     if loops:
         for key, per_sweep, launches in (("per_grid_launches", False, len(dims)),
                                          ("per_grid_per_sweep_launches", True, len(dims) * sweeps)):
@@ -1066,7 +1051,7 @@ def run_native(args, w, wname):
                                       "of interior-point bytes swept per sweep)"},
                      "roofline": dict(variant_roofline(w["prec"], r["value"]), traffic=None,
                                       kernel="k_sweep and k_sweep2 (batched)"),
-                     "batch": r, "gpu_launches": args.steps})
+                     "batch": r, "gpu_launches": args.steps * r["launches_per_step"]})
     if wname == "tuners":
         r = bench_tuners(stream, sweeps=w["sweeps"])
         return emit({"metric": METRIC + " (512-grid batch under each launch-plan search)",
@@ -1129,7 +1114,7 @@ def run_native(args, w, wname):
         for vp in ("bf16", "f64", "f32"):
             if vp != prec:
                 compare[vp] = bench_variant(w, vp, s["dev"], stream, min(n, 30 if vp == "f64" else 200))
-        if sweep_split(w, prec, n, args.fuse)[0]:
+        if sweep_route(w, prec, n, args.fuse)["passes"]:
             # the same grid in single sweeps: the DRAM-bound kernel the passes replace
             compare[prec + "_single_sweeps"] = bench_variant(w, prec, s["dev"], stream, n, fuse=1)
         if prec != "f64":
@@ -1158,7 +1143,9 @@ def run_native(args, w, wname):
 
     # dram_achieved: the ncu bytes of the launch over its live time (below
     # the algorithmic figure when arrays stay in L2)
-    roofline = sweep_roofline(w, prec, n, s["launch_ms"], args.fuse)
+    tiles = {"tile_j": args.tile_j, "kdepth": args.kdepth, "tile_i": args.tile_i}
+    route = sweep_route(w, prec, n, args.fuse, **tiles)
+    roofline = sweep_roofline(w, prec, n, s["launch_ms"], args.fuse, **tiles)
     roofline.update({"launch_ms": s["launch_ms"], "sweeps_per_launch": n})
     cpu = parity = None
     if want_oracle:
@@ -1192,7 +1179,7 @@ def run_native(args, w, wname):
                     f"{'FP32' if f32_host else 'FP64'} arrays (the inputs of the {prec} problem), jac_sweep, "
                     f"jac_download_{'f32_' if f32_host else ''}async of the state and the residual, jac_sync; "
                     "two contexts on two streams take the steps in turn")},
-        "gpu_launches": args.steps * (2 + sum(1 for q in sweep_split(w, prec, n, args.fuse) if q)),
+        "gpu_launches": args.steps * (2 + route["launches"]),
         "clocks": s["clocks"],
         "residual": gosa,
         "compare": compare,

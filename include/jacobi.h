@@ -166,12 +166,29 @@ typedef struct jac_plan {
  * measurement otherwise (Section 4).
  * The plan a sweep of this grid would run with on a device of sm_count SMs
  * (one CTA per SM; sm_count <= 0: the current device's count): the zero
- * fields of *plan (NULL: all zero) filled in by the rules above.  (A call with
- * all zeros may choose another kernel, see jac_plan; the state is the same.)  Only the
- * dimensions and the precision of *g are read; no device memory is touched,
- * and with sm_count > 0 no GPU is needed.  Errors: JAC_EINVAL for bad
+ * fields of *plan (NULL: all zero) filled in by the rules above.  A call with
+ * all zeros may choose another kernel (jac_sweep_route says which); the state
+ * is the same.  Only the dimensions and the precision of *g are read; no
+ * device memory is touched, and with sm_count > 0 no GPU is needed.  Errors: JAC_EINVAL for bad
  * dimensions, precision or plan entries, or a shape the kernels lack. */
 jac_status jac_resolve_plan(const jac_grid *g, const jac_plan *plan, int sm_count, jac_plan *out);
+
+/* What a call of n sweeps runs. */
+typedef struct jac_route {
+    int launches;          /* kernel launches */
+    int resident_sweeps;   /* sweeps that run resident */
+    int passes;            /* two-sweep passes (two sweeps each) */
+    int single_sweeps;     /* single sweeps that stream */
+} jac_route;
+
+/* No paper counterpart.
+ * The kernels that jac_sweep_dev (with a workspace of jac_sweep_workspace_size
+ * bytes) and jac_sweep (without a tape) run for n_iter sweeps of this grid and
+ * plan (NULL: all zero) on a device of sm_count SMs (<= 0: the current
+ * device's).  Host only, reads and needs what jac_resolve_plan does; without a
+ * device the L2 counts as 128 MiB.  Errors: as for jac_resolve_plan, and
+ * JAC_EINVAL for n_iter < 0. */
+jac_status jac_sweep_route(const jac_grid *g, const jac_plan *plan, int n_iter, int sm_count, jac_route *out);
 
 /* Bytes of device workspace for jac_sweep_dev on this grid and plan (host
  * only).  It has room for every kernel the library may choose for a plan of
@@ -528,6 +545,13 @@ jac_status jac_batch_grid_plan(const jac_batch *b, int g, jac_plan *out);
  * If res_host is not NULL it receives the n residuals of the last sweep.
  * Synchronises.  JAC_ETIMEOUT if a bounded device wait gave up. */
 jac_status jac_batch_sweep(jac_batch *b, int n_iter, double *res_host);
+
+/* No paper counterpart.
+ * What jac_batch_sweep of n_iter sweeps runs with the present plan: the
+ * launches of its graph, the two-sweep passes of the wide grids (0: all grids
+ * sweep singly) and the last single sweeps, which all grids share.  Builds the
+ * device tables like the next sweep would. */
+jac_status jac_batch_route(jac_batch *b, int n_iter, jac_route *out);
 
 /* No paper counterpart (measurement contrast).
  * The same sweeps as a loop of per-grid launches, for comparison: one

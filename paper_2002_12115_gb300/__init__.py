@@ -14,7 +14,7 @@ include/jacobi.h, with hand-written sm_103a CUDA kernels.
 """
 from .binding import (FFT3, FIELDS, KDEPTH_BALANCED, PRECS, JacError, Jacobi, JacobiBatch, adjoint_step_dev, check,
                       ctx_workspace_size, fft_workspace_size, field_bytes, jac_fields, jac_grid, jac_plan, jac_ws_spec, lib, pack_dev,
-                      pitch, resolve_plan, stream_handle, sweep_dev, unpack_dev, workspace_check, workspace_size)
+                      pitch, resolve_plan, stream_handle, sweep_dev, sweep_route, unpack_dev, workspace_check, workspace_size)
 
 
 def __getattr__(name):
@@ -28,4 +28,4 @@ def __getattr__(name):
 __all__ = ["FFT3", "FIELDS", "KDEPTH_BALANCED", "PRECS", "JacError", "Jacobi", "JacobiBatch", "JacobiSweep",
            "adjoint_step_dev", "check", "ctx_workspace_size", "fft_workspace_size", "field_bytes", "jac_fields", "jac_grid", "jac_plan",
            "jac_ws_spec", "jacobi_sweep", "lib", "pack_dev", "pitch", "resolve_plan", "stream_handle", "sweep_dev",
-           "unpack_dev", "workspace_check", "workspace_size"]
+           "sweep_route", "unpack_dev", "workspace_check", "workspace_size"]

@@ -53,6 +53,14 @@ class jac_plan(ctypes.Structure):
                 ("fuse", ctypes.c_int)]
 
 
+class jac_route(ctypes.Structure):
+    _fields_ = [("launches", ctypes.c_int), ("resident_sweeps", ctypes.c_int), ("passes", ctypes.c_int),
+                ("single_sweeps", ctypes.c_int)]
+
+    def as_dict(self) -> dict:
+        return {name: getattr(self, name) for name, _ in self._fields_}
+
+
 class jac_ws_spec(ctypes.Structure):
     _fields_ = [("async_upload", ctypes.c_int), ("tape_C", ctypes.c_int), ("tape_max", ctypes.c_int)]
 
@@ -68,6 +76,7 @@ _SIG = {
                            ctypes.c_size_t, _VP]),
     "jac_workspace_check": (_I, [_VP, _VP]),
     "jac_resolve_plan": (_I, [ctypes.POINTER(jac_grid), ctypes.POINTER(jac_plan), _I, ctypes.POINTER(jac_plan)]),
+    "jac_sweep_route": (_I, [ctypes.POINTER(jac_grid), ctypes.POINTER(jac_plan), _I, _I, ctypes.POINTER(jac_route)]),
     "jac_sweep_dev_noalloc": (_I, [ctypes.POINTER(jac_grid), ctypes.POINTER(jac_plan), _I, _VP, _VP]),
     "jac_pack_dev": (_I, [_I, _I, _I, _I, _I, _VP, _VP, _VP]),
     "jac_unpack_dev": (_I, [_I, _I, _I, _I, _I, _VP, _VP, _VP]),
@@ -107,6 +116,7 @@ _SIG = {
     "jac_batch_upload_dev": (_I, [_VP, _I, ctypes.POINTER(jac_fields)]),
     "jac_batch_set_plan": (_I, [_VP, _I, _VP, _VP]),
     "jac_batch_grid_plan": (_I, [_VP, _I, ctypes.POINTER(jac_plan)]),
+    "jac_batch_route": (_I, [_VP, _I, ctypes.POINTER(jac_route)]),
     "jac_batch_sweep": (_I, [_VP, _I, _VP]),
     "jac_batch_sweep_loop": (_I, [_VP, _I, _I, _VP]),
     "jac_batch_download": (_I, [_VP, _I, _VP]),
@@ -470,6 +480,20 @@ def resolve_plan(I: int, J: int, K: int, prec: str = "f32", sm_count: int = 0, t
     return {"tile_j": out.tile_j, "kdepth": out.kdepth, "tile_i": out.tile_i, "fuse": out.fuse}
 
 
+def sweep_route(I: int, J: int, K: int, prec: str = "f32", n: int = 1, sm_count: int = 0, tile_j: int = 0,
+                kdepth: int = 0, tile_i: int = 0, fuse: int = 0) -> dict:
+    """What a call of n sweeps of an I x J x K grid runs on a device of sm_count
+    SMs (0: the current device): its launches, the sweeps that run resident, the
+    two-sweep passes and the single sweeps (jac_sweep_route)."""
+    g = jac_grid()
+    g.I, g.J, g.K, g.prec, g.omega = int(I), int(J), int(K), PRECS[prec], 0.8
+    out = jac_route()
+    check(lib().jac_sweep_route(ctypes.byref(g), ctypes.byref(jac_plan(int(tile_j), int(kdepth), int(tile_i),
+                                                                       int(fuse))), int(n), int(sm_count),
+                                ctypes.byref(out)))
+    return out.as_dict()
+
+
 def workspace_size(grid: jac_grid, tile_j: int = 0, kdepth: int = 0, tile_i: int = 0, fuse: int = 0) -> int:
     n = ctypes.c_size_t()
     check(lib().jac_sweep_workspace_size(ctypes.byref(grid), ctypes.byref(jac_plan(tile_j, kdepth, tile_i, fuse)),
@@ -581,8 +605,14 @@ class JacobiBatch:
         self._check(lib().jac_batch_grid_plan(self._h, int(g), ctypes.byref(p)))
         return (p.tile_i, p.tile_j, p.kdepth)
 
+    def route(self, n: int) -> dict:
+        """What sweep(n) runs with the present plan (jac_batch_route)."""
+        out = jac_route()
+        self._check(lib().jac_batch_route(self._h, int(n), ctypes.byref(out)))
+        return out.as_dict()
+
     def sweep(self, n: int, residuals: bool = True):
-        """n sweeps of every grid in one persistent launch (graph replay)."""
+        """n sweeps of every grid, one to three launches (graph replay)."""
         out = np.empty(self.n) if residuals else None
         self._check(lib().jac_batch_sweep(self._h, int(n), _VP(out.ctypes.data) if residuals else None))
         return out

@@ -259,6 +259,9 @@ jac::SweepArgs batch_args(const jac_batch *b, int n_iter)
     return a;
 }
 
+// Two-sweep passes of the wide grids in a call of n_iter sweeps.
+int passes_of(const jac_batch *b, int n_iter) { return b->passes.ngrids ? ((n_iter - 1) / 2) & ~1 : 0; }
+
 // The n_iter sweeps of every grid, on stream st.  With parts, all but the last
 // one to four sweeps run part by part (passes come in even numbers, so every
 // grid's state stays in the same buffer); the last ones, with the residuals,
@@ -266,7 +269,7 @@ jac::SweepArgs batch_args(const jac_batch *b, int n_iter)
 jac_status enqueue_sweeps(jac_batch *b, int n_iter, cudaStream_t st)
 {
     jac::SweepArgs a = batch_args(b, n_iter);
-    const int n_pass = b->passes.ngrids ? ((n_iter - 1) / 2) & ~1 : 0;
+    const int n_pass = passes_of(b, n_iter);
     if (n_pass > 0) {
         jac_status s = jac::sweep2_batch_run(b->passes.descs, b->passes.item_base, b->passes.ngrids, b->passes.nitems,
                                              n_pass, b->par, b->omega, b->ws, st);
@@ -524,6 +527,22 @@ jac_status jac_batch_info(const jac_batch *b, int *n_items, int *n_ctas, int *wa
     if (n_ctas) *n_ctas = b->tables_ok ? (int)b->nblocks : 0;
     if (warps) *warps = b->warps;
     if (sweeps) *sweeps = b->count;
+    return JAC_OK;
+}
+
+jac_status jac_batch_route(jac_batch *b, int n_iter, jac_route *out)
+{
+    if (!b || !out) return bfail(b, JAC_EINVAL, "NULL argument");
+    if (n_iter < 0) return bfail(b, JAC_EINVAL, "n_iter must be >= 0");
+    *out = jac_route();
+    if (n_iter == 0) return JAC_OK;
+    const jac_status s = build_tables(b);
+    if (s != JAC_OK) return s;
+    out->passes = passes_of(b, n_iter);
+    out->single_sweeps = n_iter - 2 * out->passes;
+    out->launches = 1;
+    if (out->passes > 0)
+        out->launches += jac::sweep2_batch_launches(b->passes.nitems, out->passes) + (b->singles.ngrids > 0);
     return JAC_OK;
 }
 

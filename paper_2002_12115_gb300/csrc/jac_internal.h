@@ -74,14 +74,17 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
 // Whether the library's plan for this grid takes two-sweep passes (fuse 0).
 bool two_sweep_default(const jac_grid *g);
 size_t sweep2_workspace_bytes(const jac_grid *g);
-// Steps of a two-sweep pass over the grid.
-long sweep2_steps(const jac_grid *g);
+// Steps of a two-sweep pass over the grid on `sms` SMs, and the launches that
+// n_pass of them take.
+long sweep2_steps(const jac_grid *g, int sms);
+int sweep2_launches(const jac_grid *g, int n_pass, int sms);
 // Two-sweep passes of a batch: descriptors (sweep2_desc_bytes each, built on
 // the host at any address, used from device memory at a multiple of 64) and
 // first items of its grids.  No residual; n_pass even; pass t reads
 // p[(t + par) & 1].
 size_t sweep2_desc_bytes();
 jac_status sweep2_batch_desc(void *desc, const jac_grid *g, int kdepth, int *items);
+int sweep2_batch_launches(int nitems, int n_pass);
 jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids, int nitems, int n_pass, int par,
                             double omega, void *workspace, cudaStream_t st);
 // Resident sweeps (jac_resident.cu): the boxes of a small grid, one per CTA,

@@ -209,6 +209,14 @@ int default_kdepth(long cols, int nk, int ctas, jac_prec prec)
 
 jac_plan resolve_plan(const jac_grid *g, const jac_plan *plan) { return resolve_plan_sms(g, plan, num_sms()); }
 
+// Half the L2 of the current device (of 128 MiB without one): a state that
+// takes more does not stay there between sweeps.
+static size_t half_l2()
+{
+    const size_t l2 = device_l2_bytes();
+    return (l2 > 1 ? l2 : (size_t)128 << 20) / 2;
+}
+
 // Whether the library's choice for a grid is two-sweep passes: FP32 storage
 // whose two state buffers do not stay in L2 (more than half of it; the L2
 // of the current device, or 128 MiB without one).  There the single sweep is
@@ -217,10 +225,7 @@ jac_plan resolve_plan(const jac_grid *g, const jac_plan *plan) { return resolve_
 bool two_sweep_default(const jac_grid *g)
 {
     if (g->prec != JAC_F32) return false;
-    size_t l2 = device_l2_bytes();
-    if (l2 <= 1) l2 = (size_t)128 << 20;
-    const size_t state = 2 * (size_t)jac_pitch(g->I) * (size_t)g->J * (size_t)g->K * 4;
-    return state > l2 / 2;
+    return 2 * (size_t)jac_pitch(g->I) * (size_t)g->J * (size_t)g->K * 4 > half_l2();
 }
 
 // The plan of a grid for a device of `sms` SMs (one CTA per SM).
@@ -440,11 +445,14 @@ size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
 // precisions) a resident sweep takes 0.54-0.82 of a streaming one and the
 // launch up to 6 us more (the copy of the coefficients), so it pays from the
 // third sweep on; one or two sweeps stay with the streaming kernel.
+static bool resident_pays(const jac_grid *g, const jac_plan *plan, int n_iter, int sms, ResidentShape *r)
+{
+    return n_iter >= 3 && all_zero(plan) && resident_shape(g->I, g->J, g->K, g->prec, sms, r);
+}
+
 bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r)
 {
-    if (n_iter < 3) return false;
-    if (!all_zero(plan)) return false;
-    return resident_shape(g->I, g->J, g->K, g->prec, num_sms(), r) && ws_bytes >= resident_workspace_bytes(*r);
+    return resident_pays(g, plan, n_iter, num_sms(), r) && ws_bytes >= resident_workspace_bytes(*r);
 }
 
 // Whether a call of n_iter sweeps with the library's own plan (all zero) takes
@@ -457,24 +465,28 @@ bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws
 // us a sweep against 21.5 in passes, 161x161x161 (two tiles 62% full) 29.3
 // against 35.2, 300x205x399 (three tiles 78% full) 207 against 182.  The
 // single sweeps after the passes are a launch of their own (11 us).
-static bool two_sweeps_pay(const jac_grid *g, int n_iter)
+static bool two_sweeps_pay(const jac_grid *g, int n_iter, int sms)
 {
     if (g->prec != JAC_F32 || n_iter < 4) return false;
-    const double state = 2.0 * (double)jac_pitch(g->I) * g->J * g->K * 4.0;
-    const bool kept = state <= 0.5 * (double)device_l2_bytes();
+    const bool kept = !two_sweep_default(g);
     const double points = (double)(g->I - 2) * (g->J - 2) * (g->K - 2);
-    const double two = 0.5 * 1.45 * (double)sweep2_steps(g);   // us a sweep
+    const double two = 0.5 * 1.45 * (double)sweep2_steps(g, sms);   // us a sweep
     const double one = kept ? 2.0 + 7.1e-6 * points : 8.5e-6 * points;
     const int in_passes = 4 * (n_iter / 4), rest = n_iter - in_passes;
     return in_passes * two + (rest ? 11.0 + rest * one : 0.0) < n_iter * one;
 }
 
-// Whether a call of n_iter sweeps runs as two-sweep passes.
-bool use_two_sweep_passes(const jac_grid *g, const jac_plan &p, int n_iter)
+// Whether a call of n_iter sweeps runs as two-sweep passes; p is the resolved
+// plan, whose fuse the library's own plan (all zero) leaves to two_sweeps_pay.
+static bool use_two_sweep_passes(const jac_grid *g, const jac_plan *plan, const jac_plan &p, int n_iter, int sms)
 {
-    if (g->prec != JAC_F32 || p.fuse == 1 || n_iter < 4) return false;
-    return p.fuse == 2;
+    if (g->prec != JAC_F32 || n_iter < 4) return false;
+    return all_zero(plan) ? two_sweeps_pay(g, n_iter, sms) : p.fuse == 2;
 }
+
+// Passes of such a call: an even number keeps the state of n sweeps in
+// p[n % 2]; the remaining 0..3 sweeps run singly.
+static int passes_of(int n_iter) { return (n_iter / 2) & ~1; }
 
 jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double *d_residual, void *workspace,
                      size_t ws_bytes, void *stream, const LaunchOpts *opts)
@@ -485,25 +497,21 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     if (s != JAC_OK) return s;
     if (n_iter < 0) return fail(JAC_EINVAL, "n_iter must be >= 0");
     if (n_iter == 0) return JAC_OK;
-    jac_plan p = resolve_plan(g, plan);
+    const jac_plan p = resolve_plan(g, plan);
     int rw = 0, tj = 0;
     if ((s = check_plan(g->prec, p, &rw, &tj)) != JAC_OK) return s;
     if (p.fuse < 0 || p.fuse > 2) return fail(JAC_EINVAL, "fuse must be 0, 1 or 2");
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15)) return fail(JAC_EINVAL, "bad workspace");
     const size_t need = sweep_workspace_bytes(g, p);
     if (ws_bytes < need) return fail(JAC_EINVAL, "workspace too small: need " + std::to_string(need) + " bytes");
-    if (all_zero(plan) && g->prec == JAC_F32)
-        p.fuse = two_sweeps_pay(g, n_iter) && ws_bytes >= sweep2_workspace_bytes(g) ? 2 : 1;
     ResidentShape shape;
     if (!injected && use_resident(g, plan, n_iter, ws_bytes, &shape)) {
         double *res = no_res ? nullptr : (d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual);
         return resident_run(g, shape, n_iter, res, workspace, static_cast<cudaStream_t>(stream));
     }
-    if (!injected && use_two_sweep_passes(g, p, n_iter)) {
-        // an even number of passes keeps the state of n sweeps in p[n % 2];
-        // the remaining 0..3 sweeps run singly and give the residual if any
-        const int n_pass = (n_iter / 2) & ~1;
-        const int rest = n_iter - 2 * n_pass;
+    if (!injected && use_two_sweep_passes(g, plan, p, n_iter, num_sms()) && ws_bytes >= sweep2_workspace_bytes(g)) {
+        const int n_pass = passes_of(n_iter);
+        const int rest = n_iter - 2 * n_pass;          // the residual is theirs, if any
         double *res2 = nullptr;
         if (rest == 0 && !no_res) res2 = d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual;
         if ((s = sweep2_run(g, 0, n_pass, res2, workspace, ws_bytes, static_cast<cudaStream_t>(stream))) != JAC_OK)
@@ -603,6 +611,30 @@ jac_status jac_resolve_plan(const jac_grid *g, const jac_plan *plan, int sm_coun
     jac_status s = jac::check_plan(g->prec, p, &rw, &tj);
     if (s != JAC_OK) return s;
     *out = p;
+    return JAC_OK;
+}
+
+jac_status jac_sweep_route(const jac_grid *g, const jac_plan *plan, int n_iter, int sm_count, jac_route *out)
+{
+    if (!out) return jac::fail(JAC_EINVAL, "NULL argument");
+    if (n_iter < 0) return jac::fail(JAC_EINVAL, "n_iter must be >= 0");
+    jac_plan p;
+    const jac_status s = jac_resolve_plan(g, plan, sm_count, &p);
+    if (s != JAC_OK) return s;
+    const int sms = sm_count > 0 ? sm_count : jac::device_sm_count();
+    *out = jac_route();
+    jac::ResidentShape shape;
+    if (jac::resident_pays(g, plan, n_iter, sms, &shape)) {
+        out->resident_sweeps = n_iter;
+        out->launches = 1;
+        return JAC_OK;
+    }
+    if (jac::use_two_sweep_passes(g, plan, p, n_iter, sms)) {
+        out->passes = jac::passes_of(n_iter);
+        out->launches = jac::sweep2_launches(g, out->passes, sms);
+    }
+    out->single_sweeps = n_iter - 2 * out->passes;
+    out->launches += out->single_sweeps > 0;
     return JAC_OK;
 }
 

@@ -988,12 +988,31 @@ int sweep2_kdepth(long cols, int nk, int ctas, long *steps = nullptr)
 }
 
 // Steps of a pass over the grid (one tile of 1024 points, both sweeps, each).
-long sweep2_steps(const jac_grid *g)
+long sweep2_steps(const jac_grid *g, int sms)
 {
     const long nti = sweep2_tiles_i(g->I), ntj = (g->J - 2 + Sweep2Shape::R2 - 1) / Sweep2Shape::R2;
     long steps = 0;
-    sweep2_kdepth(nti * ntj, g->K - 2, device_sm_count(), &steps);
+    sweep2_kdepth(nti * ntj, g->K - 2, sms, &steps);
     return steps;
+}
+
+// Passes of `nitems` items that one launch can count in 32 bits (even).
+static int passes_per_launch(long long nitems)
+{
+    return (int)std::min<long long>(0x7ffffffe, (0xffff0000ll / (nitems * Sweep2Shape::R2)) & ~1ll);
+}
+
+int sweep2_batch_launches(int nitems, int n_pass)
+{
+    const int most = std::max(2, passes_per_launch(nitems));
+    return n_pass / most + (n_pass % most != 0);
+}
+
+int sweep2_launches(const jac_grid *g, int n_pass, int sms)
+{
+    const long cols = (long)sweep2_tiles_i(g->I) * ((g->J - 2 + Sweep2Shape::R2 - 1) / Sweep2Shape::R2);
+    const int kd = sweep2_kdepth(cols, g->K - 2, sms);
+    return sweep2_batch_launches((int)(cols * ((g->K - 2 + kd - 1) / kd)), n_pass);
 }
 
 size_t sweep2_workspace_bytes(const jac_grid *g)
@@ -1052,7 +1071,7 @@ jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStre
     });
     if (attr_err != cudaSuccess)
         return fail2(JAC_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(attr_err));
-    const int most = (int)std::min<long long>(0x7ffffffe, (0xffff0000ll / ((long long)a.nitems * S::R2)) & ~1ll);
+    const int most = passes_per_launch(a.nitems);
     if (most < 2 && a.n_pass > most) return fail2(JAC_EINVAL, "grid too large for the two-sweep launch shape");
     double *const res = a.res;
     for (int left = a.n_pass; left > 0;) {

@@ -217,6 +217,11 @@ def test_two_sweep_passes_of_a_batch(n):
                 b.upload_tensors(k, f)
             if how == "plan":
                 b.set_plan(8)
+            # 17 of the 22 grids are wide: all but the last one to four sweeps in passes
+            r = b.route(n)
+            wide = (n - 1) // 4 * 2 if how != "plan" else 0
+            assert r["passes"] == wide and r["single_sweeps"] == n - 2 * wide
+            assert r["launches"] == (3 if wide else 1)
             sweep = b.sweep_loop if how == "loop" else b.sweep
             res = [sweep(n), sweep(n + 3)]
             got.append((res, [b.download_tensor(k) for k in range(len(dims))]))

@@ -38,7 +38,11 @@ def _built():
 def test_equals_streaming(dims, prec):
     I, J, K = dims
     f = ji.himeno_fields(I, J, K, seed=900 + I + J + K)
+    from paper_2002_12115_gb300 import sweep_route
+    fits = prec != "f64" or dims not in ((77, 53, 101), (65, 65, 129))     # else streaming both times
     for n in (3, 8):
+        assert sweep_route(I, J, K, prec, n)["resident_sweeps"] == (n if fits else 0)
+        assert sweep_route(I, J, K, prec, n, fuse=1)["single_sweeps"] == n
         p1, g1 = gpu_run(f, n, prec, STREAM)
         p2, g2 = gpu_run(f, n, prec)
         assert np.array_equal(p1, p2), float(np.abs(p1 - p2).max())

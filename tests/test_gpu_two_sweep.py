@@ -44,6 +44,9 @@ def _built():
 def test_pairs_equal_single_sweeps(dims, n):
     I, J, K = dims
     f = ji.himeno_fields(I, J, K, seed=700 + I + J + K)
+    from paper_2002_12115_gb300 import sweep_route
+    assert sweep_route(I, J, K, "f32", n, fuse=2)["passes"] == n // 4 * 2
+    assert sweep_route(I, J, K, "f32", n, fuse=1)["passes"] == 0
     p1, g1 = gpu_run(f, n, "f32", SINGLE)
     p2, g2 = gpu_run(f, n, "f32", PAIRS)
     assert np.array_equal(p1, p2), float(np.abs(p1 - p2).max())
