@@ -26,8 +26,10 @@ size_t sweep_workspace_bytes(const jac_grid *g, const jac_plan &p);
 size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p);
 // Launch options of the single-grid sweep.  wait_ns and gbar_extra are set
 // only by a test of the failure path: a shorter limit for the waits on other
-// warps and CTAs, and an offset that makes the grid barrier between sweeps
-// unreachable.  Either one set runs single sweeps (no two-sweep passes).
+// warps and CTAs, and an offset that makes the launch's grid barrier
+// unreachable.  They do not change the kernel, except that a grid of one
+// resident box, which waits for nobody, streams, and that passes become
+// single sweeps.
 // no_residual: nobody reads this launch's residual, so none is summed.
 struct LaunchOpts {
     unsigned long long wait_ns = 0;
@@ -100,9 +102,10 @@ bool resident_shape(int I, int J, int K, jac_prec prec, int sms, ResidentShape *
 size_t resident_workspace_bytes(const ResidentShape &s);
 // d_residual NULL: no residual is summed.  hist not NULL: state t + 1 goes
 // whole to hist + t * hist_stride (bytes; faces and padding already there)
-// and p[1] is not used.
+// and p[1] is not used.  opts: only its wait_ns and gbar_extra are read.
 jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, double *d_residual, void *workspace,
-                        cudaStream_t st, void *hist = nullptr, size_t hist_stride = 0);
+                        cudaStream_t st, void *hist = nullptr, size_t hist_stride = 0,
+                        const LaunchOpts *opts = nullptr);
 // Whether a call of n_iter sweeps with this plan and workspace runs resident.
 bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r);
 jac_status adjoint_step_dev(const jac_grid *g, const void *p_t, const void *lam_in, void *lam_out, double *g_wrk1,

@@ -71,6 +71,9 @@ struct ResArgs {
     char *hist;                // not NULL: state t + 1 whole at hist + t * hist_stride
     size_t hist_stride;        // instead of in p_buf[(t + 1) & 1]
     WsHeader *hdr;
+    unsigned long long wait_ns;   // limit of every wait on another CTA
+    unsigned gbar_extra;       // added to the barrier's target: 0, except when a test of the failure path
+                               // makes it unreachable
 };
 
 // Boxes split n rows into parts of nearly equal length.
@@ -324,11 +327,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(const __grid_constant_
             if (has_nb) {
                 bool got = true;
                 if (lane == 0) {
-                    if (t == 0) got = wait_counter_bounded(&a.hdr->gbar, (unsigned)G);
+                    if (t == 0) got = wait_counter_bounded(&a.hdr->gbar, (unsigned)G + a.gbar_extra, a.wait_ns);
                     if (got && ld_acquire_gpu(nb_flag) < (unsigned)(t + 1)) {
                         const unsigned long long t0 = globaltimer_ns();
                         while (ld_acquire_gpu(nb_flag) < (unsigned)(t + 1))
-                            if (globaltimer_ns() - t0 > kWaitLimitNs) { got = false; break; }
+                            if (globaltimer_ns() - t0 > a.wait_ns) { got = false; break; }
                     }
                     if (!got) s_abort = 1;
                 }
@@ -499,7 +502,7 @@ size_t resident_workspace_bytes(const ResidentShape &s)
 }
 
 jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, double *d_residual, void *workspace,
-                        cudaStream_t st, void *hist, size_t hist_stride)
+                        cudaStream_t st, void *hist, size_t hist_stride, const LaunchOpts *opts)
 {
     const unsigned ctas = (unsigned)(s.nj * s.nk);
     ResArgs a;
@@ -523,6 +526,8 @@ jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, d
     a.res = d_residual;
     a.hist = static_cast<char *>(hist);
     a.hist_stride = hist_stride;
+    a.wait_ns = opts && opts->wait_ns ? opts->wait_ns : kWaitLimitNs;
+    a.gbar_extra = opts ? opts->gbar_extra : 0;
     switch (g->prec) {
     case JAC_F64: return launch_resident<double, double>(a, ctas, s.smem, st);
     case JAC_F32: return launch_resident<float, float>(a, ctas, s.smem, st);

@@ -505,9 +505,9 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     const size_t need = sweep_workspace_bytes(g, p);
     if (ws_bytes < need) return fail(JAC_EINVAL, "workspace too small: need " + std::to_string(need) + " bytes");
     ResidentShape shape;
-    if (!injected && use_resident(g, plan, n_iter, ws_bytes, &shape)) {
+    if (use_resident(g, plan, n_iter, ws_bytes, &shape) && !(injected && shape.nj * shape.nk == 1)) {
         double *res = no_res ? nullptr : (d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual);
-        return resident_run(g, shape, n_iter, res, workspace, static_cast<cudaStream_t>(stream));
+        return resident_run(g, shape, n_iter, res, workspace, static_cast<cudaStream_t>(stream), nullptr, 0, opts);
     }
     if (!injected && use_two_sweep_passes(g, plan, p, n_iter, num_sms()) && ws_bytes >= sweep2_workspace_bytes(g)) {
         const int n_pass = passes_of(n_iter);

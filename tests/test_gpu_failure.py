@@ -79,3 +79,53 @@ def test_single_sweep_launch_has_no_barrier_to_stall(pkg):
         p = jac.download()
     op, og = oracle_ref(f, 1, "f32")
     assert rel_p(p, op) <= TOL["f32"] and rel_g(g, og) <= TOL["f32"]
+
+
+def stall_and_recover(pkg, prec, dims, n, plan=None):
+    """One stalled call (JAC_ETIMEOUT, a NaN residual, a partly swept state),
+    then normal ones on the same context: bitwise the state of a context that
+    was never stalled.  Returns the stalled call's state."""
+    I, J, K = dims
+    f = ji.himeno_fields(I, J, K, seed=400 + I)
+    with pkg.Jacobi(I, J, K, prec) as jac:
+        if plan is not None:
+            jac.set_plan(*plan)
+        jac.upload(f)
+        jac.inject_stall(WAIT_NS)
+        jac.sweep(n)
+        stalled, res = np.zeros((K, J, I)), np.zeros(1)
+        jac.download_async(stalled, res)
+        with pytest.raises(pkg.JacError) as err:
+            jac.sync()
+        assert err.value.status == 5 and np.isnan(res[0])
+        got = []
+        for m in (n, n + 1):                              # the header is left as the next launch needs it
+            jac.upload(f)
+            jac.sweep(m)
+            got.append((jac.download(), jac.residual()))
+    with pkg.Jacobi(I, J, K, prec) as jac:
+        if plan is not None:
+            jac.set_plan(*plan)
+        for m, (p, g) in zip((n, n + 1), got):
+            jac.upload(f)
+            jac.sweep(m)
+            assert np.array_equal(jac.download(), p) and jac.residual() == g
+    return f, stalled
+
+
+@pytest.mark.parametrize("prec,dims", [("f32", (77, 53, 101)), ("bf16", (61, 40, 50)), ("f64", (33, 33, 65))])
+def test_resident_waits_run_out(pkg, prec, dims):
+    """The resident kernel's waits: no box sees the barrier, so none gets past
+    its first exchange.  Of its first sweep a box has stored the rows next to
+    other boxes by then and no inner row (the streaming kernel stores all)."""
+    n = 5                                                 # state n is in the buffer of state 1
+    assert pkg.sweep_route(*dims, prec, n)["resident_sweeps"] == n
+    f, stalled = stall_and_recover(pkg, prec, dims, n)
+    with pkg.Jacobi(*dims, prec) as jac:
+        jac.upload(f)
+        p0 = jac.download()
+        jac.sweep(1)
+        p1 = jac.download()
+    inside = (slice(1, -1),) * 3
+    swept, kept = np.all(stalled == p1, axis=2)[inside[:2]], np.all(stalled == p0, axis=2)[inside[:2]]
+    assert np.all(swept | kept) and swept.any() and kept.any()
