@@ -431,10 +431,10 @@ jac_status jac_sync(jac_ctx *ctx);
 /* Failure-path test aid (host-side injection; the paper has no counterpart:
  * its offload search gives up on a measurement after a time limit, Section
  * 5.1.2, and this library's kernels likewise give up their device waits).
- * The next sweep launch of this context, of whichever kernel, is made with a
- * grid-barrier target that no CTA ever reaches, and with wait_ns nanoseconds
- * as the limit of every wait on other warps and CTAs (wait_ns = 0 cancels; at
- * most 2 s).  A launch of at least two sweeps then gives up its waits,
+ * The launches of this context's next sweep call (with a tape: of its first
+ * segment), of whichever kernel, are made with grid-barrier targets that no
+ * CTA ever reaches, and with wait_ns nanoseconds as the limit of every wait on
+ * other warps and CTAs (wait_ns = 0 cancels; at most 2 s).  A launch of at least two sweeps then gives up its waits,
  * every CTA drains its own copies and exits, the workspace error word is
  * set and the residual of the launch is NaN: jac_residual, jac_sync and
  * jac_download report JAC_ETIMEOUT and clear the word.  The state of that

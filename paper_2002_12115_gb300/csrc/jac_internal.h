@@ -28,8 +28,7 @@ size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p);
 // only by a test of the failure path: a shorter limit for the waits on other
 // warps and CTAs, and an offset that makes the launch's grid barrier
 // unreachable.  They do not change the kernel, except that a grid of one
-// resident box, which waits for nobody, streams, and that passes become
-// single sweeps.
+// resident box, which waits for nobody, streams.
 // no_residual: nobody reads this launch's residual, so none is summed.
 struct LaunchOpts {
     unsigned long long wait_ns = 0;
@@ -66,13 +65,13 @@ template <bool BATCH>
 jac_status launch_sweep(jac_prec prec, int tj, const GridDesc &d0, const SweepArgs &a, unsigned nblocks,
                         cudaStream_t st);
 // Two-sweep passes (FP32 storage): n_pass passes of two sweeps each, in one
-// cooperative launch (very long calls: several); the residual of the last
-// sweep to d_residual (NULL: none).  kdepth 0: the default depth.
-// Two-sweep passes (FP32 storage): pass t reads p[t & 1] and writes the other
-// buffer.  mid (one-pass calls only) also receives the state after the first
-// sweep at every interior point; its faces are left as they are.
+// cooperative launch (very long calls: several); pass t reads p[t & 1] and
+// writes the other buffer.  The residual of the last sweep goes to d_residual
+// (NULL: none).  kdepth 0: the default depth.  mid (one-pass calls only) also
+// receives the state after the first sweep at every interior point; its faces
+// are left as they are.  opts: only its wait_ns and gbar_extra are read.
 jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_residual, void *workspace,
-                      size_t ws_bytes, cudaStream_t st, void *mid = nullptr);
+                      size_t ws_bytes, cudaStream_t st, void *mid = nullptr, const LaunchOpts *opts = nullptr);
 // Whether the library's plan for this grid takes two-sweep passes (fuse 0).
 bool two_sweep_default(const jac_grid *g);
 size_t sweep2_workspace_bytes(const jac_grid *g);

@@ -509,12 +509,13 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
         double *res = no_res ? nullptr : (d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual);
         return resident_run(g, shape, n_iter, res, workspace, static_cast<cudaStream_t>(stream), nullptr, 0, opts);
     }
-    if (!injected && use_two_sweep_passes(g, plan, p, n_iter, num_sms()) && ws_bytes >= sweep2_workspace_bytes(g)) {
+    if (use_two_sweep_passes(g, plan, p, n_iter, num_sms()) && ws_bytes >= sweep2_workspace_bytes(g)) {
         const int n_pass = passes_of(n_iter);
         const int rest = n_iter - 2 * n_pass;          // the residual is theirs, if any
         double *res2 = nullptr;
         if (rest == 0 && !no_res) res2 = d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual;
-        if ((s = sweep2_run(g, 0, n_pass, res2, workspace, ws_bytes, static_cast<cudaStream_t>(stream))) != JAC_OK)
+        if ((s = sweep2_run(g, 0, n_pass, res2, workspace, ws_bytes, static_cast<cudaStream_t>(stream), nullptr,
+                            opts)) != JAC_OK)
             return s;
         if (rest == 0) return JAC_OK;
         n_iter = rest;

@@ -132,6 +132,9 @@ struct Sweep2Args {
     WsHeader *hdr;
     int l2_keep_state;
     unsigned l2_keep_coef;
+    unsigned long long wait_ns;   // limit of the waits on other warps and CTAs
+    unsigned gbar_extra;       // added to the targets between passes: 0, except when a test of the failure
+                               // path makes them unreachable
 };
 
 struct Item2 {
@@ -357,7 +360,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
     // reads each entry): pass * nitems + item, or END; false: give up.
     uint32_t ic = 0;
     auto next_item = [&](uint32_t &entry) -> bool {
-        bool r = mbar_wait_bounded(&i_full[ic % S::NQ], (ic / S::NQ) & 1);
+        bool r = mbar_wait_bounded(&i_full[ic % S::NQ], (ic / S::NQ) & 1, a.wait_ns);
         r = __all_sync(0xffffffffu, r && !s_abort);
         entry = s_item[ic % S::NQ];
         __syncwarp();
@@ -388,7 +391,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             const CUtensorMap *pm = nullptr, *cm = d.coef;
             auto put_state = [&](const Item2 &it, int q) -> bool {
                 const uint32_t slot = pc % RP, use = pc / RP;
-                if (use > 0 && !mbar_wait_bounded(&p_empty[slot], (use - 1) & 1)) return false;
+                if (use > 0 && !mbar_wait_bounded(&p_empty[slot], (use - 1) & 1, a.wait_ns)) return false;
                 if (s_abort) return false;
                 mbar_arrive_expect_tx(&p_full[slot], (uint32_t)S::P_BYTES);
                 tma_load_3d_hint(base + (size_t)slot * S::P_BYTES, pm, &p_full[slot], it.i0 - H, it.j0 - 2,
@@ -398,7 +401,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             };
             auto put_coef = [&](const Item2 &it, int q) -> bool {
                 const uint32_t slot = cc % RC, use = cc / RC;
-                if (use > 0 && !mbar_wait_bounded(&c_empty[slot], (use - 1) & 1)) return false;
+                if (use > 0 && !mbar_wait_bounded(&c_empty[slot], (use - 1) & 1, a.wait_ns)) return false;
                 if (s_abort) return false;
                 unsigned char *st = ring_c + (size_t)slot * S::C_BYTES;
                 mbar_arrive_expect_tx(&c_full[slot], (uint32_t)S::C_BYTES);
@@ -420,7 +423,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             [[maybe_unused]] uint32_t clock = 0;      // as last read
             while (ok) {
                 const uint32_t qslot = ip % S::NQ;
-                if (ip >= S::NQ && !(ok = mbar_wait_bounded(&i_empty[qslot], ((ip / S::NQ) - 1) & 1))) break;
+                if (ip >= S::NQ && !(ok = mbar_wait_bounded(&i_empty[qslot], ((ip / S::NQ) - 1) & 1, a.wait_ns))) break;
                 s_item[qslot] = entry;
                 mbar_arrive(&i_full[qslot]);
                 ++ip;
@@ -442,7 +445,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 if (!(ok = put_coef(it, 0))) break;
                 if (t > pass) {            // every item of the passes before is stored
                     pass = t;
-                    if (!(ok = wait_counter_bounded(&a.hdr->gbar, t * nitems * S::R2))) break;
+                    if (!(ok = wait_counter_bounded(&a.hdr->gbar, t * nitems * S::R2 + a.gbar_extra, a.wait_ns))) break;
                     fence_proxy_async_global();
                 }
                 if (!(ok = put_state(it, 0) && put_state(it, 1))) break;
@@ -535,13 +538,13 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const int m = it.kb - 1 + s;
                 const bool gone = s_abort;
                 if (s == 0) {
-                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
-                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
+                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1, a.wait_ns) &&
+                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1, a.wait_ns);
                 }
                 const uint32_t q2 = pc + s + 2;
-                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1);
+                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1, a.wait_ns);
                 const uint32_t qs = qc + s;
-                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
+                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1, a.wait_ns);
                 ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
                 if (s + 1 < it.nout + 2) load_coef(m + 1, cn);
@@ -626,8 +629,8 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const uint32_t qs = qc + s;
                 const bool gone = s_abort;
                 if (s == 0) {
-                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1) &&
-                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1);
+                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1, a.wait_ns) &&
+                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1, a.wait_ns);
                 }
                 const uint32_t q2 = pc + s + 2;
                 // The newest state plane, the stage and a free intermediate
@@ -638,9 +641,9 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const bool got_q = mbar_try_wait(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
                 ok = ok && !gone;
                 if (!__all_sync(0xffffffffu, ok && got_p && got_c && got_q)) {
-                    ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1) &&
-                         mbar_wait_bounded(&c_full[qs % RC], (qs / RC) & 1) &&
-                         mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
+                    ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1, a.wait_ns) &&
+                         mbar_wait_bounded(&c_full[qs % RC], (qs / RC) & 1, a.wait_ns) &&
+                         mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1, a.wait_ns);
                     ok = __all_sync(0xffffffffu, ok);
                 }
                 if (!ok) break;
@@ -764,7 +767,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         auto cons_sync = [&]() -> bool {
             __syncwarp();
             if (lane == 0) mbar_arrive(&cons_bar);
-            const bool r = mbar_wait_bounded(&cons_bar, sync_phase & 1);
+            const bool r = mbar_wait_bounded(&cons_bar, sync_phase & 1, a.wait_ns);
             ++sync_phase;
             return __all_sync(0xffffffffu, r);
         };
@@ -800,9 +803,9 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const size_t off = ((size_t)(it.kb - 3 + s) * J + (size_t)j) * (size_t)pitch + (size_t)ib;
                 const bool gone = s_abort;
                 if (s == 3)
-                    ok = mbar_wait_bounded(&q_full[qc % RQ], (qc / RQ) & 1) &&
-                         mbar_wait_bounded(&q_full[(qc + 1) % RQ], ((qc + 1) / RQ) & 1);
-                ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1);
+                    ok = mbar_wait_bounded(&q_full[qc % RQ], (qc / RQ) & 1, a.wait_ns) &&
+                         mbar_wait_bounded(&q_full[(qc + 1) % RQ], ((qc + 1) / RQ) & 1, a.wait_ns);
+                ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1, a.wait_ns);
                 ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
                 tmem_after_sync();
@@ -1098,7 +1101,7 @@ jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStre
 }  // namespace
 
 jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_residual, void *workspace,
-                      size_t ws_bytes, cudaStream_t st, void *mid)
+                      size_t ws_bytes, cudaStream_t st, void *mid, const LaunchOpts *opts)
 {
     if (mid != nullptr && n_pass != 1) return fail2(JAC_EINVAL, "the intermediate state needs a one-pass call");
     const long cols = (long)sweep2_tiles_i(g->I) * ((g->J - 2 + Sweep2Shape::R2 - 1) / Sweep2Shape::R2);
@@ -1124,6 +1127,8 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
     set_l2_policy(la, g->prec, (size_t)d.pitch * g->J * g->K);
     a.l2_keep_state = la.l2_keep_state;
     a.l2_keep_coef = la.l2_keep_coef;
+    a.wait_ns = opts && opts->wait_ns ? opts->wait_ns : kWaitLimitNs;
+    a.gbar_extra = opts ? opts->gbar_extra : 0;
     return mid != nullptr ? launch2<false, true>(d, a, nblocks, st)
                           : launch2<false, false>(d, a, nblocks, st);
 }
@@ -1154,6 +1159,7 @@ jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids,
     a.par = par;
     a.omega = omega;
     a.hdr = static_cast<WsHeader *>(workspace);
+    a.wait_ns = kWaitLimitNs;
     Sweep2Desc unused;
     std::memset(&unused, 0, sizeof(unused));
     return launch2<true, false>(unused, a, (unsigned)std::min(nitems, device_sm_count()), st);

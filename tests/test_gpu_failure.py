@@ -84,7 +84,8 @@ def test_single_sweep_launch_has_no_barrier_to_stall(pkg):
 def stall_and_recover(pkg, prec, dims, n, plan=None):
     """One stalled call (JAC_ETIMEOUT, a NaN residual, a partly swept state),
     then normal ones on the same context: bitwise the state of a context that
-    was never stalled.  Returns the stalled call's state."""
+    was never stalled.  Returns the fields, the stalled call's state and the other
+    state buffer after it."""
     I, J, K = dims
     f = ji.himeno_fields(I, J, K, seed=400 + I)
     with pkg.Jacobi(I, J, K, prec) as jac:
@@ -98,6 +99,8 @@ def stall_and_recover(pkg, prec, dims, n, plan=None):
         with pytest.raises(pkg.JacError) as err:
             jac.sync()
         assert err.value.status == 5 and np.isnan(res[0])
+        raw = jac.storage[1 - n % 2].cpu().numpy().view(np.float64 if prec == "f64" else np.float32)
+        other = raw.reshape(K, J, pkg.pitch(I))[:, :, :I].astype(np.float64)
         got = []
         for m in (n, n + 1):                              # the header is left as the next launch needs it
             jac.upload(f)
@@ -110,7 +113,7 @@ def stall_and_recover(pkg, prec, dims, n, plan=None):
             jac.upload(f)
             jac.sweep(m)
             assert np.array_equal(jac.download(), p) and jac.residual() == g
-    return f, stalled
+    return f, stalled, other
 
 
 @pytest.mark.parametrize("prec,dims", [("f32", (77, 53, 101)), ("bf16", (61, 40, 50)), ("f64", (33, 33, 65))])
@@ -120,7 +123,7 @@ def test_resident_waits_run_out(pkg, prec, dims):
     other boxes by then and no inner row (the streaming kernel stores all)."""
     n = 5                                                 # state n is in the buffer of state 1
     assert pkg.sweep_route(*dims, prec, n)["resident_sweeps"] == n
-    f, stalled = stall_and_recover(pkg, prec, dims, n)
+    f, stalled, _ = stall_and_recover(pkg, prec, dims, n)
     with pkg.Jacobi(*dims, prec) as jac:
         jac.upload(f)
         p0 = jac.download()
@@ -129,3 +132,20 @@ def test_resident_waits_run_out(pkg, prec, dims):
     inside = (slice(1, -1),) * 3
     swept, kept = np.all(stalled == p1, axis=2)[inside[:2]], np.all(stalled == p0, axis=2)[inside[:2]]
     assert np.all(swept | kept) and swept.any() and kept.any()
+
+
+@pytest.mark.parametrize("dims,n,plan", [((129, 33, 20), 4, (0, 0, 0, 2)), ((130, 17, 23), 8, (0, 0, 0, 2)),
+                                         ((129, 129, 140), 4, None)])
+def test_pass_barrier_runs_out(pkg, dims, n, plan):
+    """The two-sweep kernel's wait between passes: the first pass is stored --
+    state 2, where single sweeps would have stored state 1 -- and no CTA starts
+    the second.  Sweeps after the passes would run on that state, with a NaN
+    residual."""
+    assert pkg.sweep_route(*dims, "f32", n, fuse=plan[3] if plan else 0)["passes"] == n // 2
+    f, stalled, other = stall_and_recover(pkg, "f32", dims, n, plan)
+    with pkg.Jacobi(*dims, "f32") as jac:
+        jac.set_plan(0, 0, 0, 1)
+        jac.upload(f)
+        assert np.array_equal(stalled, jac.download())
+        jac.sweep(2)
+        assert np.array_equal(other, jac.download())
