@@ -69,7 +69,8 @@ jac_status launch_sweep(jac_prec prec, int tj, const GridDesc &d0, const SweepAr
 // writes the other buffer.  The residual of the last sweep goes to d_residual
 // (NULL: none).  kdepth 0: the default depth.  mid (one-pass calls only) also
 // receives the state after the first sweep at every interior point; its faces
-// are left as they are.  opts: only its wait_ns and gbar_extra are read.
+// are left as they are.  opts: only its wait_ns and gbar_extra are read; with
+// either one set mid is not written.
 jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_residual, void *workspace,
                       size_t ws_bytes, cudaStream_t st, void *mid = nullptr, const LaunchOpts *opts = nullptr);
 // Whether the library's plan for this grid takes two-sweep passes (fuse 0).

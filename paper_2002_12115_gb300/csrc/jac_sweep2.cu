@@ -57,7 +57,9 @@
 //     sweeps);
 //   * a one-pass call may also store sweep 1's state at the points the
 //     items own (MID, Sweep2Args::mid): the reverse pass recomputes two
-//     checkpoint-segment states per launch that way.
+//     checkpoint-segment states per launch that way;
+//   * STALL: a test of the failure path, with its own wait limit and a barrier
+//     between passes that no CTA reaches.
 //
 // What bounds it: latency and issue of 18 compute warps where the state stays in
 // L2 (a step of a CTA, one plane of a tile, both sweeps, takes 1.34 us), and
@@ -132,9 +134,8 @@ struct Sweep2Args {
     WsHeader *hdr;
     int l2_keep_state;
     unsigned l2_keep_coef;
-    unsigned long long wait_ns;   // limit of the waits on other warps and CTAs
-    unsigned gbar_extra;       // added to the targets between passes: 0, except when a test of the failure
-                               // path makes them unreachable
+    unsigned long long wait_ns;   // STALL: limit of the waits on other warps and CTAs
+    unsigned gbar_extra;       // STALL: added to the targets between passes, which makes them unreachable
 };
 
 struct Item2 {
@@ -321,7 +322,7 @@ __device__ __forceinline__ void ss_axes4(const float (&x)[6], const float (&yp)[
     }
 }
 
-template <bool BATCH, bool MID>
+template <bool BATCH, bool MID, bool STALL>
 __global__ void __launch_bounds__(Sweep2Shape::THREADS, 1)
 k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
 {
@@ -343,6 +344,10 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int G = gridDim.x;
+    // A test of the failure path has a kernel of its own: arguments in place of
+    // these constants cost 3% of 513x513x1025 (1277 -> 1317 us a sweep).
+    const unsigned long long limit = STALL ? a.wait_ns : kWaitLimitNs;
+    const unsigned extra = STALL ? a.gbar_extra : 0u;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < RP; ++s) { mbar_init(&p_full[s], 1); mbar_init(&p_empty[s], R1 + 1); }
@@ -360,7 +365,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
     // reads each entry): pass * nitems + item, or END; false: give up.
     uint32_t ic = 0;
     auto next_item = [&](uint32_t &entry) -> bool {
-        bool r = mbar_wait_bounded(&i_full[ic % S::NQ], (ic / S::NQ) & 1, a.wait_ns);
+        bool r = mbar_wait_bounded(&i_full[ic % S::NQ], (ic / S::NQ) & 1, limit);
         r = __all_sync(0xffffffffu, r && !s_abort);
         entry = s_item[ic % S::NQ];
         __syncwarp();
@@ -391,7 +396,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             const CUtensorMap *pm = nullptr, *cm = d.coef;
             auto put_state = [&](const Item2 &it, int q) -> bool {
                 const uint32_t slot = pc % RP, use = pc / RP;
-                if (use > 0 && !mbar_wait_bounded(&p_empty[slot], (use - 1) & 1, a.wait_ns)) return false;
+                if (use > 0 && !mbar_wait_bounded(&p_empty[slot], (use - 1) & 1, limit)) return false;
                 if (s_abort) return false;
                 mbar_arrive_expect_tx(&p_full[slot], (uint32_t)S::P_BYTES);
                 tma_load_3d_hint(base + (size_t)slot * S::P_BYTES, pm, &p_full[slot], it.i0 - H, it.j0 - 2,
@@ -401,7 +406,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             };
             auto put_coef = [&](const Item2 &it, int q) -> bool {
                 const uint32_t slot = cc % RC, use = cc / RC;
-                if (use > 0 && !mbar_wait_bounded(&c_empty[slot], (use - 1) & 1, a.wait_ns)) return false;
+                if (use > 0 && !mbar_wait_bounded(&c_empty[slot], (use - 1) & 1, limit)) return false;
                 if (s_abort) return false;
                 unsigned char *st = ring_c + (size_t)slot * S::C_BYTES;
                 mbar_arrive_expect_tx(&c_full[slot], (uint32_t)S::C_BYTES);
@@ -423,7 +428,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
             [[maybe_unused]] uint32_t clock = 0;      // as last read
             while (ok) {
                 const uint32_t qslot = ip % S::NQ;
-                if (ip >= S::NQ && !(ok = mbar_wait_bounded(&i_empty[qslot], ((ip / S::NQ) - 1) & 1, a.wait_ns))) break;
+                if (ip >= S::NQ && !(ok = mbar_wait_bounded(&i_empty[qslot], ((ip / S::NQ) - 1) & 1, limit))) break;
                 s_item[qslot] = entry;
                 mbar_arrive(&i_full[qslot]);
                 ++ip;
@@ -445,7 +450,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 if (!(ok = put_coef(it, 0))) break;
                 if (t > pass) {            // every item of the passes before is stored
                     pass = t;
-                    if (!(ok = wait_counter_bounded(&a.hdr->gbar, t * nitems * S::R2 + a.gbar_extra, a.wait_ns))) break;
+                    if (!(ok = wait_counter_bounded(&a.hdr->gbar, t * nitems * S::R2 + extra, limit))) break;
                     fence_proxy_async_global();
                 }
                 if (!(ok = put_state(it, 0) && put_state(it, 1))) break;
@@ -538,13 +543,13 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const int m = it.kb - 1 + s;
                 const bool gone = s_abort;
                 if (s == 0) {
-                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1, a.wait_ns) &&
-                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1, a.wait_ns);
+                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1, limit) &&
+                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1, limit);
                 }
                 const uint32_t q2 = pc + s + 2;
-                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1, a.wait_ns);
+                ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1, limit);
                 const uint32_t qs = qc + s;
-                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1, a.wait_ns);
+                if (qs >= RQ) ok = ok && mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1, limit);
                 ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
                 if (s + 1 < it.nout + 2) load_coef(m + 1, cn);
@@ -629,8 +634,8 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const uint32_t qs = qc + s;
                 const bool gone = s_abort;
                 if (s == 0) {
-                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1, a.wait_ns) &&
-                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1, a.wait_ns);
+                    ok = mbar_wait_bounded(&p_full[pc % RP], (pc / RP) & 1, limit) &&
+                         mbar_wait_bounded(&p_full[(pc + 1) % RP], ((pc + 1) / RP) & 1, limit);
                 }
                 const uint32_t q2 = pc + s + 2;
                 // The newest state plane, the stage and a free intermediate
@@ -641,9 +646,9 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const bool got_q = mbar_try_wait(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1);
                 ok = ok && !gone;
                 if (!__all_sync(0xffffffffu, ok && got_p && got_c && got_q)) {
-                    ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1, a.wait_ns) &&
-                         mbar_wait_bounded(&c_full[qs % RC], (qs / RC) & 1, a.wait_ns) &&
-                         mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1, a.wait_ns);
+                    ok = ok && mbar_wait_bounded(&p_full[q2 % RP], (q2 / RP) & 1, limit) &&
+                         mbar_wait_bounded(&c_full[qs % RC], (qs / RC) & 1, limit) &&
+                         mbar_wait_bounded(&q_empty[qs % RQ], ((qs / RQ) - 1) & 1, limit);
                     ok = __all_sync(0xffffffffu, ok);
                 }
                 if (!ok) break;
@@ -767,7 +772,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
         auto cons_sync = [&]() -> bool {
             __syncwarp();
             if (lane == 0) mbar_arrive(&cons_bar);
-            const bool r = mbar_wait_bounded(&cons_bar, sync_phase & 1, a.wait_ns);
+            const bool r = mbar_wait_bounded(&cons_bar, sync_phase & 1, limit);
             ++sync_phase;
             return __all_sync(0xffffffffu, r);
         };
@@ -803,9 +808,9 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                 const size_t off = ((size_t)(it.kb - 3 + s) * J + (size_t)j) * (size_t)pitch + (size_t)ib;
                 const bool gone = s_abort;
                 if (s == 3)
-                    ok = mbar_wait_bounded(&q_full[qc % RQ], (qc / RQ) & 1, a.wait_ns) &&
-                         mbar_wait_bounded(&q_full[(qc + 1) % RQ], ((qc + 1) / RQ) & 1, a.wait_ns);
-                ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1, a.wait_ns);
+                    ok = mbar_wait_bounded(&q_full[qc % RQ], (qc / RQ) & 1, limit) &&
+                         mbar_wait_bounded(&q_full[(qc + 1) % RQ], ((qc + 1) / RQ) & 1, limit);
+                ok = ok && mbar_wait_bounded(&q_full[(qs - 1) % RQ], ((qs - 1) / RQ) & 1, limit);
                 ok = __all_sync(0xffffffffu, ok && !gone);
                 if (!ok) break;
                 tmem_after_sync();
@@ -1062,14 +1067,14 @@ jac_status build_desc2(Sweep2Desc *d, const jac_grid *g, int kdepth)
 // All passes of a call.  Items of all passes and the arrivals of the pass
 // barrier are counted in 32 bits: very long calls take several launches, each
 // of an even number of passes.
-template <bool BATCH, bool MID>
+template <bool BATCH, bool MID, bool STALL>
 jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStream_t st)
 {
     using S = Sweep2Shape;
     static std::once_flag attr_once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(attr_once, [] {
-        attr_err = cudaFuncSetAttribute(k_sweep2<BATCH, MID>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        attr_err = cudaFuncSetAttribute(k_sweep2<BATCH, MID, STALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)S::SMEM);
     });
     if (attr_err != cudaSuccess)
@@ -1092,7 +1097,7 @@ jac_status launch2(const Sweep2Desc &d, Sweep2Args a, unsigned nblocks, cudaStre
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep2<BATCH, MID>, d, a);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sweep2<BATCH, MID, STALL>, d, a);
         if (e != cudaSuccess) return fail2(JAC_ECUDA, std::string("two-sweep launch: ") + cudaGetErrorString(e));
     }
     return JAC_OK;
@@ -1127,10 +1132,13 @@ jac_status sweep2_run(const jac_grid *g, int kdepth, int n_pass, double *d_resid
     set_l2_policy(la, g->prec, (size_t)d.pitch * g->J * g->K);
     a.l2_keep_state = la.l2_keep_state;
     a.l2_keep_coef = la.l2_keep_coef;
-    a.wait_ns = opts && opts->wait_ns ? opts->wait_ns : kWaitLimitNs;
-    a.gbar_extra = opts ? opts->gbar_extra : 0;
-    return mid != nullptr ? launch2<false, true>(d, a, nblocks, st)
-                          : launch2<false, false>(d, a, nblocks, st);
+    if (opts && (opts->wait_ns != 0 || opts->gbar_extra != 0)) {
+        a.wait_ns = opts->wait_ns ? opts->wait_ns : kWaitLimitNs;
+        a.gbar_extra = opts->gbar_extra;
+        return launch2<false, false, true>(d, a, nblocks, st);
+    }
+    return mid != nullptr ? launch2<false, true, false>(d, a, nblocks, st)
+                          : launch2<false, false, false>(d, a, nblocks, st);
 }
 
 // ---- batches: the descriptors of many grids in device memory
@@ -1159,10 +1167,9 @@ jac_status sweep2_batch_run(const void *descs, const int *item_base, int ngrids,
     a.par = par;
     a.omega = omega;
     a.hdr = static_cast<WsHeader *>(workspace);
-    a.wait_ns = kWaitLimitNs;
     Sweep2Desc unused;
     std::memset(&unused, 0, sizeof(unused));
-    return launch2<true, false>(unused, a, (unsigned)std::min(nitems, device_sm_count()), st);
+    return launch2<true, false, false>(unused, a, (unsigned)std::min(nitems, device_sm_count()), st);
 }
 
 }  // namespace jac
