@@ -694,12 +694,8 @@ def bench_batch(args, stream, sweeps=100, steps=3, autotune=True, loops=True, tu
             plan = at.ga_tune_batch(b, M=10, T=10, n_sweeps=10, reps=2)
         else:
             plan = at.tune_batch(b, n_sweeps=10, reps=2, passes=1)
-        # a plan asks for single sweeps; without one the wide grids sweep in passes
-        tuned_ms = ms_per_call()
-        if default_ms <= tuned_ms:
-            b.set_plan(0, None, None)
-        plan = {"plan": plan, "ms_per_step": tuned_ms, "default_ms_per_step": default_ms,
-                "used": "default" if default_ms <= tuned_ms else "plan"}
+        plan = {"plan": plan, "ms_per_step": ms_per_call(), "default_ms_per_step": default_ms,
+                "used": "default" if plan["no_plan"] else "plan"}
     b.sweep(sweeps)          # capture + warm-up
     b.sweep(sweeps)
     a, e = events()
@@ -766,6 +762,7 @@ def bench_tuners(stream, sweeps=100):
         t0 = time.perf_counter()
         plan = search()
         out[name] = {"value": rate(), "plans_measured": count["n"], "search_s": time.perf_counter() - t0,
+                     "no_plan": plan["no_plan"], "value_of_plan": npts / plan["s_per_sweep"] / 1e9,
                      "plan": {k: plan[k] for k in ("warps", "tile_i", "kdepth")}}
     b.close()
     torch.cuda.empty_cache()
@@ -796,6 +793,7 @@ def bench_tuners(stream, sweeps=100):
         t0 = time.perf_counter()
         plan = search()
         res[name] = {"value": sub_rate(), "search_s": time.perf_counter() - t0,
+                     "no_plan": plan["no_plan"], "value_of_plan": nsub / plan["s_per_sweep"] / 1e9,
                      "plan": {k: plan[k] for k in ("warps", "tile_i", "kdepth")}}
         if name == "joint_exhaustive":
             ts = plan["times"]

@@ -6,7 +6,12 @@ whose fitness is the measured run time, Sections 3.2 and 4); a loop's
 suitability cannot be predicted, only measured.  This module applies the
 same principle to the sweep's launch plan: candidate plans are run on the
 GPU, timed with CUDA events (median of several repetitions), and the fastest
-is kept and cached.
+is kept and cached.  A plan asks for streaming sweeps of a given shape; without
+one the library may run a grid resident or in two-sweep passes.  So every
+search also times no plan at all, and where that is as fast or faster it leaves
+the grid or batch without one: the result's ``no_plan`` says so, its other
+entries describe the best plan of the search and ``default_s_per_sweep`` the
+time without.
 
   * ``tune_grid``  -- one grid: tile width x rows x k-block depth;
   * ``tune_batch`` -- a batch: warp count for the launch, then coordinate
@@ -26,8 +31,7 @@ from itertools import product
 
 from .binding import JacError
 
-# plans measured on this project's GPUs ship with the package; set
-# JAC_AUTOTUNE_CACHE to keep a cache elsewhere
+# set JAC_AUTOTUNE_CACHE to keep the cache elsewhere
 CACHE_PATH = os.environ.get("JAC_AUTOTUNE_CACHE",
                             os.path.join(os.path.dirname(os.path.abspath(__file__)), "autotune_cache.json"))
 
@@ -72,20 +76,58 @@ def time_call(fn, reps: int = 3, stream=None) -> float:
     return statistics.median(times)
 
 
+# Prefix of cache keys.  Entries under another one were written by searches that
+# did not time the library's own choice and are not read.
+_KEY = "v2"
+
+
+def _no_plan(batch) -> None:
+    zeros = [0] * len(batch.dims)
+    batch.set_plan(0, zeros, zeros)
+
+
+def _settle(batch, plan: dict, t: float, expand, n_sweeps: int, reps: int) -> dict:
+    """Leaves the batch on the plan a search found (n_sweeps sweeps in t
+    seconds), or without one where that is as fast; returns the plan with both
+    times and the decision."""
+    _no_plan(batch)
+    batch.sweep(n_sweeps, residuals=False)           # capture + warm-up
+    t_default = time_call(lambda: batch.sweep(n_sweeps, residuals=False), reps)
+    out = dict(plan, s_per_sweep=t / n_sweeps, default_s_per_sweep=t_default / n_sweeps, no_plan=t_default <= t)
+    _install(batch, out, expand)
+    return out
+
+
+def _install(batch, plan: dict, expand) -> None:
+    if plan["no_plan"]:
+        _no_plan(batch)
+    else:
+        batch.set_plan(plan["warps"], *expand(plan))
+
+
 def _tile_widths(prec: str) -> list[int]:
     return [64, 32, 16] if prec == "f64" else [128, 64, 32, 16]
 
 
 def tune_grid(jac, n_sweeps: int = 20, reps: int = 3, kdepths=(2, 4, 8, 16, 32, 64), warps=(4, 8, 16),
               cache_path: str | None = CACHE_PATH) -> dict:
-    """Best (tile_i, tile_j, kdepth) of a Jacobi context by measurement.
-    The context must hold uploaded fields; its state advances while tuning."""
-    key = f"grid|{_gpu_name()}|{jac.prec}|{jac.I}x{jac.J}x{jac.K}"
+    """Best (tile_i, tile_j, kdepth) of a Jacobi context by measurement, or no
+    plan where that is as fast.  The context must hold uploaded fields; its state
+    advances while tuning."""
+    key = f"{_KEY}|grid|{_gpu_name()}|{jac.prec}|{jac.I}x{jac.J}x{jac.K}"
     cache = _load_cache(cache_path) if cache_path else {}
+
+    def measure(plan) -> float:
+        jac.set_plan(*plan)
+        jac.sweep(n_sweeps)  # warm-up of this shape
+        return time_call(lambda: jac.sweep(n_sweeps), reps)
+
+    def install(best) -> None:
+        jac.set_plan(*((0, 0, 0) if best["no_plan"] else (best["tile_j"], best["kdepth"], best["tile_i"])))
+
     if key in cache:
-        best = cache[key]
-        jac.set_plan(best["tile_j"], best["kdepth"], best["tile_i"])
-        return best
+        install(cache[key])
+        return cache[key]
     full = 64 if jac.prec == "f64" else 128
     trials = []
     for ti, w, kd in product(_tile_widths(jac.prec), warps, kdepths):
@@ -93,16 +135,15 @@ def tune_grid(jac, n_sweeps: int = 20, reps: int = 3, kdepths=(2, 4, 8, 16, 32, 
             continue
         plan = (w * (full // ti), kd, ti)
         try:
-            jac.set_plan(*plan)
+            trials.append((measure(plan), plan))
         except JacError:
             continue
-        jac.sweep(1)  # warm-up of this shape
-        t = time_call(lambda: jac.sweep(n_sweeps), reps)
-        trials.append((t, plan))
     trials.sort()
     t, (tj, kd, ti) = trials[0]
-    best = {"tile_i": ti, "tile_j": tj, "kdepth": kd, "s_per_sweep": t / n_sweeps, "trials": len(trials)}
-    jac.set_plan(tj, kd, ti)
+    t_default = measure((0, 0, 0))
+    best = {"tile_i": ti, "tile_j": tj, "kdepth": kd, "s_per_sweep": t / n_sweeps,
+            "default_s_per_sweep": t_default / n_sweeps, "no_plan": t_default <= t, "trials": len(trials)}
+    install(best)
     if cache_path:
         cache[key] = best
         _store_cache(cache_path, cache)
@@ -116,7 +157,7 @@ def tune_batch(batch, n_sweeps: int = 10, reps: int = 3, passes: int = 2, kdepth
     The batch must hold uploaded fields; its state advances while tuning."""
     dims = batch.dims
     sig = ",".join(f"{I}x{J}x{K}" for I, J, K in dims)
-    key = f"batch|{_gpu_name()}|{batch.prec}|{len(dims)}|{hashlib.sha1(sig.encode()).hexdigest()[:12]}"
+    key = f"{_KEY}|batch|{_gpu_name()}|{batch.prec}|{len(dims)}|{hashlib.sha1(sig.encode()).hexdigest()[:12]}"
     cache = _load_cache(cache_path) if cache_path else {}
     i_classes = sorted({d[0] for d in dims})
     k_classes = sorted({d[2] for d in dims})
@@ -136,10 +177,8 @@ def tune_batch(batch, n_sweeps: int = 10, reps: int = 3, passes: int = 2, kdepth
         return time_call(lambda: batch.sweep(n_sweeps, residuals=False), reps)
 
     if key in cache:
-        plan = cache[key]
-        ti, kd = expand(plan)
-        batch.set_plan(plan["warps"], ti, kd)
-        return plan
+        _install(batch, cache[key], expand)
+        return cache[key]
 
     widths = _tile_widths(batch.prec)
     best_plan = None
@@ -173,10 +212,7 @@ def tune_batch(batch, n_sweeps: int = 10, reps: int = 3, passes: int = 2, kdepth
             log(f"warps {w}: {t_cur / n_sweeps * 1e3:.3f} ms/sweep")
         if t_cur < best_t:
             best_plan, best_t = plan, t_cur
-    best_plan = dict(best_plan)
-    best_plan["s_per_sweep"] = best_t / n_sweeps
-    ti, kd = expand(best_plan)
-    batch.set_plan(best_plan["warps"], ti, kd)
+    best_plan = _settle(batch, best_plan, best_t, expand, n_sweeps, reps)
     if cache_path:
         cache[key] = best_plan
         _store_cache(cache_path, cache)
@@ -305,12 +341,7 @@ def ga_tune_batch(batch, M: int = 10, T: int = 10, n_sweeps: int = 10, reps: int
         return time_call(lambda: batch.sweep(n_sweeps, residuals=False), reps)
 
     bits, t, history = ga_search(genome.n_bits, measure, M=M, T=T, seed=seed, log=log)
-    plan = genome.decode(bits)
-    ti, kd = expand(plan)
-    batch.set_plan(plan["warps"], ti, kd)
-    plan["s_per_sweep"] = t / n_sweeps
-    plan["history"] = history
-    return plan
+    return dict(_settle(batch, genome.decode(bits), t, expand, n_sweeps, reps), history=history)
 
 
 # --------------------------------------------------------------------------
@@ -383,10 +414,7 @@ def class_exhaustive_tune_batch(batch, n_sweeps: int = 10, reps: int = 2, kdepth
             log(f"warps {w}: combined per-class plan {t / n_sweeps * 1e3:.3f} ms/sweep")
         if t < best_t:
             best_plan, best_t = plan, t
-    ti, kd = expand(best_plan)
-    batch.set_plan(best_plan["warps"], ti, kd)
-    best_plan = dict(best_plan, s_per_sweep=best_t / n_sweeps, measured=count)
-    return best_plan
+    return dict(_settle(batch, best_plan, best_t, expand, n_sweeps, reps), measured=count)
 
 
 def joint_exhaustive_tune_batch(batch, n_sweeps: int = 5, reps: int = 2, kdepths=(4, 8, 16, 32, 64, 12, 24, 48),
@@ -410,9 +438,7 @@ def joint_exhaustive_tune_batch(batch, n_sweeps: int = 5, reps: int = 2, kdepths
         results.append((measure(plan), plan))
     results.sort(key=lambda r: r[0])
     t, plan = results[0]
-    ti, kd = expand(plan)
-    batch.set_plan(plan["warps"], ti, kd)
     if log:
         log(f"{len(results)} plans: best {t / n_sweeps * 1e3:.3f} ms/sweep")
-    return dict(plan, s_per_sweep=t / n_sweeps, measured=len(results),
+    return dict(_settle(batch, plan, t, expand, n_sweeps, reps), measured=len(results),
                 times=sorted(r[0] / n_sweeps for r in results))
