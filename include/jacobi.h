@@ -138,9 +138,9 @@ typedef struct jac_grid {
  * the state is bitwise the same.  Calls of three sweeps or more on grids whose
  * coefficients fit in the shared memory of all SMs together run resident (one
  * launch that keeps them there and exchanges only the rows between
- * neighbouring CTAs), and FP32 grids run two sweeps per pass where that is
- * estimated to be faster, whatever the size of their state.  Any non-zero
- * field selects the kernels as described here. */
+ * neighbouring CTAs) where that is estimated to be faster, and other FP32
+ * grids run two sweeps per pass where that is, whatever the size of their
+ * state.  Any non-zero field selects the kernels as described here. */
 enum { JAC_KDEPTH_BALANCED = -1 };
 typedef struct jac_plan {
     int tile_j;   /* rows per work item */

@@ -106,7 +106,7 @@ size_t resident_workspace_bytes(const ResidentShape &s);
 jac_status resident_run(const jac_grid *g, const ResidentShape &s, int n_iter, double *d_residual, void *workspace,
                         cudaStream_t st, void *hist = nullptr, size_t hist_stride = 0,
                         const LaunchOpts *opts = nullptr);
-// Whether a call of n_iter sweeps with this plan and workspace runs resident.
+// Whether a call of n_iter sweeps with this plan and workspace can run resident.
 bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r);
 jac_status adjoint_step_dev(const jac_grid *g, const void *p_t, const void *lam_in, void *lam_out, double *g_wrk1,
                             double *g_a3, double *const *g_coef, int kdepth, void *workspace, size_t ws_bytes,

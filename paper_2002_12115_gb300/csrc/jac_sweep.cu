@@ -438,21 +438,64 @@ size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
     return need;
 }
 
-// Whether a call runs resident (jac_resident.cu): the library's own plan, a
+// Whether a call can run resident (jac_resident.cu): the library's own plan, a
 // grid that fits in shared memory and a workspace with room for the flags (a
-// caller with a workspace sized for the streaming kernel keeps that one).
-// Measured with both kernels on every grid tried (17x17x17 to 65x65x129, all
-// precisions) a resident sweep takes 0.54-0.82 of a streaming one and the
-// launch up to 6 us more (the copy of the coefficients), so it pays from the
-// third sweep on; one or two sweeps stay with the streaming kernel.
-static bool resident_pays(const jac_grid *g, const jac_plan *plan, int n_iter, int sms, ResidentShape *r)
+// caller with a workspace sized for the streaming kernel keeps that one).  One
+// or two sweeps stay with the streaming kernel.
+static bool resident_fits(const jac_grid *g, const jac_plan *plan, int n_iter, int sms, ResidentShape *r)
 {
     return n_iter >= 3 && all_zero(plan) && resident_shape(g->I, g->J, g->K, g->prec, sms, r);
 }
 
 bool use_resident(const jac_grid *g, const jac_plan *plan, int n_iter, size_t ws_bytes, ResidentShape *r)
 {
-    return resident_pays(g, plan, n_iter, num_sms(), r) && ws_bytes >= resident_workspace_bytes(*r);
+    return resident_fits(g, plan, n_iter, num_sms(), r) && ws_bytes >= resident_workspace_bytes(*r);
+}
+
+// Microseconds of a resident sweep: the exchange, the points of the largest
+// box -- those in rows next to another box before the exchange, the others
+// beside it -- and the halo elements that the busiest communication warp
+// collects.  Fitted to 210 grids of all precisions, 5 to 536 columns wide: 8%
+// rms, 27% at most.
+static double resident_us(const jac_grid *g, const ResidentShape &s)
+{
+    const int rows = s.bj * s.bk;
+    const int edge_rows = (s.bj <= 2 || s.bk <= 2) ? rows : 2 * (s.bj + s.bk) - 4;
+    const double edge = 1e-3 * edge_rows * (g->I - 2), inner = 1e-3 * (rows - edge_rows) * (g->I - 2);
+    const double halo = 1e-3 * s.ws * std::max(s.nj > 1 ? s.bk : 0, s.nk > 1 ? s.bj : 0);
+    return g->prec == JAC_F64 ? 3.1 + 4.5 * edge + 2.9 * inner + 4.1 * halo
+                              : 2.7 + 0.8 * edge + 0.13 * inner + 1.5 * halo;
+}
+
+// Microseconds of a streaming sweep of a grid whose coefficients stay on chip:
+// the barrier and the first planes, then the planes of a CTA's items one after
+// the other.  The same 210 grids: 4% rms, 12% at most.
+static double streaming_us(const jac_grid *g, const jac_plan &p, int sms)
+{
+    const int warps = p.tile_j * p.tile_i / (32 * vector_points(g->prec)), nk = g->K - 2;
+    const long long cols = (long long)((g->I - 2) / p.tile_i + 1) * ((g->J - 2 + p.tile_j - 1) / p.tile_j);
+    long long planes;
+    if (p.kdepth == JAC_KDEPTH_BALANCED) {
+        planes = (cols * nk + sms - 1) / sms;
+    } else {
+        const long long items = cols * ((nk + p.kdepth - 1) / p.kdepth);
+        planes = (items + sms - 1) / sms * std::min(p.kdepth, nk);
+    }
+    if (g->prec == JAC_F64) return 3.5 + 2.7 * (double)planes;
+    return warps == 16 ? 2.4 + 1.45 * (double)planes : 2.3 + 1.0 * (double)planes;
+}
+
+// Whether resident is the faster of the two for a call that can take it: on
+// most grids it is (0.5 to 0.9 of the time a sweep), but the boxes of wide, flat
+// grids have no inner rows to update during the exchange and much halo per
+// point: 402x145x5 BF16 5.5 us a sweep against 4.1 streaming, 449x160x3 FP32 4.3
+// against 3.4, 147x114x11 FP32 5.2 against 4.4, 264x122x8 FP64 14.5 against
+// 11.7.  The launch takes 2 us more (the copy of the coefficients).  Over 210
+// grids and calls of 3, 20 and 120 sweeps the choice is 0.1% slower than the
+// better of the two on average and 7% at most.  p is the resolved plan.
+static bool resident_pays(const jac_grid *g, const jac_plan &p, int n_iter, int sms, const ResidentShape &s)
+{
+    return n_iter * resident_us(g, s) + 2.0 < n_iter * streaming_us(g, p, sms);
 }
 
 // Whether a call of n_iter sweeps with the library's own plan (all zero) takes
@@ -505,7 +548,8 @@ jac_status sweep_dev(const jac_grid *g, const jac_plan *plan, int n_iter, double
     const size_t need = sweep_workspace_bytes(g, p);
     if (ws_bytes < need) return fail(JAC_EINVAL, "workspace too small: need " + std::to_string(need) + " bytes");
     ResidentShape shape;
-    if (use_resident(g, plan, n_iter, ws_bytes, &shape) && !(injected && shape.nj * shape.nk == 1)) {
+    if (use_resident(g, plan, n_iter, ws_bytes, &shape) && resident_pays(g, p, n_iter, num_sms(), shape) &&
+        !(injected && shape.nj * shape.nk == 1)) {
         double *res = no_res ? nullptr : (d_residual ? d_residual : &static_cast<WsHeader *>(workspace)->residual);
         return resident_run(g, shape, n_iter, res, workspace, static_cast<cudaStream_t>(stream), nullptr, 0, opts);
     }
@@ -625,7 +669,7 @@ jac_status jac_sweep_route(const jac_grid *g, const jac_plan *plan, int n_iter, 
     const int sms = sm_count > 0 ? sm_count : jac::device_sm_count();
     *out = jac_route();
     jac::ResidentShape shape;
-    if (jac::resident_pays(g, plan, n_iter, sms, &shape)) {
+    if (jac::resident_fits(g, plan, n_iter, sms, &shape) && jac::resident_pays(g, p, n_iter, sms, shape)) {
         out->resident_sweeps = n_iter;
         out->launches = 1;
         return JAC_OK;

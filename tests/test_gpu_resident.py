@@ -19,7 +19,9 @@ pytestmark = pytest.mark.gpu
 STREAM = (0, 0, 0, 1)
 BAR = {"f64": 1e-12, "f32": 8 * 2.0 ** -24, "bf16": 8 * 2.0 ** -24}
 SHAPES = [(3, 3, 3), (3, 17, 9), (5, 6, 7), (17, 17, 17), (33, 33, 65), (77, 53, 101), (700, 5, 6), (49, 49, 97),
-          (65, 65, 129), (3, 90, 80), (130, 12, 40)]
+          (65, 65, 129), (3, 90, 80), (130, 12, 40), (600, 3, 70)]
+# they do not fit, or their boxes' halos take longer than streaming
+STREAMING = {("f64", (77, 53, 101)), ("f64", (65, 65, 129)), ("f64", (700, 5, 6)), ("f32", (700, 5, 6))}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -39,9 +41,9 @@ def test_equals_streaming(dims, prec):
     I, J, K = dims
     f = ji.himeno_fields(I, J, K, seed=900 + I + J + K)
     from paper_2002_12115_gb300 import sweep_route
-    fits = prec != "f64" or dims not in ((77, 53, 101), (65, 65, 129))     # else streaming both times
-    for n in (3, 8):
-        assert sweep_route(I, J, K, prec, n)["resident_sweeps"] == (n if fits else 0)
+    for n in (3, 8, 9):
+        if n > 3:                # three sweeps may not be worth the copy of the coefficients
+            assert sweep_route(I, J, K, prec, n)["resident_sweeps"] == (0 if (prec, dims) in STREAMING else n)
         assert sweep_route(I, J, K, prec, n, fuse=1)["single_sweeps"] == n
         p1, g1 = gpu_run(f, n, prec, STREAM)
         p2, g2 = gpu_run(f, n, prec)

@@ -32,6 +32,25 @@ def test_routes_without_a_plan(dims, prec, n, want):
     assert route(*dims, prec, n) == want
 
 
+@pytest.mark.parametrize("dims,prec", [
+    ((402, 145, 5), "bf16"), ((449, 160, 3), "f32"), ((147, 114, 11), "f32"), ((404, 44, 23), "f32"),
+    ((143, 158, 9), "f32"), ((321, 22, 34), "f32"), ((254, 37, 51), "bf16"), ((264, 122, 8), "f64"),
+    ((120, 40, 30), "f64")])
+def test_wide_flat_grids_stream(dims, prec):
+    """Their coefficients fit in shared memory, but a resident sweep takes 1.05
+    to 1.6 times a streaming one: boxes without inner rows, and much halo."""
+    for n in (4, 20, 100):
+        assert route(*dims, prec, n)[1] == 0
+
+
+@pytest.mark.parametrize("dims,prec,n", [
+    ((17, 17, 17), "f64", 5), ((33, 33, 65), "f64", 5), ((49, 49, 97), "f64", 5), ((77, 53, 101), "f32", 5),
+    ((65, 65, 129), "f32", 5), ((65, 65, 129), "bf16", 5), ((61, 40, 50), "bf16", 5), ((218, 133, 4), "f32", 20),
+    ((80, 104, 3), "f64", 5), ((70, 20, 4), "bf16", 5)])
+def test_small_grids_run_resident(dims, prec, n):
+    assert route(*dims, prec, n)[1] == n
+
+
 def test_routes_of_explicit_plans():
     """Any non-zero entry leaves out the resident kernel; fuse 1 and 2 decide
     the passes, fuse 0 beside another entry the size of the state."""
