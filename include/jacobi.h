@@ -191,10 +191,11 @@ typedef struct jac_route {
 jac_status jac_sweep_route(const jac_grid *g, const jac_plan *plan, int n_iter, int sm_count, jac_route *out);
 
 /* Bytes of device workspace for jac_sweep_dev on this grid and plan (host
- * only).  It has room for every kernel the library may choose for a plan of
- * all zeros; jac_sweep_dev also accepts a smaller workspace (256 bytes and one
- * double per CTA of the plan) and then keeps to that plan.  No paper counterpart (the caller-owned scratch of the
- * stateless form). */
+ * only): for a plan of all zeros with room for every kernel the library may
+ * choose.  jac_sweep_dev also accepts a smaller workspace then (256 bytes and
+ * one double per CTA of the resolved plan) and keeps to the kernels it is
+ * enough for.  No paper counterpart (the caller-owned scratch of the stateless
+ * form). */
 jac_status jac_sweep_workspace_size(const jac_grid *g, const jac_plan *plan, size_t *bytes);
 
 /* n_iter sweeps of grid g on the given stream (a cudaStream_t, NULL for the

@@ -20,10 +20,10 @@ void set_thread_error(const std::string &m);
 jac_status validate_grid(const jac_grid *g);
 jac_plan resolve_plan(const jac_grid *g, const jac_plan *plan);
 jac_plan resolve_plan_sms(const jac_grid *g, const jac_plan *plan, int sms);
-// Bytes of workspace a sweep with this plan needs, and the bytes with which
-// every path open to the library's own plan may run (never less).
+// Bytes of workspace a sweep with this resolved plan needs, and those with
+// which every path open to `plan` may run (more where it is all zero).
 size_t sweep_workspace_bytes(const jac_grid *g, const jac_plan &p);
-size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p);
+size_t sweep_workspace_reported(const jac_grid *g, const jac_plan *plan);
 // Launch options of the single-grid sweep.  wait_ns and gbar_extra are set
 // only by a test of the failure path: a shorter limit for the waits on other
 // warps and CTAs, and an offset that makes the launch's grid barrier

@@ -429,10 +429,11 @@ static bool all_zero(const jac_plan *plan)
     return !plan || (plan->tile_i == 0 && plan->tile_j == 0 && plan->kdepth == 0 && plan->fuse == 0);
 }
 
-size_t sweep_workspace_reported(const jac_grid *g, const jac_plan &p)
+size_t sweep_workspace_reported(const jac_grid *g, const jac_plan *plan)
 {
     ResidentShape r;
-    size_t need = sweep_workspace_bytes(g, p);
+    size_t need = sweep_workspace_bytes(g, resolve_plan(g, plan));
+    if (!all_zero(plan)) return need;
     if (g->prec == JAC_F32) need = std::max(need, sweep2_workspace_bytes(g));
     if (resident_shape(g->I, g->J, g->K, g->prec, num_sms(), &r)) need = std::max(need, resident_workspace_bytes(r));
     return need;
@@ -632,7 +633,7 @@ jac_status jac_sweep_workspace_size(const jac_grid *g, const jac_plan *plan, siz
     if (!bytes) return jac::fail(JAC_EINVAL, "bytes is NULL");
     jac_status s = jac::validate_grid(g);
     if (s != JAC_OK) return s;
-    *bytes = jac::sweep_workspace_reported(g, jac::resolve_plan(g, plan));
+    *bytes = jac::sweep_workspace_reported(g, plan);
     return JAC_OK;
 }
 

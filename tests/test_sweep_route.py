@@ -91,6 +91,27 @@ def test_bench_names_the_kernel_that_runs(dims, n):
     assert r["algorithmic_bytes_per_launch"] == per_point * bench.n_interior(w)
 
 
+@pytest.mark.parametrize("dims,prec,kw", [((33, 33, 65), "f64", dict(kdepth=4)), ((77, 53, 101), "f32", dict(fuse=1)),
+                                          ((65, 65, 129), "bf16", dict(tile_j=16, tile_i=128, kdepth=8)),
+                                          ((129, 129, 257), "f32", dict(kdepth=64))])
+def test_workspace_of_an_explicit_plan_is_that_plan_s(dims, prec, kw):
+    """256 bytes and a double per CTA of the plan, rounded up to 256 bytes; the
+    flags of the resident kernel and a pass's partials only where the library
+    may choose them."""
+    import paper_2002_12115_gb300 as pkg
+    g = pkg.jac_grid()
+    g.I, g.J, g.K, g.prec, g.omega = *dims, pkg.PRECS[prec], 0.8
+    for b in range(2):
+        g.p[b] = 0x1000 * (b + 1)
+    for q in range(1, len(g.coef)):
+        g.coef[q] = 0x10000 * q
+    p = pkg.resolve_plan(*dims, prec, **kw)
+    items = (((dims[0] - 2) // p["tile_i"] + 1) * -(-(dims[1] - 2) // p["tile_j"]) * -(-(dims[2] - 2) // p["kdepth"]))
+    size, default = pkg.workspace_size(g, **kw), pkg.workspace_size(g)
+    assert size == 256 + -(-8 * min(items, 148) // 256) * 256        # 148 or 152 SMs: the same
+    assert default >= size
+
+
 @pytest.mark.parametrize("kw", [dict(tile_j=5), dict(kdepth=-2), dict(fuse=3)])
 def test_bad_plans_and_counts_are_rejected(kw):
     with pytest.raises(JacError, match="JAC_EINVAL"):
