@@ -180,15 +180,20 @@ jac_status ensure_workspace(jac_ctx *c)
     if (c->borrowed)
         return ctx_fail(c, JAC_EINVAL, "the sweep needs " + std::to_string(need) +
                                            " bytes of scratch, more than a borrowed workspace holds");
-    cudaError_t e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return ctx_cuda(c, e, "cudaStreamSynchronize");
-    if (c->ws) cudaFree(c->ws);
-    c->ws = nullptr;
-    c->ws_bytes = 0;
-    e = cudaMalloc(&c->ws, need);
+    // the header moves along: it holds the last sweep's residual and the error word
+    void *ws = nullptr;
+    cudaError_t e = cudaMalloc(&ws, need);
     if (e != cudaSuccess) return ctx_fail(c, JAC_ENOMEM, "workspace allocation failed");
-    e = cudaMemsetAsync(c->ws, 0, need, c->stream);
-    if (e != cudaSuccess) return ctx_cuda(c, e, "cudaMemsetAsync");
+    e = cudaMemsetAsync(ws, 0, need, c->stream);
+    if (e == cudaSuccess && c->ws)
+        e = cudaMemcpyAsync(ws, c->ws, jac::kWsHeaderBytes, cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) {
+        cudaFree(ws);
+        return ctx_cuda(c, e, "workspace copy");
+    }
+    if (c->ws) cudaFree(c->ws);
+    c->ws = ws;
     c->ws_bytes = need;
     return JAC_OK;
 }

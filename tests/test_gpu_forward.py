@@ -186,6 +186,24 @@ def test_api_errors():
         assert jac.count() == 2 and jac.residual() > 0
 
 
+def test_a_plan_with_a_larger_workspace_keeps_the_residual():
+    """An owned context allocates a larger workspace for a plan with more CTAs
+    (120 -> 152 here); the residual of the sweeps before is still there."""
+    from paper_2002_12115_gb300 import Jacobi
+    I, J, K = 129, 962, 30
+    f = ji.himeno_fields(I, J, K, seed=12)
+    with Jacobi(I, J, K, "bf16", owned=True) as jac:
+        jac.upload(f)
+        jac.sweep(2)
+        g = jac.residual()
+        assert g > 0
+        jac.set_plan(0, 8, 0)
+        assert jac.residual() == g
+        jac.sweep(2)
+        p = jac.download()
+    assert np.array_equal(p, gpu_run(f, 4, "bf16")[0])
+
+
 def test_unhoisted_matches_hoisted():
     """Per-sweep copy-in / copy-out gives the same state when the state is
     representable (FP64 storage)."""
