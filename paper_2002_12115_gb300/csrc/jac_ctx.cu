@@ -35,6 +35,7 @@ struct jac_ctx {
     double *stage_all = nullptr;      // JAC_NFIELDS*I*J*K doubles, jac_upload_async only (first use)
     void *ws = nullptr;               // sweep workspace
     size_t ws_bytes = 0;
+    bool ws_sized = false;            // ws is large enough for `plan`
     jac_plan plan{0, 0, 0, 0};
     long long count = 0;
     bool uploaded = false;
@@ -149,6 +150,7 @@ jac_status check_spec(jac_ctx *c, const jac_ws_spec *spec)
 // sweep scratch (the kernels need a zero header).
 jac_status ws_carve(jac_ctx *c, void *ws, size_t ws_bytes, const jac_ws_spec *spec)
 {
+    c->ws_sized = false;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255))
         return ctx_fail(c, JAC_EINVAL, "workspace must be non-NULL and 256-byte aligned");
     const WsLayout L = ws_layout(c->I, c->J, c->K, c->prec, spec);
@@ -170,13 +172,19 @@ jac_status ws_carve(jac_ctx *c, void *ws, size_t ws_bytes, const jac_ws_spec *sp
     return JAC_OK;
 }
 
+// A workspace large enough for the plan.  Its size is worked out when the
+// plan or the workspace changes, not in every call (1 us of host time).
 jac_status ensure_workspace(jac_ctx *c)
 {
+    if (c->ws_sized) return JAC_OK;
     jac_grid g = make_grid(c);
     size_t need = 0;
     jac_status s = jac_sweep_workspace_size(&g, &c->plan, &need);
     if (s != JAC_OK) return ctx_from_thread(c, s);
-    if (need <= c->ws_bytes) return JAC_OK;
+    if (need <= c->ws_bytes) {
+        c->ws_sized = true;
+        return JAC_OK;
+    }
     if (c->borrowed)
         return ctx_fail(c, JAC_EINVAL, "the sweep needs " + std::to_string(need) +
                                            " bytes of scratch, more than a borrowed workspace holds");
@@ -195,6 +203,7 @@ jac_status ensure_workspace(jac_ctx *c)
     if (c->ws) cudaFree(c->ws);
     c->ws = ws;
     c->ws_bytes = need;
+    c->ws_sized = true;
     return JAC_OK;
 }
 
@@ -500,6 +509,7 @@ jac_status jac_set_plan(jac_ctx *c, const jac_plan *plan)
         if (s != JAC_OK) return ctx_from_thread(c, s);
     }
     c->plan = p;
+    c->ws_sized = false;
     return ensure_workspace(c);
 }
 
