@@ -16,8 +16,8 @@ and FP64 paths of the same grid, the reverse pass of the last 20 of the 100
 sweeps with a checkpoint every 5 (the rest of that workload), the 129 x 129 x
 257 grid over 1000 sweeps in all three precisions, the per-sweep host-device
 transfer variant of that grid, and the batched workload (512 grids of 17..129
-points per side, 100 sweeps in one graph-replayed launch, against per-grid
-launch loops).
+points per side, 100 sweeps in one graph replay, against per-grid launch
+loops).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME]
     python bench.py --impl reference ...    # the FP64 CPU oracle as the reference arm

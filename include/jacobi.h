@@ -505,8 +505,8 @@ jac_status jac_sweep_adjoint(jac_ctx *ctx, const double *lambda_T, double *g_wrk
 
 /* ---------------------------------------------------------------------
  * Batched grids: many independent grids of uneven sizes swept together in
- * one persistent launch (a CUDA graph replayed on every call), each grid in
- * its own device storage.  No paper counterpart: the paper offloads one
+ * one to three persistent launches (a CUDA graph replayed on every call), each
+ * grid in its own device storage.  No paper counterpart: the paper offloads one
  * application at a time; this serves many small Himeno-style problems.
  * --------------------------------------------------------------------- */
 typedef struct jac_batch jac_batch;
@@ -541,8 +541,8 @@ jac_status jac_batch_grid_plan(const jac_batch *b, int g, jac_plan *out);
  * n_iter sweeps of every grid in one persistent launch (captured in a CUDA
  * graph on first use for this n_iter and buffer parity, then replayed).  A
  * FP32 batch without a plan whose state leaves L2 runs all but the last one to
- * four sweeps in two launches instead: its wide grids in two-sweep passes, the
- * others singly; the state is bitwise the same.
+ * four sweeps in up to two launches of their own: its wide grids in two-sweep
+ * passes, the others singly; the state is bitwise the same.
  * If res_host is not NULL it receives the n residuals of the last sweep.
  * Synchronises.  JAC_ETIMEOUT if a bounded device wait gave up. */
 jac_status jac_batch_sweep(jac_batch *b, int n_iter, double *res_host);

@@ -534,8 +534,8 @@ def adjoint_step_dev(grid: jac_grid, p_t: int, lam_in: int, lam_out: int, g_wrk1
 
 
 class JacobiBatch:
-    """Many independent grids of uneven sizes, swept together in one
-    persistent launch replayed from a CUDA graph (a jac_batch)."""
+    """Many independent grids of uneven sizes, swept together in one to three
+    persistent launches replayed from a CUDA graph (a jac_batch)."""
 
     def __init__(self, dims, prec: str = "f32", omega: float = 0.8, stream=None):
         import torch

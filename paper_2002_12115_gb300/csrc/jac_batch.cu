@@ -441,7 +441,7 @@ jac_status jac_batch_sweep(jac_batch *b, int n_iter, double *res_host)
     const std::pair<int, int> key(n_iter, b->par);
     auto it = b->graphs.find(key);
     if (it == b->graphs.end()) {
-        // capture the single persistent launch once; later calls replay it
+        // capture the launches (one, or up to three with passes) once; later calls replay them
         cudaStream_t cap = nullptr;
         cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
         if (e != cudaSuccess) return bcuda(b, e, "capture stream");

@@ -37,6 +37,9 @@
 //   17x17x17 FP64 6.3 -> 3.7      33x33x65 FP64 6.4 -> 5.1   49x49x97 FP64 15.9 -> 10.9
 //   33x33x65 FP32 4.5 -> 3.5      77x53x101 FP32 7.0 -> 4.8  65x65x129 FP32 6.5 -> 4.7
 //   65x65x129 BF16 6.1 -> 4.2
+// (80 registers at 768 threads: ptxas spills 20 bytes in FP32, 24 with BF16
+// coefficients, 36 in FP64.)  Wide, flat grids are faster streaming: the rule is
+// resident_pays in jac_sweep.cu.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -465,7 +468,9 @@ jac_status launch_resident(const ResArgs &a, unsigned nblocks, size_t smem, cuda
 // next to other boxes at tu per point (128 points at a time: one per lane of
 // a warp on each of the SM's four FP64 pipes), then the exchange, which the
 // inner rows overlap, and the halo rows it collects.  tu and the exchange are
-// measured (33x33x65 FP64, 77x53x101 FP32).  Against the split with the fewest
+// measured on 33x33x65 FP64 and 77x53x101 FP32; BF16 takes FP32's.  The model
+// orders the splits of one grid and leaves out how wide the halo rows are; what
+// a sweep takes is estimated by resident_us in jac_sweep.cu.  Against the split with the fewest
 // points in its largest box, which left 77x53x101 FP32 no inner rows (17 x 2
 // instead of 9 x 4): 5.7 -> 4.8 us a sweep.
 bool resident_shape(int I, int J, int K, jac_prec prec, int sms, ResidentShape *out)

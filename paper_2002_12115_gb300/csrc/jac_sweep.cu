@@ -502,7 +502,10 @@ static bool resident_pays(const jac_grid *g, const jac_plan &p, int n_iter, int 
 // Whether a call of n_iter sweeps with the library's own plan (all zero) takes
 // two-sweep passes: the faster of the two by the measured rates of both
 // kernels (21 FP32 grids, 65x200x200 to 513x513x1025).  A step of a pass's
-// busiest CTA takes 1.30-1.43 us on 16 of them and up to 1.7 on the others.
+// busiest CTA takes 1.30-1.43 us on 16 of them and up to 1.7 on the others;
+// 1.45 leans towards single sweeps.  On 70 more grids, where the estimate of a
+// pass is 0.6 to 1.1 of that of two single sweeps, no call of 4, 6 or 20 sweeps
+// took more than 1.02 of the time of single sweeps.
 // A single sweep takes 2 us and 7.1 ns per 1000 points where both state buffers
 // stay in half the L2 and 8.5 ns per 1000 points otherwise.  What decides is
 // how well 128 columns by 8 rows tile the grid: 129x129x257 (full tiles) 31.0

@@ -46,8 +46,9 @@
 //     from global memory one plane ahead;
 //   * both sweeps take the update in two parts (ss_axes, ss_rest), and sweep 1
 //     forms the b brackets before it loads a coefficient, so that 96 registers
-//     hold one part's coefficients and the state values still needed.  Spilled
-//     registers went through an L1 of a few KB, behind the copies' traffic;
+//     hold one part's coefficients and the state values still needed but for 12
+//     bytes that ptxas spills (4 with MID, 64 without that order).  Spilled
+//     registers go through an L1 of a few KB, behind the copies' traffic;
 //   * two points share an instruction (f32x2) where both operands lie in
 //     aligned register pairs: a3 S - 1 and the axis terms;
 //   * every wait is bounded; on expiry the kernel sets the workspace error
@@ -63,8 +64,8 @@
 //
 // What bounds it: latency and issue of 18 compute warps where the state stays in
 // L2 (a step of a CTA, one plane of a tile, both sweeps, takes 1.34 us), and
-// DRAM elsewhere: 513x513x1025 reads and writes 1.06 times the bytes a pass
-// needs at 6.1 TB/s.  Kept against, on one GB300 (Gpt/s, FP32):
+// DRAM elsewhere: 513x513x1025 reads and writes 1.05 times the bytes a pass
+// needs at 6.2 TB/s.  Kept against, on one GB300 (Gpt/s, FP32):
 //                                             129x129x257   257x257x513   513x513x1025
 //   both sweeps in one warp, coefficients of
 //     sweep 2 read again from L2 (41% of all
@@ -72,7 +73,7 @@
 //   ... kept in tensor memory                                     150            153
 //   separate warps for the two sweeps                             164            143
 //   ... and items by ticket                        161            171            150
-//   barriers tested together, no spills, f32x2     189            172            158
+//   barriers tested together, 12 B spilled, f32x2  189            172            158
 //   i-neighbours first, all CTAs in step
 //     (this kernel)                                192            216            208
 // The order alone (by ticket) ran at 184 and 157, the clock alone at 174 and
@@ -684,7 +685,7 @@ k_sweep2(const __grid_constant__ Sweep2Desc d, const Sweep2Args a)
                     bjk[e] = ((vp2[e] - vm2[e]) - vp0[e]) + vm0[e];
                     bik[e] = ((ep1[e + 2] - em1[e + 2]) - ep1[e]) + em1[e];
                 }
-                // formed before the coefficients are loaded: nothing is spilled
+                // formed before the coefficients are loaded: 12 bytes are spilled instead of 64
                 tmem_loaded(bij); tmem_loaded(bjk); tmem_loaded(bik);
                 float dd[VI], ec[VI];
                 {

@@ -80,7 +80,7 @@ def test_default_plan_takes_passes_where_the_state_leaves_l2():
 
 
 @pytest.mark.parametrize("dims,n", [((129, 129, 140), 16), ((257, 65, 70), 12), ((385, 40, 33), 21), ((300, 205, 61), 14)])
-def test_passes_by_ticket_are_repeatable_and_equal_single_sweeps(dims, n):
+def test_passes_are_repeatable_and_equal_single_sweeps(dims, n):
     """Several passes with more items than CTAs (the last rounds of a pass and
     of planes not full), or with a shared pass barrier over few items: which
     CTA is ahead differs from run to run, the state and the residual do not.
