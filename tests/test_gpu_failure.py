@@ -1,10 +1,11 @@
 """The failure path of the bounded device waits, made to run out on purpose
 without faulting or hanging anything.
 
-jac_inject_stall gives the next sweep launch a grid-barrier target between
-sweeps that no CTA ever reaches, and a wait limit of a few milliseconds.
-The state producer's barrier wait then gives up, every CTA drains its own
-copies and exits, and the launch ends with the workspace error word set:
+jac_inject_stall gives the next sweep call's launches a grid-barrier target
+that no CTA ever reaches, and a wait limit of a few milliseconds.  The waits
+for it -- of the streaming kernel's and the two-sweep kernel's producers, of
+the resident kernel's communication warps -- then give up, every CTA drains its
+own copies and exits, and the launch ends with the workspace error word set:
 the residual written is NaN, jac_sync and jac_residual report JAC_ETIMEOUT
 and clear the word, and the same context then sweeps normally again (the
 result checked against the oracle).  This is the library's counterpart of
@@ -114,6 +115,20 @@ def stall_and_recover(pkg, prec, dims, n, plan=None):
             jac.sweep(m)
             assert np.array_equal(jac.download(), p) and jac.residual() == g
     return f, stalled, other
+
+
+@pytest.mark.parametrize("prec,dims", [("f32", (70, 21, 19)), ("bf16", (131, 9, 12)), ("f64", (37, 33, 29))])
+def test_streaming_waits_run_out(pkg, prec, dims):
+    """The streaming kernel's wait between sweeps: the first sweep is stored
+    whole and no CTA starts the second."""
+    n, plan = 4, (0, 0, 0, 1)
+    assert pkg.sweep_route(*dims, prec, n, fuse=1)["single_sweeps"] == n
+    f, stalled, other = stall_and_recover(pkg, prec, dims, n, plan)
+    with pkg.Jacobi(*dims, prec) as jac:
+        jac.upload(f)
+        assert np.array_equal(stalled, jac.download())
+        jac.sweep(1)
+        assert np.array_equal(other, jac.download())
 
 
 @pytest.mark.parametrize("prec,dims", [("f32", (77, 53, 101)), ("bf16", (61, 40, 50)), ("f64", (33, 33, 65))])
